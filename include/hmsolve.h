@@ -272,8 +272,11 @@ int hm_far_apply_noalloc(hm_handle h, const void *dx, void *dy, int32_t nrhs);
  * consecutive block rows, a row reading the results of earlier rows of its cluster from their
  * shared memory (complex-FP32 sweeps; the FP64 sweeps take kind 1 for them).  Kinds 1-3, 5
  * and 6 give bitwise the same result, and kind 4 gives bitwise the same result for every
- * number of groups.  (0, 0) -- the default -- lets the library time kind 1 with 1, 2 and 4
- * groups and each tile on its first calls of each width and keep the fastest.
+ * number of groups.  (0, 0) is the default: two-level sweeps, in which 16 consecutive block rows
+ * form a super-row whose unit triangle is inverted once per setup, so that its rows run side by
+ * side (a fixed summation order of its own, bitwise the same for every batch width).  Where
+ * hbm_budget leaves no room for their data, the library instead times kind 1 with 1, 2 and 4
+ * groups and each tile on its first calls of each width and keeps the fastest.
  * Kinds 2 and 3 apply to groups of at most 16 columns (kind 1 otherwise).  With compressed
  * fill-in blocks (fill_tol > 0) kinds 2-4 take kind 1.  `tile` (kind 1) selects the
  * register tile of each thread -- rows x columns x tiles per thread -- for groups of 5-16

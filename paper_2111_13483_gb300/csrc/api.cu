@@ -15,8 +15,13 @@ cudaError_t Arena::alloc(void **p, size_t bytes)
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     bytes = (bytes + 255) & ~size_t(255);
-    if (budget && used + bytes > budget) return cudaErrorMemoryAllocation;
-    cudaError_t e = cudaMalloc(p, bytes);
+    const bool over = budget && used + bytes > budget;
+    cudaError_t e = over ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        *p = nullptr;
+        return reclaim && reclaim(owner) ? alloc(p, bytes) : e;
+    }
     if (e == cudaSuccess) {
         used += bytes;
         ptrs.push_back(*p);
@@ -176,6 +181,14 @@ int hmat_create(const hm_desc *d, const hm_opts *opts, hm_handle *out)
     h->dev = h->opts.device;
     cudaSetDevice(h->dev);
     h->arena.budget = h->opts.hbm_budget;
+    h->arena.owner = h;
+    h->arena.reclaim = [](void *p) {   // the two-level sweeps' memory: the other sweeps do without
+        hm_ctx *c = (hm_ctx *)p;
+        if (!c->s2.on) return false;
+        cudaStreamSynchronize(c->stream);
+        sweep2_release(c);
+        return true;
+    };
     if (h->opts.stream)
         h->stream = (cudaStream_t)h->opts.stream;
     else {
@@ -302,6 +315,7 @@ int precond_setup(hm_handle h)
     e = setup_run(h, &bad);
     if (!e && bad < 0) e = compress_run(h);
     if (!e && bad < 0) e = pack_run(h);
+    if (!e && bad < 0) e = sweep2_setup(h);
     cudaEventRecord(e1, h->stream);
     cudaEventSynchronize(e1);
     float ms = 0;

@@ -17,6 +17,9 @@ struct Arena {
     size_t used = 0, budget = 0;
     std::vector<void *> ptrs;
     std::vector<size_t> sizes;
+    // frees memory the handle can do without when an allocation fails; true if it freed any
+    bool (*reclaim)(void *) = nullptr;
+    void *owner = nullptr;
     cudaError_t alloc(void **p, size_t bytes);
     void release(void *p, size_t bytes);
     void release_all();
@@ -133,6 +136,24 @@ struct FarPlan {
     std::vector<int> nptr, nent;
 };
 
+// Two-level sweeps (sweep2.cu): block rows per super-row, and one block row as a direction's sweep
+// walks it: its rows in solve order, the plan entries of its dependencies outside the super-row
+// (from p0, ext of them), its rows of N_S, and the rows of the super-row they contract over.
+constexpr int S2_K = 16;
+struct S2Row {
+    int ro, no, p0, ext;
+    int64_t noff;
+    int zrow, zlen;
+};
+struct S2State {   // index 0 forward, 1 backward
+    bool on = false;
+    S2Row *rows[2] = {nullptr, nullptr};
+    int64_t *off[2] = {nullptr, nullptr};
+    int4 *deps[2] = {nullptr, nullptr};
+    void *N[2] = {nullptr, nullptr};
+    void *buf = nullptr;   // ticket and hand-over buffers
+};
+
 // Online choice of the schedule of a sweep launch -- the number of independent column
 // groups and the blocks per CTA (1, or a super-row of SWEEP_SR) -- per precision, direction
 // and width class: candidates are timed on real calls (every candidate computes the same
@@ -225,6 +246,7 @@ struct hm_ctx {
     float2 *d_t32 = nullptr, *d_s32 = nullptr, *d_work32 = nullptr;
     uint4 *d_ytag = nullptr;   // tagged sweep results (complex FP32 sweeps), n x 64
     int t32_cols = 0;
+    hm::S2State s2;            // the default sweeps
     bool batch_open = false;   // an hm_batch holds this handle
     hm::SweepTune sweep_tune[2][2][5];   // [FP32][forward][width class]
     int sweep_fixed = 0;                 // a schedule code set by hm_set_sweep_schedule, 0 = tuned
@@ -303,6 +325,9 @@ template <class T>
 cudaError_t far_product(hm_ctx *h, const T *U, const T *V, T *t, T *s, const T *ucl, T *y, int nrhs);
 cudaError_t ensure_solve_workspace(hm_ctx *h, int nrhs);
 void sweep_tune_release(hm_ctx *h);
+cudaError_t sweep2_setup(hm_ctx *h);
+void sweep2_release(hm_ctx *h);
+template <class T> cudaError_t sweep2_run(hm_ctx *h, bool fwd, const T *W, const T *x, T *y, int nrhs);
 int gmres_solve(hm_ctx *h, const double2 *dV, int nrhs, int64_t ldv, double tol, int restart, int maxit,
                 double2 *dI, int64_t ldi, int *iters, double *relres);
 }  // namespace hm

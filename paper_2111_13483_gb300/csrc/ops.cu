@@ -4,6 +4,8 @@
 //
 // L^{-1} / L^{-T} are the products of the left / right scaling coefficients (Eqs. 20, 23,
 // 24) applied as block-triangular sweeps over the coefficient panels W_k (L_jk = W_kj^T).
+// By default they are the two-level sweeps of sweep2.cu; the kinds below are selectable, and the
+// default where the handle's budget has no room for the two-level data.
 // Each sweep is one sync-free launch: a CTA takes the next block row from a ticket counter
 // (so every block it waits on belongs to a CTA that is already running), stages the
 // coefficient blocks of its dependencies in fixed chunks, waits on their ready flags (a
@@ -24,26 +26,11 @@
 #include "hm_internal.h"
 #include "tc.cuh"
 #include "tile.cuh"
+#include "wait.cuh"
 
 namespace hm {
 
 namespace {
-
-// The handle's error word block: err[ERR_CODE] is set by a failing wait, err[ERR_HOLD] names a
-// block row the sweeps leave out (a test hook: -1 = none; every wait on that row then runs
-// out), err[ERR_BOUND..+1] holds the bound on any single wait in ns (2 s unless a test sets it).
-__device__ __forceinline__ unsigned long long wait_bound(const int *err)
-{
-    return __ldcg((const unsigned long long *)(err + ERR_BOUND));
-}
-__device__ __forceinline__ bool held_back(const int *err, int blk) { return __ldcg(err + ERR_HOLD) == blk; }
-
-__device__ __forceinline__ unsigned long long gtimer()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
 
 // One thread waits until flags[k] == epoch; false (and ERR_TIMEOUT recorded) when the
 // bound expires or another CTA already failed.
@@ -1510,9 +1497,10 @@ template <class T>
 static cudaError_t sweep(hm_ctx *h, const OpData<T> &d, bool forward, const T *x, T *y, int nrhs)
 {
     cudaError_t e;
+    h->prof.cols[forward ? K_SWEEP_FWD : K_SWEEP_BWD] += nrhs;
+    if (h->s2.on && !h->sweep_fixed) return sweep2_run<T>(h, forward, d.W, x, y, nrhs);
     if ((e = cudaMemsetAsync(h->d_ticket, 0, sizeof(int), h->stream))) return e;
     const int ep = ++h->epoch;
-    h->prof.cols[forward ? K_SWEEP_FWD : K_SWEEP_BWD] += nrhs;
     SweepTune *tu;
     int slot = 0;
     const int code = sweep_groups(h, sizeof(T) == 8, forward, nrhs, &tu, &slot);
@@ -1641,7 +1629,7 @@ cudaError_t ensure_solve_workspace(hm_ctx *h, int nrhs)
         if ((e = h->arena.alloc((void **)&h->d_work32, sizeof(float2) * (size_t)n * 5 * nrhs))) return e;
         h->t32_cols = nrhs;
     }
-    if (h->opts.precision == 1 && !h->d_ytag) {   // tagged sweep results, 64 columns, epochs start at 1
+    if (h->opts.precision == 1 && !h->d_ytag && (!h->s2.on || h->sweep_fixed)) {   // tagged sweep results, 64 columns, epochs start at 1
         if ((e = h->arena.alloc((void **)&h->d_ytag, sizeof(uint4) * (size_t)n * 64))) return e;
         if ((e = cudaMemsetAsync(h->d_ytag, 0, sizeof(uint4) * (size_t)n * 64, h->stream))) return e;
     }
