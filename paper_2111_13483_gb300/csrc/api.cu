@@ -218,8 +218,9 @@ int hmat_create(const hm_desc *d, const hm_opts *opts, hm_handle *out)
         (e = upload(h, &h->d_seg_ptr, F.seg_ptr)) || (e = upload(h, &h->d_segs, F.segs)) ||
         (e = upload(h, &h->d_seg_kcum, F.seg_kcum)) || (e = upload(h, &h->d_part_ptr, F.part_ptr)) ||
         (e = upload(h, &h->d_flptr, F.lptr)) ||
-        (e = upload(h, &h->d_flent, F.lent)) || (e = upload(h, &h->d_nptr, F.nptr)) ||
-        (e = upload(h, &h->d_nent, F.nent)) || (e = upload(h, &h->d_leaf_ptr, h->leaf_ptr)) ||
+        (e = upload(h, &h->d_flent, F.lent)) || (e = upload(h, &h->d_zpart, F.zpart)) ||
+        (e = upload(h, &h->d_zkcum, F.zkcum)) || (e = upload(h, &h->d_zsegs, F.zsegs)) ||
+        (e = upload(h, &h->d_leaf_ptr, h->leaf_ptr)) ||
         (e = upload(h, &h->d_new2cl, P.new2cl)) || (e = upload(h, &h->d_cl2new, P.cl2new)) ||
         (e = upload(h, &h->d_new2orig, P.new2orig)) || (e = upload(h, &h->d_perm, h->perm)) ||
         (e = upload(h, &h->d_pos, P.pos)) || (e = upload(h, &h->d_size, P.size)) ||

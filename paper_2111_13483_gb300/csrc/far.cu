@@ -17,6 +17,8 @@
 // (so that the uneven leaves spread over all SMs); k_far_sum adds the parts in order.  Every output sums its terms in
 // one fixed order, so results are deterministic and do not depend on how many right-hand
 // sides share the launch.
+#include <algorithm>
+
 #include "cplx.cuh"
 #include "hm_internal.h"
 #include "tc.cuh"
@@ -45,6 +47,36 @@ template <class T> __device__ __forceinline__ void far_cp(T *dst, const T *src)
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
 }
 
+// The task's factor columns, in item order (at most 64 columns, so at most 64 items of rank >= 1): column R of
+// item s_item[R], its l-th, at s_src[R]; returns their number.  One thread per column: a walk by one thread
+// waited on memory twice per item, about 5 us per task.
+template <class T>
+__device__ __forceinline__ int far_items(int i0, int i1, const int64_t *item_off, const int *item_ld, const int *item_rank,
+                                         const int *item_isv, const T *U, const T *V, int *s_item, int *s_l,
+                                         const T **s_src)
+{
+    __shared__ int s_cum[65];
+    const int ni = min(i1 - i0, 64), tid = threadIdx.x;
+    if (tid < ni) s_cum[tid + 1] = item_rank[i0 + tid];
+    __syncthreads();
+    if (tid == 0) {
+        s_cum[0] = 0;
+        for (int q = 0; q < ni; ++q) s_cum[q + 1] += s_cum[q];
+    }
+    __syncthreads();
+    const int R = min(s_cum[ni], 64);
+    if (tid < R) {
+        int q = 0;
+        while (s_cum[q + 1] <= tid) ++q;
+        const int it = i0 + q, l = tid - s_cum[q];
+        s_item[tid] = it;
+        s_l[tid] = l;
+        s_src[tid] = (item_isv[it] ? V : U) + item_off[it] + (int64_t)l * item_ld[it];
+    }
+    __syncthreads();
+    return R;
+}
+
 template <class T, int TR, int TC, int NT>
 __global__ void __launch_bounds__(256) k_far_t(const int *task_lo, const int *task_hi, const int *task_ptr,
                                                const int64_t *item_off, const int *item_ld, const int *item_rank,
@@ -54,21 +86,9 @@ __global__ void __launch_bounds__(256) k_far_t(const int *task_lo, const int *ta
     extern __shared__ unsigned char smraw[];
     __shared__ int s_item[64], s_l[64];
     __shared__ const T *s_src[64];
-    __shared__ int s_R;
     const int task = blockIdx.x;
     const int lo = task_lo[task], hi = task_hi[task], i0 = task_ptr[task], i1 = task_ptr[task + 1];
-    if (threadIdx.x == 0) {
-        int R = 0;
-        for (int it = i0; it < i1; ++it)
-            for (int l = 0; l < item_rank[it] && R < 64; ++l, ++R) {
-                s_item[R] = it;
-                s_l[R] = l;
-                s_src[R] = (item_isv[it] ? V : U) + item_off[it] + (int64_t)l * item_ld[it];
-            }
-        s_R = R;
-    }
-    __syncthreads();
-    const int R = s_R;
+    const int R = far_items(i0, i1, item_off, item_ld, item_rank, item_isv, U, V, s_item, s_l, s_src);
     const int nrt = (R + TR - 1) / TR, ntiles = nrt * ((nrhs + TC - 1) / TC);
     const int ldw = stage_ldw(R, TR), ldr = stage_ldr(nrhs, TC);
     T *const bufs[2] = {(T *)smraw, (T *)smraw + budget / 2};
@@ -114,6 +134,110 @@ __global__ void __launch_bounds__(256) k_far_t(const int *task_lo, const int *ta
                     dst[(int64_t)(item_row[it] + s_l[row0 + a]) * nrhs + r0 + c] = acc.v[tt][a][c];
                 }
     }
+}
+
+// ---- complex FP64 ---------------------------------------------------------------------------
+// GB300 issues a DFMA for two lanes per SM and clock: one warp instruction holds its scheduler for 64
+// cycles whatever its lanes do, and shared-memory loads are free beside it.  So the outputs are laid flat
+// over the lanes (28 rows x 16 columns are 14 full warps; 2 x 2 register tiles left an eighth of the
+// lanes idle), and the contraction is split F64_NK ways (entry kk of the whole contraction to
+// way kk mod F64_NK, partial sums added in order), so that one column keeps all four schedulers busy
+// too.  The split does not depend on the columns: a column's bits are the same in any batch.
+// The near-field blocks of a leaf join its phase-2 segments where Z itself is applied.
+// Measured at 64 columns on the 30,720-unknown sphere: phase 1 23.5 -> 22.8 ms, phase 2 38.6 and the near field
+// 34.6 (a CTA of its own per leaf) -> 47.2 ms together; one column: 0.64 -> 0.46 and 1.37 + 0.80 -> 1.42 ms.
+// Phase 2 runs at the DFMA rate (0.63 T/s measured by a chain of FMAs).
+constexpr int F64_NK = 4, F64_NH = 2;   // ways the contraction and the outputs are split over the warps
+constexpr int F64_T = 32 * F64_NK * F64_NH;
+
+// acc[u] += sum over this warp's kk of Ws[kk * ldw + i] Ys[kk * ldr + c], output e = lane + 32 (F64_NH u + half) = c * no + i
+template <int NU>
+__device__ __forceinline__ void f64_mac(double2 (&acc)[NU], const double2 *Ws, int ldw, const double2 *Ys, int ldr, int k0,
+                                        int klen, int no, int len)
+{
+    const int w = (threadIdx.x >> 5) - k0 & F64_NK - 1;   // the chunk starts at entry k0
+    const int e0 = (threadIdx.x & 31) + 32 * (threadIdx.x >> 7), di = 32 * F64_NH % no, dc = 32 * F64_NH / no;
+    for (int kk = w; kk < klen; kk += F64_NK) {
+        const double2 *wp = Ws + kk * ldw, *yp = Ys + kk * ldr;
+        int i = e0 % no, c = e0 / no;
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            const int e = e0 + 32 * F64_NH * u;
+            if (e - (int)(threadIdx.x & 31) >= len) break;
+            if (e < len) acc[u] = cfma(wp[i], yp[c], acc[u]);
+            i += di;
+            c += dc;
+            if (i >= no) i -= no, ++c;
+        }
+    }
+}
+
+// the warps' partial sums through shared memory: put(e, sum) for every output e < len
+template <int NU, class Put> __device__ __forceinline__ void f64_reduce(const double2 (&acc)[NU], double2 *sm, int len, Put &&put)
+{
+    const int e0 = (threadIdx.x & 31) + 32 * (threadIdx.x >> 7), w = threadIdx.x >> 5 & F64_NK - 1;
+#pragma unroll
+    for (int u = 0; u < NU; ++u) {
+        const int e = e0 + 32 * F64_NH * u;
+        if (e < len) sm[w * len + e] = acc[u];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < len; e += F64_T) {
+        double2 v = sm[e];
+        for (int q = 1; q < F64_NK; ++q) {
+            v.x += sm[q * len + e].x;
+            v.y += sm[q * len + e].y;
+        }
+        put(e, v);
+    }
+}
+
+// phase 1, tasks as in k_far_t
+template <int NU>
+__global__ void __launch_bounds__(F64_T) k_far_t64(const int *task_lo, const int *task_hi, const int *task_ptr,
+                                                   const int64_t *item_off, const int *item_ld, const int *item_rank,
+                                                   const int *item_row, const int *item_isv, const double2 *U,
+                                                   const double2 *V, const double2 *u, int nrhs, double2 *t, double2 *s,
+                                                   int half)
+{
+    extern __shared__ unsigned char smraw[];
+    __shared__ int s_item[64], s_l[64];
+    __shared__ const double2 *s_src[64];
+    const int task = blockIdx.x;
+    const int lo = task_lo[task], hi = task_hi[task], i0 = task_ptr[task], i1 = task_ptr[task + 1];
+    const int R = far_items(i0, i1, item_off, item_ld, item_rank, item_isv, U, V, s_item, s_l, s_src), len = R * nrhs, ldw = R | 1;
+    double2 *const bufs[2] = {(double2 *)smraw, (double2 *)smraw + half};
+    double2 acc[NU];
+#pragma unroll
+    for (int q = 0; q < NU; ++q) acc[q] = make_double2(0.0, 0.0);
+    auto stage = [&](int c0, int which) {   // as in k_far_t: Ws[qq * ldw + rr], then Ys[qq * nrhs + r]
+        const int ch = min(FAR_T1, hi - c0);
+        double2 *Ws = bufs[which], *Ys = Ws + ch * ldw;
+        for (int rr = threadIdx.x / FAR_T1; rr < R; rr += F64_T / FAR_T1) {
+            const int qq = threadIdx.x % FAR_T1;
+            if (qq < ch) far_cp(Ws + qq * ldw + rr, s_src[rr] + (c0 - lo + qq));
+        }
+        const double2 *uc = u + (int64_t)c0 * nrhs;
+        for (int e = threadIdx.x; e < ch * nrhs; e += F64_T) far_cp(Ys + e, uc + e);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    if (lo < hi) stage(lo, 0);
+    for (int c0 = lo, it = 0; c0 < hi; c0 += FAR_T1, ++it) {
+        const int ch = min(FAR_T1, hi - c0);
+        if (c0 + FAR_T1 < hi) {
+            stage(c0 + FAR_T1, (it + 1) & 1);
+            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        } else
+            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        __syncthreads();
+        const double2 *Ws = bufs[it & 1];
+        f64_mac<NU>(acc, Ws, ldw, Ws + ch * ldw, nrhs, c0 - lo, ch, R, len);
+        __syncthreads();
+    }
+    f64_reduce<NU>(acc, (double2 *)smraw, len, [&](int e, double2 v) {
+        const int rr = e % R, r = e / R, it = s_item[rr];
+        (item_isv[it] ? t : s)[(int64_t)(item_row[it] + s_l[rr]) * nrhs + r] = v;
+    });
 }
 
 // Phase 2: one CTA per leaf over the leaf's segments (FarSegD, list order, len <= 32).
@@ -224,6 +348,98 @@ __global__ void __launch_bounds__(256) k_far_y(int nl, const int *leaf_ptr, cons
     tile_store(acc, part + (size_t)pp * n * nrhs + cl2new[a], 1, n, ni, nrhs, nrt, ntiles);
 }
 
+// complex FP64, phase 2 (see f64_mac): the segments of the far list and, with nearp, those of the leaf's
+// near-field blocks (zpart / zkcum / zsegs), which gives Z u in one pass
+template <int NU>
+__global__ void __launch_bounds__(F64_T) k_far_y64(int nl, const int *leaf_ptr, const int *part_ptr, const int *kcum,
+                                                   const FarSegD *segs, const int *zpart, const int *zkcum,
+                                                   const FarSegD *zsegs, const double2 *U, const double2 *V,
+                                                   const double2 *nearp, const double2 *t, const double2 *s,
+                                                   const double2 *u, const int *cl2new, int n, int nrhs, double2 *part,
+                                                   int half)
+{
+    extern __shared__ unsigned char smraw[];
+    const int l = blockIdx.x / FAR_PARTS, pp = blockIdx.x % FAR_PARTS;
+    if (l >= nl) return;
+    const int a = leaf_ptr[l], ni = leaf_ptr[l + 1] - a, len = ni * nrhs, ldw = ni | 1;
+    const int kmax = half / (ldw + nrhs);   // >= 32
+    double2 *const bufs[2] = {(double2 *)smraw, (double2 *)smraw + half};
+    double2 acc[NU];
+#pragma unroll
+    for (int q = 0; q < NU; ++q) acc[q] = make_double2(0.0, 0.0);
+    for (int tab = 0; tab < (nearp ? 2 : 1); ++tab) {
+        const int *pt = tab ? zpart : part_ptr, *kc = tab ? zkcum : kcum;
+        const FarSegD *sg = tab ? zsegs : segs;
+        const double2 *F0 = tab ? nearp : U, *F1 = tab ? nearp : V;
+        const int w1 = pt[blockIdx.x + 1];
+        auto chunk_count = [&](int p) {   // segments from p on whose stacked length fits kmax
+            const int q = p + threadIdx.x;
+            return __syncthreads_count(q < w1 && kc[q + 1] - kc[p] <= kmax);
+        };
+        auto stage = [&](int p, int cnt, double2 *buf) {   // as in k_far_y
+            const int k0 = kc[p], klen = kc[p + cnt] - k0;
+            double2 *Wst = buf, *Yst = buf + kmax * ldw;
+            int q = -1, qlo = 0, qhi = 0;
+            const double2 *F = nullptr;
+            int64_t fi = 0, fk = 0;
+            for (int e = threadIdx.x; e < klen * ni; e += F64_T) {
+                const int kk = e / ni, i = e - kk * ni;
+                while (kk >= qhi) {
+                    ++q;
+                    qlo = kc[p + q] - k0;
+                    qhi = kc[p + q + 1] - k0;
+                    const FarSegD g = sg[p + q];
+                    F = ((g.src & 1) ? F1 : F0) + g.foff;
+                    fi = g.fi;
+                    fk = g.fk;
+                }
+                cp_async_el(Wst + kk * ldw + i, F + (int64_t)i * fi + (int64_t)(kk - qlo) * fk);
+            }
+            q = -1;
+            qhi = 0;
+            const double2 *Yb = nullptr;
+            for (int e = threadIdx.x; e < klen * nrhs; e += F64_T) {
+                const int kk = e / nrhs, r = e - kk * nrhs;
+                while (kk >= qhi) {
+                    ++q;
+                    qlo = kc[p + q] - k0;
+                    qhi = kc[p + q + 1] - k0;
+                    const FarSegD g = sg[p + q];
+                    const int ys = g.src >> 1;
+                    Yb = (ys == 0 ? t : (ys == 1 ? s : u)) + g.yrow * nrhs;
+                }
+                cp_async_el(Yst + e, Yb + (int64_t)(kk - qlo) * nrhs + r);
+            }
+            cp_async_commit();
+            return klen;
+        };
+        const int p0 = pt[blockIdx.x];
+        int p = p0;
+        if (p >= w1) continue;
+        int cnt = chunk_count(p), klen = stage(p, cnt, bufs[0]);
+        for (int it = 0;; ++it) {
+            const int pn = p + cnt;
+            int cntn = 0, klenn = 0;
+            if (pn < w1) {
+                cntn = chunk_count(pn);
+                klenn = stage(pn, cntn, bufs[(it + 1) & 1]);
+                cp_async_wait<1>();
+            } else
+                cp_async_wait<0>();
+            __syncthreads();
+            const double2 *buf = bufs[it & 1];
+            f64_mac<NU>(acc, buf, ldw, buf + kmax * ldw, nrhs, kc[p] - kc[p0], klen, ni, len);
+            __syncthreads();
+            if (pn >= w1) break;
+            p = pn;
+            cnt = cntn;
+            klen = klenn;
+        }
+    }
+    double2 *out = part + (size_t)pp * n * nrhs + cl2new[a];
+    f64_reduce<NU>(acc, (double2 *)smraw, len, [&](int e, double2 v) { out[e % ni + (int64_t)(e / ni) * n] = v; });
+}
+
 // ---- complex FP32 on the tensor cores ------------------------------------------------------
 // The same two phases with the block products on the tensor-core micro-kernel of tc.cuh
 // (TF32 operands split into a rounded part and a remainder, FP32 accumulation in tensor
@@ -248,23 +464,11 @@ __global__ void __launch_bounds__(256, 2) k_far_t_tc(const int *task_lo, const i
     extern __shared__ unsigned char smraw[];
     __shared__ int s_item[64], s_l[64];
     __shared__ const float2 *s_src[64];
-    __shared__ int s_R;
     __shared__ uint64_t s_mbar[2];
     __shared__ uint32_t s_tmem;
     const int task = blockIdx.x;
     const int lo = task_lo[task], hi = task_hi[task], i0 = task_ptr[task], i1 = task_ptr[task + 1];
-    if (threadIdx.x == 0) {
-        int R = 0;
-        for (int it = i0; it < i1; ++it)
-            for (int l = 0; l < item_rank[it] && R < 64; ++l, ++R) {
-                s_item[R] = it;
-                s_l[R] = l;
-                s_src[R] = (item_isv[it] ? V : U) + item_off[it] + (int64_t)l * item_ld[it];
-            }
-        s_R = R;
-    }
-    __syncthreads();
-    const int R = s_R;
+    const int R = far_items(i0, i1, item_off, item_ld, item_rank, item_isv, U, V, s_item, s_l, s_src);
     if (R == 0) return;
     unsigned char *region = tc::align1024(smraw);
     float2 *rawA = (float2 *)(region + 2 * tc::STAGE2), *rawB = rawA + 2 * tc::KC2 * FTC_LD;
@@ -526,20 +730,59 @@ static cudaError_t far_tc_launch(hm_ctx *h, const float2 *U, const float2 *V, fl
     return cudaGetLastError();
 }
 
-template <class T>
-cudaError_t far_product(hm_ctx *h, const T *U, const T *V, T *t, T *s, const T *ucl, T *y, int nrhs)
+// complex FP64: y = Z_F u, or Z u with the near-field segments.  NU: outputs per lane of the largest block (64 rank
+// rows in phase 1, the largest leaf in phase 2).
+template <int NT, int NY>
+static cudaError_t far64_run(hm_ctx *h, const double2 *U, const double2 *V, double2 *t, double2 *s, const double2 *ucl,
+                             double2 *y, int nrhs, bool near)
+{
+    const FarPlan &F = h->fplan;
+    const int n = h->plan.n, maxn = h->max_leaf;
+    const int ht = std::max(FAR_T1 * (65 + nrhs), (F64_NK * 64 * nrhs + 1) / 2);
+    const int hy = std::max(32 * ((maxn | 1) + nrhs), (F64_NK * maxn * nrhs + 1) / 2);
+    static DeviceOnce attr;
+    if (attr.need()) {   // nrhs <= 16, blocks of up to 64 rows
+        const int smax = (int)(sizeof(double2) * 2 * 32 * (65 + 16));
+        cudaError_t e;
+        if ((e = cudaFuncSetAttribute(k_far_t64<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax)) ||
+            (e = cudaFuncSetAttribute(k_far_y64<NY>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax)))
+            return e;
+        attr.done();
+    }
+    const int ntask = (int)F.p1_lo.size();
+    if (ntask > 0)
+        HM_LAUNCH(h, K_FAR1,
+                  k_far_t64<NT><<<ntask, F64_T, sizeof(double2) * 2 * ht, h->stream>>>(
+                      h->d_p1_lo, h->d_p1_hi, h->d_p1_ptr, h->d_p1_off, h->d_p1_ld, h->d_p1_rank, h->d_p1_row,
+                      h->d_p1_isv, U, V, ucl, nrhs, t, s, ht));
+    double2 *part = (double2 *)h->d_farpart;
+    HM_LAUNCH(h, K_FAR2,
+              k_far_y64<NY><<<h->nl * FAR_PARTS, F64_T, sizeof(double2) * 2 * hy, h->stream>>>(
+                  h->nl, h->d_leaf_ptr, h->d_part_ptr, h->d_seg_kcum, h->d_segs, h->d_zpart, h->d_zkcum, h->d_zsegs, U, V,
+                  near ? h->d_near : nullptr, t, s, ucl, h->d_cl2new, n, nrhs, part, hy));
+    const int64_t len = (int64_t)n * nrhs;
+    HM_LAUNCH(h, K_FAR2, k_far_sum<double2><<<nblk(len, 256), 256, 0, h->stream>>>(len, part, y));
+    return cudaGetLastError();
+}
+
+cudaError_t far_product64(hm_ctx *h, const double2 *U, const double2 *V, double2 *t, double2 *s, const double2 *ucl,
+                          double2 *y, int nrhs, bool near)
 {
     h->prof.cols[K_FAR1] += nrhs;
     h->prof.cols[K_FAR2] += nrhs;
-    if constexpr (sizeof(T) == 8)
-        if (h->far_kind == 2) return far_tc_launch(h, U, V, t, s, ucl, y, nrhs);
-    FarLaunch<T> f{h, U, V, t, s, ucl, y, nrhs};
-    return tile_dispatch<T>(nrhs, f);
+    if (nrhs <= 4) return far64_run<4, 4>(h, U, V, t, s, ucl, y, nrhs, near);
+    if (h->max_leaf <= 32) return far64_run<16, 8>(h, U, V, t, s, ucl, y, nrhs, near);
+    return far64_run<16, 16>(h, U, V, t, s, ucl, y, nrhs, near);
 }
 
-template cudaError_t far_product<double2>(hm_ctx *, const double2 *, const double2 *, double2 *, double2 *,
-                                          const double2 *, double2 *, int);
-template cudaError_t far_product<float2>(hm_ctx *, const float2 *, const float2 *, float2 *, float2 *,
-                                         const float2 *, float2 *, int);
+cudaError_t far_product32(hm_ctx *h, const float2 *U, const float2 *V, float2 *t, float2 *s, const float2 *ucl, float2 *y,
+                          int nrhs)
+{
+    h->prof.cols[K_FAR1] += nrhs;
+    h->prof.cols[K_FAR2] += nrhs;
+    if (h->far_kind == 2) return far_tc_launch(h, U, V, t, s, ucl, y, nrhs);
+    FarLaunch<float2> f{h, U, V, t, s, ucl, y, nrhs};
+    return tile_dispatch<float2>(nrhs, f);
+}
 
 }  // namespace hm

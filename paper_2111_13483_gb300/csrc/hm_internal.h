@@ -131,9 +131,10 @@ struct FarPlan {
     // each leaf's segments in FAR_PARTS consecutive parts of about equal contraction length:
     // part (l, p) covers segments part_ptr[l*FAR_PARTS + p] .. part_ptr[l*FAR_PARTS + p + 1]
     std::vector<int> part_ptr;
-    // near-field incidence lists (cluster order) for Z_N products: per leaf l, entries
-    // (b << 1 | side), side 0 = l is the row leaf t, 1 = l is the column leaf s (t != s)
-    std::vector<int> nptr, nent;
+    // the near-field blocks of each leaf as segments of the same form (F from the near blocks, Y = u), in
+    // FAR_PARTS parts: the Z u of the refinement residual
+    std::vector<int> zpart, zkcum;
+    std::vector<FarSegD> zsegs;
 };
 
 // Two-level sweeps (sweep2.cu): block rows per super-row, and one block row as a direction's sweep
@@ -194,12 +195,14 @@ struct hm_ctx {
     int64_t *d_near_off = nullptr;
     int *d_far_r0 = nullptr, *d_far_r1 = nullptr, *d_far_c0 = nullptr, *d_far_c1 = nullptr, *d_far_rank = nullptr;
     int64_t *d_far_uoff = nullptr, *d_far_voff = nullptr, *d_far_toff = nullptr;
-    int *d_flptr = nullptr, *d_flent = nullptr, *d_nptr = nullptr, *d_nent = nullptr, *d_far_item = nullptr;
+    int *d_flptr = nullptr, *d_flent = nullptr, *d_far_item = nullptr;
     int *d_p1_lo = nullptr, *d_p1_hi = nullptr, *d_p1_ptr = nullptr, *d_p1_ld = nullptr, *d_p1_rank = nullptr,
         *d_p1_row = nullptr, *d_p1_isv = nullptr;
     int64_t *d_p1_off = nullptr;
     int *d_seg_ptr = nullptr, *d_seg_kcum = nullptr, *d_part_ptr = nullptr;
-    hm::FarSegD *d_segs = nullptr;
+    hm::FarSegD *d_segs = nullptr, *d_zsegs = nullptr;
+    int *d_zpart = nullptr, *d_zkcum = nullptr;
+    int max_leaf = 0;
     int *d_leaf_ptr = nullptr, *d_perm = nullptr;
     int *d_new2cl = nullptr, *d_cl2new = nullptr, *d_new2orig = nullptr, *d_pos = nullptr;
     // device: plan
@@ -321,8 +324,10 @@ cudaError_t make_fp32_copies(hm_ctx *h);
 cudaError_t to_solve_order(hm_ctx *h, const double2 *src, int64_t lds, double2 *dst, int nrhs);
 cudaError_t to_orig_order(hm_ctx *h, const double2 *src, double2 *dst, int64_t ldd, int nrhs);
 cudaError_t z_apply_orig(hm_ctx *h, const double2 *x, double2 *y, int nrhs);
-template <class T>
-cudaError_t far_product(hm_ctx *h, const T *U, const T *V, T *t, T *s, const T *ucl, T *y, int nrhs);
+cudaError_t far_product64(hm_ctx *h, const double2 *U, const double2 *V, double2 *t, double2 *s, const double2 *ucl,
+                          double2 *y, int nrhs, bool near);   // near: Z_F + Z_N
+cudaError_t far_product32(hm_ctx *h, const float2 *U, const float2 *V, float2 *t, float2 *s, const float2 *ucl, float2 *y,
+                          int nrhs);
 cudaError_t ensure_solve_workspace(hm_ctx *h, int nrhs);
 void sweep_tune_release(hm_ctx *h);
 cudaError_t sweep2_setup(hm_ctx *h);

@@ -1162,38 +1162,6 @@ __global__ void __launch_bounds__(256) k_diag(int mode, int nb, const int *size,
     }
 }
 
-// Near-field product for the refinement residual: y += Z_N u, u in cluster order, y in solve
-// order.  One CTA per leaf, summing near blocks (t, s) and mirrored (s, t) blocks (FP64).
-__global__ void __launch_bounds__(128) k_near_mv(int nl, const int *leaf_ptr, const int *nptr, const int *nent,
-                                                 const int *near_t, const int *near_s, const int64_t *near_off,
-                                                 const double2 *near, const double2 *u, const int *cl2new, int n,
-                                                 int nrhs, double2 *y)
-{
-    const int l = blockIdx.x;
-    if (l >= nl) return;
-    const int a = leaf_ptr[l], ni = leaf_ptr[l + 1] - a;
-    const int on = cl2new[a];
-    for (int e = threadIdx.x; e < ni * nrhs; e += blockDim.x) {
-        const int i = e % ni, r = e / ni;
-        double2 acc = y[on + i + (int64_t)r * n];
-        for (int p = nptr[l]; p < nptr[l + 1]; ++p) {
-            const int b = nent[p] >> 1, side = nent[p] & 1;
-            const int t = near_t[b], s = near_s[b];
-            const int mt = leaf_ptr[t + 1] - leaf_ptr[t];
-            const double2 *B = near + near_off[b];
-            if (side == 0) {   // row l = t: sum_c B[i, c] u_s[c]
-                const int ms = leaf_ptr[s + 1] - leaf_ptr[s];
-                const double2 *us = u + (int64_t)leaf_ptr[s] * nrhs + r;
-                for (int c = 0; c < ms; ++c) acc = cfma(B[i + (int64_t)c * mt], us[(int64_t)c * nrhs], acc);
-            } else {           // row l = s (t != s): sum_q B[q, i] u_t[q]
-                const double2 *ut = u + (int64_t)leaf_ptr[t] * nrhs + r;
-                for (int q = 0; q < mt; ++q) acc = cfma(B[q + (int64_t)i * mt], ut[(int64_t)q * nrhs], acc);
-            }
-        }
-        y[on + i + (int64_t)r * n] = acc;
-    }
-}
-
 // ---- host side -------------------------------------------------------------------------
 static inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
@@ -1553,20 +1521,16 @@ static cudaError_t sweep(hm_ctx *h, const OpData<T> &d, bool forward, const T *x
     return e;
 }
 
-// y (solve order) = Z_F x (solve order); ucl receives the cluster-order copy of x with the
+// y (solve order) = Z_F x, or (Z_F + Z_N) x with near (FP64), x in solve order; ucl receives the cluster-order copy of x with the
 // right-hand sides interleaved (ucl[i*nrhs + r])
 template <class T>
-static cudaError_t far_apply(hm_ctx *h, const OpData<T> &d, const T *x, T *y, int nrhs, T *ucl)
+static cudaError_t far_apply(hm_ctx *h, const OpData<T> &d, const T *x, T *y, int nrhs, T *ucl, bool near = false)
 {
-    Plan &P = h->plan;
-    FarPlan &F = h->fplan;
-    const int n = P.n;
+    const int n = h->plan.n;
     HM_LAUNCH(h, K_PERMUTE, k_gather_il<T><<<nblk((int64_t)n * nrhs, 256), 256, 0, h->stream>>>(n, nrhs, h->d_cl2new, x,
                                                                                             ucl));
-    (void)F;
-    cudaError_t e = far_product<T>(h, d.U, d.V, d.t, d.s, ucl, y, nrhs);
-    if (e) return e;
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 16) return far_product64(h, d.U, d.V, d.t, d.s, ucl, y, nrhs, near);
+    else return far_product32(h, d.U, d.V, d.t, d.s, ucl, y, nrhs);
 }
 
 template <class T>
@@ -1667,11 +1631,7 @@ static cudaError_t op_chain(hm_ctx *h, const OpData<T> &d, int op, const T *x, T
         if (h->opts.preconditioner == 1) {   // block Jacobi: no coefficients, L = I
             switch (op) {
             case 0:   // A x = D^{-1} (Z_N + Z_F) x, D = diag(Z_kk)
-                if ((e = far_apply<T>(h, d, x, w1, nrhs, w2))) return e;   // w2: cluster-order copy of x
-                HM_LAUNCH(h, K_NEAR,
-                          k_near_mv<<<h->nl, 128, 0, h->stream>>>(h->nl, h->d_leaf_ptr, h->d_nptr, h->d_nent,
-                                                                  h->d_near_t, h->d_near_s, h->d_near_off, h->d_near,
-                                                                  w2, h->d_cl2new, n, nrhs, w1));
+                if ((e = far_apply<T>(h, d, x, w1, nrhs, w2, true))) return e;
                 return diag<T>(h, d, 1, w1, (const T *)nullptr, y, nrhs);
             case 1:
             case 2:
@@ -1682,11 +1642,7 @@ static cudaError_t op_chain(hm_ctx *h, const OpData<T> &d, int op, const T *x, T
         if (h->opts.preconditioner == 2 && op == 0) {
             // null-field comparison: A x = M^{-1} (Z_N + Z_F) x, M^{-1} = L^{-T} D^{-1} L^{-1}
             // with the factors of the elimination without fill
-            if ((e = far_apply<T>(h, d, x, w1, nrhs, w2))) return e;   // w2: cluster-order copy of x
-            HM_LAUNCH(h, K_NEAR,
-                      k_near_mv<<<h->nl, 128, 0, h->stream>>>(h->nl, h->d_leaf_ptr, h->d_nptr, h->d_nent, h->d_near_t,
-                                                              h->d_near_s, h->d_near_off, h->d_near, w2, h->d_cl2new,
-                                                              n, nrhs, w1));
+            if ((e = far_apply<T>(h, d, x, w1, nrhs, w2, true))) return e;
             if ((e = sweep<T>(h, d, true, w1, w0, nrhs))) return e;
             if ((e = diag<T>(h, d, 1, w0, (const T *)nullptr, w1, nrhs))) return e;
             return sweep<T>(h, d, false, w1, y, nrhs);
@@ -1760,11 +1716,7 @@ cudaError_t z_apply_orig(hm_ctx *h, const double2 *x, double2 *y, int nrhs)
     double2 *w0 = h->d_work, *w1 = h->d_work + (size_t)n * nrhs, *w2 = h->d_work + (size_t)2 * n * nrhs;
     HM_LAUNCH(h, K_PERMUTE,
               k_gather_cols<<<nblk((int64_t)n * nrhs, 256), 256, 0, h->stream>>>(n, nrhs, h->d_new2orig, x, n, w0));
-    if ((e = far_apply<double2>(h, data64(h), w0, w1, nrhs, w2))) return e;   // leaves the cluster-order copy in w2
-    HM_LAUNCH(h, K_NEAR,
-              k_near_mv<<<h->nl, 128, 0, h->stream>>>(h->nl, h->d_leaf_ptr, h->d_nptr, h->d_nent, h->d_near_t,
-                                                      h->d_near_s, h->d_near_off, h->d_near, w2, h->d_cl2new, n,
-                                                      nrhs, w1));
+    if ((e = far_apply<double2>(h, data64(h), w0, w1, nrhs, w2, true))) return e;
     HM_LAUNCH(h, K_PERMUTE,
               k_scatter_cols<<<nblk((int64_t)n * nrhs, 256), 256, 0, h->stream>>>(n, nrhs, h->d_new2orig, w1, y, n));
     return cudaGetLastError();

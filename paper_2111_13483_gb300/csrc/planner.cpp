@@ -535,6 +535,23 @@ void plan_order(hm_ctx *h)
     plan_superrows(P);
 }
 
+// each leaf's segments (ptr) in FAR_PARTS consecutive parts of about equal contraction length
+static void cut_parts(const std::vector<int> &ptr, const std::vector<int> &kcum, std::vector<int> &part)
+{
+    const int nl = (int)ptr.size() - 1;
+    part.assign((size_t)nl * FAR_PARTS + 1, ptr[nl]);
+    for (int l = 0; l < nl; ++l) {
+        const int b = ptr[l], e = ptr[l + 1];
+        const int64_t K = kcum[e] - kcum[b];
+        int q = b;
+        for (int p = 0; p < FAR_PARTS; ++p) {
+            part[(size_t)l * FAR_PARTS + p] = q;
+            const int64_t target = K * (p + 1) / FAR_PARTS;
+            while (q < e && kcum[q] - kcum[b] < target) ++q;
+        }
+    }
+}
+
 void plan_far(hm_ctx *h)
 {
     FarPlan &F = h->fplan;
@@ -561,15 +578,6 @@ void plan_far(hm_ctx *h)
     F.lent.clear();
     F.lent.reserve(F.lptr[nl]);
     for (int l = 0; l < nl; ++l) F.lent.insert(F.lent.end(), lists[l].begin(), lists[l].end());
-    std::vector<std::vector<int>> nl_lists(nl);
-    for (size_t b = 0; b < h->near_t.size(); ++b) {
-        nl_lists[h->near_t[b]].push_back((int)(b << 1));
-        if (h->near_t[b] != h->near_s[b]) nl_lists[h->near_s[b]].push_back((int)((b << 1) | 1));
-    }
-    F.nptr.assign(nl + 1, 0);
-    for (int l = 0; l < nl; ++l) F.nptr[l + 1] = F.nptr[l] + (int)nl_lists[l].size();
-    F.nent.clear();
-    for (int l = 0; l < nl; ++l) F.nent.insert(F.nent.end(), nl_lists[l].begin(), nl_lists[l].end());
     // phase-2 segments: every list entry of leaf l cut into contraction pieces of <= 32
     F.seg_ptr.assign(nl + 1, 0);
     F.segs.clear();
@@ -605,18 +613,35 @@ void plan_far(hm_ctx *h)
     }
     F.seg_kcum.assign(F.segs.size() + 1, 0);
     for (size_t q = 0; q < F.segs.size(); ++q) F.seg_kcum[q + 1] = F.seg_kcum[q] + F.segs[q].len;
-    F.part_ptr.assign((size_t)nl * FAR_PARTS + 1, 0);
-    for (int l = 0; l < nl; ++l) {
-        const int b = F.seg_ptr[l], e = F.seg_ptr[l + 1];
-        const int64_t K = F.seg_kcum[e] - F.seg_kcum[b];
-        int q = b;
-        for (int p = 0; p < FAR_PARTS; ++p) {
-            F.part_ptr[(size_t)l * FAR_PARTS + p] = q;
-            const int64_t target = K * (p + 1) / FAR_PARTS;
-            while (q < e && F.seg_kcum[q] - F.seg_kcum[b] < target) ++q;
-        }
+    cut_parts(F.seg_ptr, F.seg_kcum, F.part_ptr);
+    // the near-field blocks as segments: leaf l is the row leaf t (F = B) or the column leaf s (F = B^T)
+    std::vector<std::vector<int>> nl_lists(nl);
+    for (size_t b = 0; b < h->near_t.size(); ++b) {
+        nl_lists[h->near_t[b]].push_back((int)(b << 1));
+        if (h->near_t[b] != h->near_s[b]) nl_lists[h->near_s[b]].push_back((int)((b << 1) | 1));
     }
-    F.part_ptr[(size_t)nl * FAR_PARTS] = (int)F.segs.size();
+    std::vector<int> zptr(nl + 1, 0);
+    F.zsegs.clear();
+    for (int l = 0; l < nl; ++l) {
+        for (int en : nl_lists[l]) {
+            const int b = en >> 1, side = en & 1, o = side ? h->near_t[b] : h->near_s[b];
+            const int mt = h->leaf_ptr[h->near_t[b] + 1] - h->leaf_ptr[h->near_t[b]], K = h->leaf_ptr[o + 1] - h->leaf_ptr[o];
+            const FarSegD g = {h->near_off[b], h->leaf_ptr[o], side ? mt : 1, side ? 1 : mt, 0, 2 << 1};
+            for (int k0 = 0; k0 < K; k0 += 32) {
+                FarSegD q = g;
+                q.foff += (int64_t)k0 * g.fk;
+                q.yrow += k0;
+                q.len = std::min(32, K - k0);
+                F.zsegs.push_back(q);
+            }
+        }
+        zptr[l + 1] = (int)F.zsegs.size();
+    }
+    F.zkcum.assign(F.zsegs.size() + 1, 0);
+    for (size_t q = 0; q < F.zsegs.size(); ++q) F.zkcum[q + 1] = F.zkcum[q] + F.zsegs[q].len;
+    cut_parts(zptr, F.zkcum, F.zpart);
+    h->max_leaf = 0;
+    for (int l = 0; l < nl; ++l) h->max_leaf = std::max(h->max_leaf, h->leaf_ptr[l + 1] - h->leaf_ptr[l]);
     // rank-vector tasks: group the factor columns by the range they contract over
     // (V_b over the column range for t_b, U_b over the row range for s_b), 64 per task,
     // larger tasks first
