@@ -28,7 +28,6 @@
 
 namespace hm {
 
-constexpr int DOT_CHUNK = 4096;
 constexpr int MAX_OUTER = 40;
 
 // Packed column p, vector i of a family: base + (idx[p] + i * istep) * n.
@@ -42,17 +41,43 @@ struct VRef {
     }
 };
 
+// Rows of one CTA of the dot products.  By the length of the vectors alone, so that a column's sums do not
+// depend on the others.  Short vectors need many CTAs (ten columns of 7,680 rows in chunks of 4096 kept 20
+// SMs busy, 90 us a pass; in chunks of 512 it takes 9), long ones fewer partial sums.
+__host__ __device__ __forceinline__ int dot_chunk(int n) { return n < 16384 ? 512 : 1024; }
+
+// Sums v[0 .. 15] over the warp: lane l returns that of v[l >> 1].  Each step folds half of the remaining vectors onto
+// the other half's lanes, 16 complex additions instead of the 80 of a butterfly per vector (an FP64 addition holds
+// the scheduler 64 cycles, as many as the FMAs of a row).
+__device__ __forceinline__ double2 warp_sum16(double2 (&v)[16])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 8, o = 16; h > 0; h >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const double2 keep = up ? v[q + h] : v[q], give = up ? v[q] : v[q + h];
+            v[q].x = keep.x + __shfl_xor_sync(0xffffffffu, give.x, o);
+            v[q].y = keep.y + __shfl_xor_sync(0xffffffffu, give.y, o);
+        }
+    }
+    v[0].x += __shfl_xor_sync(0xffffffffu, v[0].x, 1);
+    v[0].y += __shfl_xor_sync(0xffffffffu, v[0].y, 1);
+    return v[0];
+}
+
 // part[((p*ldp + i) * nchunk + chunk)] = sum over the chunk's rows of conj(basis_i) w, i < J[p]
-// (J == nullptr: one vector)
+// (J == nullptr: one vector); with self, vector i = J[p] is w itself
 __global__ void __launch_bounds__(256, 2) k_dots(int n, VRef basis, const int *J, VRef w, double2 *part, int nchunk,
-                                                 int ldp)
+                                                 int ldp, int self)
 {
     constexpr int QB = 16;   // vectors per pass (16 accumulators per thread: two CTAs per SM)
-    __shared__ double2 red[8][QB + 1];
-    const int chunk = blockIdx.x, p = blockIdx.y;
-    const int lo = chunk * DOT_CHUNK, hi = min(n, lo + DOT_CHUNK);
+    __shared__ double2 red[8][QB];
+    const int chunk = blockIdx.x, p = blockIdx.y, rows = dot_chunk(n);
+    const int lo = chunk * rows, hi = min(n, lo + rows);
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    const int Jp = J ? J[p] : 1;
+    const int Jb = J ? J[p] : 1, Jp = Jb + self;
     const double2 *wc = w.at(p);
     for (int i0 = 0; i0 < Jp; i0 += QB) {
         const int ni = min(QB, Jp - i0);
@@ -60,20 +85,20 @@ __global__ void __launch_bounds__(256, 2) k_dots(int n, VRef basis, const int *J
 #pragma unroll
         for (int q = 0; q < QB; ++q) acc[q] = make_double2(0, 0);
         for (int row = lo + threadIdx.x; row < hi; row += blockDim.x) {
-            double2 wv = wc[row];
+            const double2 wv = wc[row];
 #pragma unroll
             for (int q = 0; q < QB; ++q)
-                if (q < ni) acc[q] = cjfma(basis.at(p, i0 + q)[row], wv, acc[q]);
+                if (q < ni) acc[q] = cjfma(i0 + q < Jb ? basis.at(p, i0 + q)[row] : wv, wv, acc[q]);
         }
-#pragma unroll
-        for (int q = 0; q < QB; ++q) {
-            if (q >= ni) break;
-            double2 v = acc[q];
+        if (ni == 1) {
             for (int o = 16; o > 0; o >>= 1) {
-                v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-                v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+                acc[0].x += __shfl_xor_sync(0xffffffffu, acc[0].x, o);
+                acc[0].y += __shfl_xor_sync(0xffffffffu, acc[0].y, o);
             }
-            if (lane == 0) red[wp][q] = v;
+            if (lane == 0) red[wp][0] = acc[0];
+        } else {
+            const double2 v = warp_sum16(acc);
+            if (!(lane & 1)) red[wp][lane >> 1] = v;
         }
         __syncthreads();
         if (threadIdx.x < ni) {
@@ -88,58 +113,70 @@ __global__ void __launch_bounds__(256, 2) k_dots(int n, VRef basis, const int *J
     }
 }
 
-// out[oidx[p]*ldo + i] = sum over chunks of part (fixed order), i < J[p]
+// h_i = sum over chunks of part (fixed order), i < J[p]: to out[oidx[p]*ldo + i], and added to fold[oidx[p]*ldo + i]
+// where given; vector J[p] of a pass with self: its norm to nrm[oidx[p]]
 __global__ void k_dots_final(int k, int ldp, const int *J, int nchunk, const double2 *part, double2 *out, int ldo,
-                             const int *oidx)
+                             const int *oidx, double2 *fold, double *nrm)
 {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= k * ldp) return;
     const int p = e / ldp, i = e % ldp;
-    if (i >= J[p]) return;
+    if (i > J[p] || (i == J[p] && !nrm)) return;
     double2 v = make_double2(0, 0);
     const double2 *q = part + (int64_t)e * nchunk;
     for (int c = 0; c < nchunk; ++c) {
         v.x += q[c].x;
         v.y += q[c].y;
     }
-    out[(int64_t)oidx[p] * ldo + i] = v;
+    if (i == J[p]) {
+        nrm[oidx[p]] = sqrt(fmax(0.0, v.x));
+        return;
+    }
+    const int64_t o = (int64_t)oidx[p] * ldo + i;
+    out[o] = v;
+    if (fold) {
+        fold[o].x += v.x;
+        fold[o].y += v.y;
+    }
 }
 
-// out[oidx[p]] = sqrt(max(0, Re sum over chunks of part[p]))   (a 2-norm from k_dots with J = 1)
+// out[oidx[p]] = sqrt(max(0, Re sum over chunks of part[p]))   (a 2-norm from k_dots with J = 1, or of the
+// partial sums of k_axpy_basis); one warp per column
 __global__ void k_norm_final(int k, int nchunk, const double2 *part, double *out, const int *oidx)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (p >= k) return;
     double v = 0.0;
     const double2 *q = part + (int64_t)p * nchunk;
-    for (int c = 0; c < nchunk; ++c) v += q[c].x;
-    out[oidx[p]] = sqrt(fmax(0.0, v));
+    for (int c = lane; c < nchunk; c += 32) v += q[c].x;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) out[oidx[p]] = sqrt(fmax(0.0, v));
 }
 
-// w_p -= sum_{i<J[p]} h[hidx[p]*ldh + i] basis_i(p)
-__global__ void k_axpy_basis(int n, int k, VRef basis, const int *J, const double2 *h, int ldh, const int *hidx,
-                             VRef w)
+// w_p -= sum_{i<J[p]} h[hidx[p]*ldh + i] basis_i(p); with part, part[p * gridDim.x + block] = the block's share of
+// ||w_p||^2 after it
+__global__ void __launch_bounds__(256) k_axpy_basis(int n, VRef basis, const int *J, const double2 *h, int ldh,
+                                                    const int *hidx, VRef w, double2 *part)
 {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= (int64_t)n * k) return;
-    const int row = (int)(e % n), p = (int)(e / n);
-    double2 *wp = w.at(p);
-    double2 acc = wp[row];
-    const double2 *hp = h + (int64_t)hidx[p] * ldh;
-    for (int i = 0; i < J[p]; ++i) acc = cfms(hp[i], basis.at(p, i)[row], acc);
-    wp[row] = acc;
-}
-
-// dst[idx[p]*ld + i] += src[idx[p]*ld + i], i < J[p]
-__global__ void k_hfold(int k, int ldp, const int *J, const int *idx, const double2 *src, double2 *dst, int ld)
-{
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= k * ldp) return;
-    const int p = e / ldp, i = e % ldp;
-    if (i >= J[p]) return;
-    const int64_t o = (int64_t)idx[p] * ld + i;
-    dst[o].x += src[o].x;
-    dst[o].y += src[o].y;
+    __shared__ double red[8];
+    const int row = blockIdx.x * 256 + threadIdx.x, p = blockIdx.y, Jp = J[p];
+    double2 acc = make_double2(0, 0);
+    if (row < n) {
+        double2 *wp = w.at(p);
+        acc = wp[row];
+        const double2 *hp = h + (int64_t)hidx[p] * ldh;
+        for (int i = 0; i < Jp; ++i) acc = cfms(hp[i], basis.at(p, i)[row], acc);
+        wp[row] = acc;
+    }
+    if (!part) return;
+    double v = fma(acc.x, acc.x, acc.y * acc.y);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < 8; ++q) v += red[q];
+        part[(int64_t)p * gridDim.x + blockIdx.x] = make_double2(v, 0);
+    }
 }
 
 // v_p = w_p / nrm[nidx[p]] (0 when the norm is 0)
@@ -304,11 +341,17 @@ struct Engine {
     std::vector<Slot> sl;
     static constexpr int NIDX = 24;
 
+    // partial sums: m + 2 dot products in chunks, or one norm in the blocks of k_axpy_basis
+    static size_t part_len(int n, int S, int m)
+    {
+        const int chunk = dot_chunk(n);
+        return (size_t)S * std::max((size_t)(n + chunk - 1) / chunk * (m + 2), (size_t)(n + 255) / 256);
+    }
+
     static size_t bytes(int n, int S, int m)
     {
-        const int nchunk = (n + DOT_CHUNK - 1) / DOT_CHUNK;
         size_t b = sizeof(double2) * (size_t)n * S * (5 + (m + 1) + 3);
-        b += sizeof(double2) * (size_t)nchunk * S * (m + 1);
+        b += sizeof(double2) * part_len(n, S, m);
         b += sizeof(double2) * (size_t)S * ((m + 1) * 2 + (m + 1) * m + (m + 1) + 2 * m);
         b += sizeof(double) * (size_t)S * (m + 5) + sizeof(int) * (size_t)S * (NIDX + 2);
         return b;
@@ -320,7 +363,7 @@ struct Engine {
         S = slots;
         m = restart;
         n = h->plan.n;
-        nchunk = (n + DOT_CHUNK - 1) / DOT_CHUNK;
+        nchunk = (n + dot_chunk(n) - 1) / dot_chunk(n);
         fp32 = h->opts.precision == 1;
         left = h->opts.preconditioner == 2;
         sl.assign(S, Slot());
@@ -334,7 +377,7 @@ struct Engine {
         if ((e = A((void **)&B, vs)) || (e = A((void **)&XO, vs)) || (e = A((void **)&R, vs)) ||
             (e = A((void **)&C, vs)) || (e = A((void **)&XT, vs)) || (e = A((void **)&Vb, vs * (m + 1))) ||
             (e = A((void **)&PX, vs)) || (e = A((void **)&PY, vs)) || (e = A((void **)&PT, vs)) ||
-            (e = A((void **)&part, sizeof(double2) * (size_t)nchunk * S * (m + 1))) ||
+            (e = A((void **)&part, sizeof(double2) * part_len(n, S, m))) ||
             (e = A((void **)&h2, sizeof(double2) * (size_t)S * (m + 1))) ||
             (e = A((void **)&s.hj, sizeof(double2) * (size_t)S * (m + 1))) ||
             (e = A((void **)&s.H, sizeof(double2) * (size_t)S * (m + 1) * m)) ||
@@ -390,8 +433,8 @@ struct Engine {
     // 2-norms of k packed vectors v -> out[oidx[p]]
     void norms(int k, VRef v, double *out, const int *oidx)
     {
-        HM_LAUNCH(h, K_DOTS, k_dots<<<dim3(nchunk, k), 256, 0, h->stream>>>(n, v, nullptr, v, part, nchunk, 1));
-        HM_LAUNCH(h, K_SMALL, k_norm_final<<<nblk(k, 128), 128, 0, h->stream>>>(k, nchunk, part, out, oidx));
+        HM_LAUNCH(h, K_DOTS, k_dots<<<dim3(nchunk, k), 256, 0, h->stream>>>(n, v, nullptr, v, part, nchunk, 1, 0));
+        HM_LAUNCH(h, K_SMALL, k_norm_final<<<nblk(k, 4), 128, 0, h->stream>>>(k, nchunk, part, out, oidx));
     }
 
     cudaError_t fetch(const double *d, std::vector<double> &hv)
@@ -604,20 +647,21 @@ struct Engine {
         cudaStream_t st = h->stream;
         vec(0, k, ref(Vb, vi), ref(Vb, vi), packed(PX));
         if ((e = op(0, PX, PY, k))) return e;
-        norms(k, w, s.wn, id);   // ||w|| before orthogonalisation (happy-breakdown reference)
-        // CGS2: h = V^H w, w -= V h, twice; coefficients accumulated in hj
-        HM_LAUNCH(h, K_DOTS, k_dots<<<dim3(nchunk, k), 256, 0, st>>>(n, basis, J, w, part, nchunk, m + 1));
+        // CGS2: h = V^H w, w -= V h, twice; coefficients accumulated in hj.  The first pass also gives ||w|| before
+        // orthogonalisation (happy-breakdown reference), the second subtraction h_{j+1,j} = ||w|| after it
+        const unsigned nr = nblk(n, 256);
+        HM_LAUNCH(h, K_DOTS, k_dots<<<dim3(nchunk, k), 256, 0, st>>>(n, basis, J, w, part, nchunk, m + 2, 1));
         HM_LAUNCH(h, K_SMALL,
-                  k_dots_final<<<nblk(k * (m + 1), 128), 128, 0, st>>>(k, m + 1, J, nchunk, part, s.hj, m + 1, id));
-        HM_LAUNCH(h, K_VEC,
-                  k_axpy_basis<<<nblk((int64_t)n * k, 256), 256, 0, st>>>(n, k, basis, J, s.hj, m + 1, id, w));
-        HM_LAUNCH(h, K_DOTS, k_dots<<<dim3(nchunk, k), 256, 0, st>>>(n, basis, J, w, part, nchunk, m + 1));
+                  k_dots_final<<<nblk(k * (m + 2), 128), 128, 0, st>>>(k, m + 2, J, nchunk, part, s.hj, m + 1, id, nullptr,
+                                                                       s.wn));
+        HM_LAUNCH(h, K_VEC, k_axpy_basis<<<dim3(nr, k), 256, 0, st>>>(n, basis, J, s.hj, m + 1, id, w, nullptr));
+        HM_LAUNCH(h, K_DOTS, k_dots<<<dim3(nchunk, k), 256, 0, st>>>(n, basis, J, w, part, nchunk, m + 2, 0));
         HM_LAUNCH(h, K_SMALL,
-                  k_dots_final<<<nblk(k * (m + 1), 128), 128, 0, st>>>(k, m + 1, J, nchunk, part, h2, m + 1, id));
-        HM_LAUNCH(h, K_VEC, k_axpy_basis<<<nblk((int64_t)n * k, 256), 256, 0, st>>>(n, k, basis, J, h2, m + 1, id, w));
-        HM_LAUNCH(h, K_SMALL, k_hfold<<<nblk(k * (m + 1), 128), 128, 0, st>>>(k, m + 1, J, id, h2, s.hj, m + 1));
-        // h_{j+1,j} = ||w||, v_{j+1} = w / h_{j+1,j}
-        norms(k, w, s.nrm, id);
+                  k_dots_final<<<nblk(k * (m + 2), 128), 128, 0, st>>>(k, m + 2, J, nchunk, part, h2, m + 1, id, s.hj,
+                                                                       nullptr));
+        HM_LAUNCH(h, K_VEC, k_axpy_basis<<<dim3(nr, k), 256, 0, st>>>(n, basis, J, h2, m + 1, id, w, part));
+        HM_LAUNCH(h, K_SMALL, k_norm_final<<<nblk(k, 4), 128, 0, st>>>(k, (int)nr, part, s.nrm, id));
+        // v_{j+1} = w / h_{j+1,j}
         HM_LAUNCH(h, K_VEC, k_scale<<<nblk((int64_t)n * k, 256), 256, 0, st>>>(n, k, s.nrm, id, w, ref(Vb, vo)));
         HM_LAUNCH(h, K_SMALL, k_givens<<<nblk(k, 64), 64, 0, st>>>(k, m, id, s));
         std::vector<double> res(S), wpre(S), wn(S);
