@@ -343,10 +343,10 @@ int hm_set_update_schedule(hm_handle h, int32_t kind);
  * 1 = one CTA; 2, 4 or 8 = a thread-block cluster of that many CTAs on as many SMs, each
  * eliminating a share of the columns, the pivot column passed through distributed shared
  * memory with one cluster barrier per pivot (same arithmetic per entry: the inverses are bitwise
- * those of one CTA); 0 = the default (8: on the 30,720-unknown sphere the 1,112 inversions of a
- * setup took 200, 162, 123 and 109 ms with 1, 2, 4 and 8 CTAs -- each column step still costs
- * a cluster barrier and the pivot search).  Both precisions; the block-Jacobi setup always
- * uses one CTA per block.  Takes effect at the next precond_setup.  HM_EINVAL for other values.
+ * those of one CTA); 0 = the default: 2 for blocks of up to 28 unknowns, 4 above (on the
+ * 30,720-unknown sphere the 1,107 inversions of a setup took 175, 113, 83 and 105 ms with 1, 2, 4
+ * and 8 CTAs).  Both precisions; the block-Jacobi setup always uses one CTA per block.
+ * Takes effect at the next precond_setup.  HM_EINVAL for other values.
  */
 int hm_set_pivot_schedule(hm_handle h, int32_t ctas);
 

@@ -255,7 +255,7 @@ struct hm_ctx {
     int sweep_fixed = 0;                 // a schedule code set by hm_set_sweep_schedule, 0 = tuned
     int far_kind = 1;                    // complex-FP32 far field: 1 CUDA cores, 2 tensor cores
     int update_kind = 1;                 // complex-FP32 Schur updates: 1 CUDA cores, 2 tensor cores
-    int pivot_cl = 8;                    // CTAs per pivot inversion (1 = one CTA; 2, 4, 8 = a cluster)
+    int pivot_cl = 0;                    // CTAs per pivot inversion (1, or a cluster of 2, 4, 8; 0 = by size)
     // fill-in compression packing (compress.cu): CTA b takes the blocks first[b] .. first[b+1]
     std::vector<int> cw_first;
     int *d_cw = nullptr;                 // first, then the block order, then the shared-memory offsets

@@ -9,7 +9,7 @@
 //                       ld n_k): W_kj = -alpha_kj of Eq. 14, the left coefficients being
 //                       their transposes (Sec. 3.2);
 //   Dinv + doff[k]      D_k^{-1} for the Eq. 28 preconditioner.
-// Step k: pivot inverse (one CTA), panel (M_k/64 CTAs), Schur updates
+// Step k: pivot inverse, panel, Schur updates
 // A_ij -= A_ik W_kj for i >= j in S_k (Eq. 19; diagonal blocks in full; one CTA per block
 // pair in FP64, one CTA per row block and group of up to 8 column blocks in FP32).  Stream
 // order gives the step dependencies.
@@ -18,6 +18,7 @@
 // complex FP32 in the mixed-precision setup, where the pivot blocks are still inverted in
 // FP64 (their inverse is kept in FP64 and as an FP32 copy for the panels and the inner
 // operator) and everything else stays FP32, so no step converts between the two.
+#include <algorithm>
 #include <cstdio>
 
 #include "cluster.cuh"
@@ -83,6 +84,25 @@ __global__ void k_scatter_near(int n_near, const int *near_t, const int *near_s,
     }
 }
 
+// the warp's largest key, the lowest row on ties; row n with no key
+__device__ __forceinline__ void gj_pick(unsigned long long &best, int &bi, int n)
+{
+    const bool any = bi < n;
+    const unsigned hi = any ? (unsigned)(best >> 32) : 0u;
+    const unsigned mhi = __reduce_max_sync(0xffffffffu, hi);
+    const bool c1 = any && hi == mhi;
+    const unsigned mlo = __reduce_max_sync(0xffffffffu, c1 ? (unsigned)best : 0u);
+    bi = (int)__reduce_min_sync(0xffffffffu, c1 && (unsigned)best == mlo ? (unsigned)bi : (unsigned)n);
+    best = (unsigned long long)mhi << 32 | mlo;
+}
+// conj(p) / |p|^2, |p|^2 = pv: the two divisions run on two lanes at once (a division is some ten FP64 instructions of
+// 64 cycles each)
+__device__ __forceinline__ double2 gj_reciprocal(double2 p, double pv)
+{
+    const double q = ((threadIdx.x & 1) ? -p.y : p.x) / pv;
+    return make_double2(__shfl_sync(0xffffffffu, q, 0), __shfl_sync(0xffffffffu, q, 1));
+}
+
 // Pivot search of Gauss-Jordan step c by one warp over rows r >= c of column `col` of a
 // (row-major, leading dimension ld): the largest |a_rc|^2, the lowest row on ties.  The
 // squares are compared as the integer bit patterns of non-negative doubles (same order as
@@ -98,192 +118,141 @@ __device__ __forceinline__ int gj_pivot(const double2 *a, int ld, int col, int c
         unsigned long long key = (unsigned long long)__double_as_longlong(fma(v.x, v.x, v.y * v.y));
         if (key > best || (key == best && r < bi) || bi == n) { best = key; bi = r; }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-        int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (oi < n && (ob > best || (ob == best && oi < bi) || bi == n)) { best = ob; bi = oi; }
-    }
+    gj_pick(best, bi, n);
     const double pv = __longlong_as_double((long long)best);
     *bad = !(pv > 1e-300) || best >= 0x7ff0000000000000ull;
-    const double2 pvv = a[bi * ld + col];
-    *d = make_double2(pvv.x / pv, -pvv.y / pv);
+    *d = gj_reciprocal(a[bi * ld + col], pv);
     return bi;
 }
 
 // Entry (r, j) of Gauss-Jordan step c: row c takes the scaled pivot row rc; column c becomes
 // -f d; every other entry cur - f rc (f = entry r of the pivot column after the interchange,
-// d = 1 / pivot).  Both inverse kernels use these two functions, so their results agree bit
-// for bit.
-__device__ __forceinline__ double2 gj_row(double2 ap, double2 d, bool pivot_col) { return pivot_col ? d : cmul(ap, d); }
-__device__ __forceinline__ double2 gj_entry(bool is_row, bool is_col, double2 rc, double2 f, double2 d, double2 cur)
+// d = 1 / pivot).
+__device__ __forceinline__ double2 gj_col(double2 f, double2 d)
 {
-    if (is_row) return rc;
-    if (is_col) return make_double2(-(f.x * d.x - f.y * d.y), -(f.x * d.y + f.y * d.x));
+    return make_double2(-(f.x * d.x - f.y * d.y), -(f.x * d.y + f.y * d.x));
+}
+__device__ __forceinline__ double2 gj_other(double2 rc, double2 f, double2 cur)
+{
     return make_double2(fma(-f.x, rc.x, fma(f.y, rc.y, cur.x)), fma(-f.x, rc.y, fma(-f.y, rc.x, cur.y)));
 }
 
 // In-place Gauss-Jordan inverse with partial pivoting (largest modulus, lowest row on
 // ties) of D_k = Ad[k], in FP64 whatever S is; result to Dinv[k] (and its FP32 copy when
-// Dinv32 is given).  err <- k+1 on a singular pivot.  Per column: one warp finds the pivot;
-// one pass forms the scaled pivot row and the pivot column and moves the old row c into
-// the pivot's row; one pass eliminates (four fused multiply-adds per entry) and writes the
-// new row c.
-template <class S>
-__global__ void __launch_bounds__(256) k_pivot_inverse(int kbase, const int *size, const int64_t *doff, const S *Ad,
-                                                       double2 *Dinv, float2 *Dinv32, int *err)
+// Dinv32 is given).  err <- k+1 on a singular pivot.  One block per CTA, or per cluster of CL CTAs of
+// which CTA q keeps the columns j = q, q + CL, ....  Rows lie on the lanes, a warp takes a column at a
+// time, and the columns are kept in two copies that the steps read and write in turn, so a step has no
+// barrier inside.  Step c eliminates with the pivot row p, 1 / pivot and the interchanged column c found in the step
+// before (two alternating buffers; in a cluster they are pushed to every CTA through distributed shared
+// memory).  Warp 0 of the CTA that holds column c + 1 eliminates that column first, searches it for the next
+// pivot and publishes it, while the other warps eliminate the rest; one barrier ends the step.  The
+// results agree bit for bit whatever CL is: each entry goes through cmul, gj_col and gj_other alone.  The
+// row interchanges are undone by writing column x of the result from the column they moved there.
+//
+// What binds it: an FP64 instruction holds its scheduler 64 cycles and so does the next one that needs its result
+// (a division 565), so the chain to the next pivot -- a product, an elimination, two squares, a search, a
+// division -- takes about 1 us beside the elimination itself (four instructions per column, 32 rows and
+// scheduler) and, in a cluster, the pushes and a barrier (400 cycles).  Four warps, one per scheduler, leave
+// the chain's scheduler to it.  Searching, scaling and eliminating one after the other with a barrier
+// between took 3.5 us a pivot on eight CTAs: 104 ms per setup of the 30,720-unknown sphere, now 83.
+template <int CL> __device__ __forceinline__ void pivot_sync()
 {
-    const int k = kbase + blockIdx.x;   // one block per CTA (block Jacobi inverts all at once)
-    extern __shared__ double2 sm[];
-    const int n = size[k];
-    const int ld = n + 1;                      // padded
-    double2 *a = sm;                           // n x ld, row-major a[r*ld + c]
-    double2 *rowc = sm + n * ld;               // n: pivot row after scaling
-    double2 *colc = rowc + n;                  // n: pivot column (rows after the interchange)
-    __shared__ int piv[64];
-    __shared__ int s_p;
-    __shared__ double2 s_d;
-    const S *D = Ad + doff[k];
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-        int r = e % n, c = e / n;
-        a[r * ld + c] = cwiden(D[e]);
-    }
-    __syncthreads();
-    for (int c = 0; c < n; ++c) {
-        if (threadIdx.x < 32) {
-            double2 d;
-            bool bad;
-            const int bi = gj_pivot(a, ld, c, c, n, &d, &bad);
-            if (threadIdx.x == 0) {
-                s_p = bi;
-                piv[c] = bi;
-                s_d = d;
-                if (bad) atomicCAS(err, 0, k + 1);
-            }
-        }
-        __syncthreads();
-        const int p = s_p;
-        const double2 d = s_d;
-        // rows c and p interchanged: the new row c is the old row p
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            const double2 ap = a[p * ld + j];
-            rowc[j] = gj_row(ap, d, j == c);
-            colc[j] = a[(j == p ? c : j) * ld + c];
-            if (p != c) a[p * ld + j] = a[c * ld + j];
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-            const int r = e / n, j = e % n;
-            a[r * ld + j] = gj_entry(r == c, j == c, rowc[j], colc[r], d, a[r * ld + j]);
-        }
-        __syncthreads();
-    }
-    // undo the row interchanges as column interchanges, last first
-    for (int c = n - 1; c >= 0; --c) {
-        int p = piv[c];
-        if (p != c)
-            for (int r = threadIdx.x; r < n; r += blockDim.x) {
-                double2 t = a[r * ld + c];
-                a[r * ld + c] = a[r * ld + p];
-                a[r * ld + p] = t;
-            }
-        __syncthreads();
-    }
-    double2 *out = Dinv + doff[k];
-    float2 *out32 = Dinv32 ? Dinv32 + doff[k] : nullptr;
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-        int r = e % n, c = e / n;
-        const double2 v = a[r * ld + c];
-        out[e] = v;
-        if (out32) out32[e] = make_float2((float)v.x, (float)v.y);
-    }
+    if (CL > 1) cluster_sync();
+    else __syncthreads();
 }
 
-// The same inverse on a cluster of CL CTAs (one block per cluster), so that the FP64 pipes of
-// CL SMs share the elimination.  CTA q keeps the columns j = q, q + CL, ... of the in-place
-// array (row-major, n x nloc).  Step c: the CTA that owns column c finds the pivot and
-// stores p, 1 / pivot and the interchanged column c into every CTA of the cluster (two
-// alternating buffers, distributed shared memory), then one cluster barrier; every CTA then
-// interchanges, scales and eliminates its own columns with gj_row / gj_entry, entry for entry
-// the operations of k_pivot_inverse, so the inverse is bitwise the same.  The row
-// interchanges are undone by writing column x of the result from the column the interchanges
-// moved there.  Every CTA takes all n + 1 cluster barriers (a CTA without columns too).
-// Buffer b = c & 1 is rewritten at step c + 2 only after every CTA has passed the barrier of
-// step c + 1, which it reaches after its elimination of step c.
 template <class S, int CL>
-__global__ void __launch_bounds__(128) k_pivot_inverse_cl(int kbase, const int *size, const int64_t *doff, const S *Ad,
-                                                          double2 *Dinv, float2 *Dinv32, int *err)
+__global__ void __launch_bounds__(128) k_pivot_inverse(int kbase, const int *size, const int64_t *doff, const S *Ad,
+                                                       double2 *Dinv, float2 *Dinv32, int *err)
 {
-    const int q = (int)cluster_rank();
+    const int q = CL > 1 ? (int)cluster_rank() : 0, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const int k = kbase + (int)(blockIdx.x / CL);
     extern __shared__ double2 sm[];
     const int n = size[k];
     const int nloc = (n - q + CL - 1) / CL;    // columns q, q + CL, ... below n
-    const int ld = nloc + 1;
-    double2 *a = sm;                           // n x ld, a[r * ld + jl] = column jl * CL + q
-    double2 *rowc = sm + n * ld;               // nloc: the scaled pivot row
-    __shared__ double2 s_col[2][64];           // pivot column after the interchange (pushed)
-    __shared__ double2 s_d[2];                 // 1 / pivot (pushed)
-    __shared__ int s_p[2];                     // pivot row (pushed)
+    double2 *a = sm;                           // 2 x nloc x n: a[(copy * nloc + jl) * n + r] = column jl * CL + q
+    __shared__ double2 s_col[2][64];           // pivot column after the interchange
+    __shared__ double2 s_d[2];                 // 1 / pivot
+    __shared__ int s_p[2];                     // pivot row
     __shared__ int piv[64];
     __shared__ int at[64];
     const S *D = Ad + doff[k];
     for (int e = threadIdx.x; e < n * nloc; e += blockDim.x) {
         const int r = e % n, jl = e / n;
-        a[r * ld + jl] = cwiden(D[r + (int64_t)(jl * CL + q) * n]);
+        a[e] = cwiden(D[r + (int64_t)(jl * CL + q) * n]);
     }
-    cluster_sync();   // every CTA of the cluster is running before any remote store
+    // one warp: the pivot of column c in col (rows >= c), to every CTA's buffer c & 1 with the column
+    auto publish = [&](const double2 *col, int c) {
+        double2 d;
+        bool bad;
+        const int p = gj_pivot(col, 1, 0, c, n, &d, &bad), b = c & 1;
+        if (lane == 0 && bad) atomicCAS(err, 0, k + 1);
+        for (int dst = 0; CL > 1 && dst < CL; ++dst) {
+            for (int r = lane; r < n; r += 32)
+                st_remote_d2(cluster_map(smem_addr(&s_col[b][r]), (unsigned)dst), col[r == p ? c : r]);
+            if (lane == dst) {
+                st_remote_d2(cluster_map(smem_addr(&s_d[b]), (unsigned)dst), d);
+                st_remote_s32(cluster_map(smem_addr(&s_p[b]), (unsigned)dst), p);
+            }
+        }
+        if (CL == 1) {
+            for (int r = lane; r < n; r += 32) s_col[b][r] = col[r == p ? c : r];
+            if (lane == 0) {
+                s_d[b] = d;
+                s_p[b] = p;
+            }
+        }
+    };
+    pivot_sync<CL>();   // the columns are loaded; every CTA of the cluster is running before any remote store
+    if (q == 0 && wp == 0) publish(a, 0);
+    pivot_sync<CL>();
     for (int c = 0; c < n; ++c) {
-        const int b = c & 1;
-        if (q == c % CL) {
-            const int col = c / CL;
-            __shared__ int o_p;
-            __shared__ double2 o_d;
-            if (threadIdx.x < 32) {
-                double2 d;
-                bool bad;
-                const int bi = gj_pivot(a, ld, col, c, n, &d, &bad);
-                if (threadIdx.x == 0) {
-                    o_p = bi;
-                    o_d = d;
-                    if (bad) atomicCAS(err, 0, k + 1);
-                }
-            }
-            __syncthreads();
-            const int p = o_p;
-            for (int x = threadIdx.x; x < CL * (n + 1); x += blockDim.x) {
-                const int dst = x / (n + 1), r = x % (n + 1);
-                if (r < n)
-                    st_remote_d2(cluster_map(smem_addr(&s_col[b][r]), (unsigned)dst), a[(r == p ? c : r) * ld + col]);
-                else {
-                    st_remote_d2(cluster_map(smem_addr(&s_d[b]), (unsigned)dst), o_d);
-                    st_remote_s32(cluster_map(smem_addr(&s_p[b]), (unsigned)dst), p);
-                }
-            }
-        }
-        cluster_sync();
-        const int p = s_p[b];
+        const int b = c & 1, p = s_p[b];
         const double2 d = s_d[b];
+        const double2 *cur = a + b * nloc * n;
+        double2 *nxt = a + (b ^ 1) * nloc * n;
         if (threadIdx.x == 0) piv[c] = p;
-        for (int jl = threadIdx.x; jl < nloc; jl += blockDim.x) {
-            const int j = jl * CL + q;
-            rowc[jl] = gj_row(a[p * ld + jl], d, j == c);
-            if (p != c) a[p * ld + jl] = a[c * ld + jl];
+        auto eliminate = [&](int jl, double2 rc) {
+            const double2 *x = cur + jl * n;
+            double2 *y = nxt + jl * n;
+            if (jl * CL + q == c)   // the warp's whole column: one branch, not both products for every entry
+                for (int r = lane; r < n; r += 32) y[r] = r == c ? d : gj_col(s_col[b][r], d);
+            else
+                for (int r = lane; r < n; r += 32) {
+                    const double2 v = gj_other(rc, s_col[b][r], x[r == p ? c : r]);
+                    y[r] = r == c ? rc : v;
+                }
+        };
+        const bool mine = c + 1 < n && (c + 1) % CL == q;   // the next pivot's column is here
+        const int first = mine ? (c + 1) / CL : nloc;
+        if (mine && wp == 0) {
+            eliminate(first, cmul(cur[first * n + p], d));
+            __syncwarp();
+            publish(nxt + first * n, c + 1);
         }
-        __syncthreads();
-        for (int e = threadIdx.x; e < n * nloc; e += blockDim.x) {
-            const int r = e / nloc, jl = e % nloc;
-            a[r * ld + jl] = gj_entry(r == c, jl * CL + q == c, rowc[jl], s_col[b][r], d, a[r * ld + jl]);
+        // the other columns [lo, hi) of this warp (the search takes warp 0 as long as six columns); lane l scales the
+        // pivot row's entry of the l-th of them
+        const int cols = mine ? nloc - 1 : nloc, c0 = mine ? max(cols - 18, 0) / 4 : (cols + 3) / 4;
+        const int each = (cols - c0 + 2) / 3, lo = wp == 0 ? 0 : min(c0 + (wp - 1) * each, cols);
+        const int hi = wp == 0 ? c0 : min(lo + each, cols);
+        const int j0 = lo + lane < first ? lo + lane : lo + lane + 1;
+        double2 rcl = make_double2(0.0, 0.0);
+        if (lo + lane < hi) rcl = cmul(cur[j0 * n + p], d);
+        for (int t = lo; t < hi; ++t) {
+            const double2 rc = make_double2(__shfl_sync(0xffffffffu, rcl.x, t - lo), __shfl_sync(0xffffffffu, rcl.y, t - lo));
+            eliminate(t < first ? t : t + 1, rc);
         }
-        __syncthreads();
+        pivot_sync<CL>();
     }
+    a += (n & 1) * nloc * n;   // the copy the last step wrote
     // at[x] = the column of the array that the interchanges (undone last first) move to x
-    if (threadIdx.x == 0) {
-        for (int x = 0; x < n; ++x) at[x] = x;
-        for (int c = n - 1; c >= 0; --c) {
-            const int t = at[c];
-            at[c] = at[piv[c]];
-            at[piv[c]] = t;
+    for (int x = threadIdx.x; x < n; x += blockDim.x) {   // position x followed back through them
+        int pos = x;
+        for (int c = 0; c < n; ++c) {
+            const int p = piv[c];
+            pos = pos == c ? p : pos == p ? c : pos;
         }
+        at[x] = pos;
     }
     __syncthreads();
     double2 *out = Dinv + doff[k];
@@ -291,139 +260,105 @@ __global__ void __launch_bounds__(128) k_pivot_inverse_cl(int kbase, const int *
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
         const int r = e % n, x = e / n, src = at[x];
         if (src % CL != q) continue;
-        const double2 v = a[r * ld + src / CL];
+        const double2 v = a[src / CL * n + r];
         out[e] = v;
         if (out32) out32[e] = make_float2((float)v.x, (float)v.y);
     }
 }
 
-// W_k[:, c0:c0+64] = D_k^{-1} (A_col_k[c0:c0+64, :])^T in S arithmetic
+// W_k[:, c0 : c0 + PC] = D_k^{-1} (A_col_k[c0 : c0 + PC, :])^T in S arithmetic.  Few columns per CTA spread a step's panel
+// over the SMs: 64 FP64 columns of an 18-unknown block held one SM's DFMA pipe for 20 us.
+template <class S> constexpr int PANEL_COLS = sizeof(S) == 16 ? 16 : 32;
+template <class S> size_t panel_smem(int nk) { return sizeof(S) * (size_t)nk * ((nk | 1) + (PANEL_COLS<S> | 1)); }
 template <class S>
 __global__ void __launch_bounds__(256) k_panel(int k, const int *size, const int *M, const int64_t *coff,
                                                const int64_t *doff, const S *Dinv, const S *A, S *W)
 {
+    constexpr int PC = PANEL_COLS<S>, LC = PC | 1;
     extern __shared__ unsigned char psraw[];
-    S *dinv = (S *)psraw;             // dinv[r*65 + q] = D_k^{-1}[r, q]
-    S *ac = dinv + 64 * 65;           // ac[q*65 + col] = A_col[c0+col, q]
-    const int n = size[k], Mk = M[k];
-    const int c0 = blockIdx.x * 64;
-    const int nc = min(64, Mk - c0);
+    const int n = size[k], Mk = M[k], ld = n | 1;
+    S *dinv = (S *)psraw;             // dinv[r*ld + q] = D_k^{-1}[r, q]
+    S *ac = dinv + n * ld;            // ac[q*LC + col] = A_col[c0+col, q]
+    const int c0 = blockIdx.x * PC;
+    const int nc = min(PC, Mk - c0);
     const S *Di = Dinv + doff[k];
     const S *Ac = A + coff[k];
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
         int r = e % n, q = e / n;
-        dinv[r * 65 + q] = Di[e];
+        dinv[r * ld + q] = Di[e];
     }
     for (int e = threadIdx.x; e < nc * n; e += blockDim.x) {
         int col = e % nc, q = e / nc;
-        ac[q * 65 + col] = Ac[(c0 + col) + (int64_t)q * Mk];
+        ac[q * LC + col] = Ac[(c0 + col) + (int64_t)q * Mk];
     }
     __syncthreads();
     S *Wk = W + coff[k];
     for (int e = threadIdx.x; e < n * nc; e += blockDim.x) {
         int r = e % n, col = e / n;
         S acc = czero(S());
-        for (int q = 0; q < n; ++q) acc = cfma(dinv[r * 65 + q], ac[q * 65 + col], acc);
+        for (int q = 0; q < n; ++q) acc = cfma(dinv[r * ld + q], ac[q * LC + col], acc);
         Wk[r + (int64_t)(c0 + col) * n] = acc;
     }
 }
 
-// Schur updates of step k (Eq. 19), FP64 setup: one CTA per pair (a >= b) of S_k,
-// A_ij -= A_ik W_kj, in S arithmetic (the FP32 setup uses k_update_grp below).  C (ni x nj) -= A (ni x nk) W (nk x nj) on a 16U x 16U tile: thread
-// (tx, ty) owns rows tx + 16u and columns ty + 16v (u, v < U).  The shared tiles are
-// zero-padded to the tile size, so every thread runs the same unpredicated FMA sequence;
-// padded outputs are dropped.
-template <class S, int QC, int U>
-__device__ __forceinline__ void update_tile(S (*As)[65], S (*Ws)[65], const S *Aik, int Mk, const S *Wkj, int nk,
-                                            int ni, int nj, S *C, int ldc)
+// Schur updates of step k (Eq. 19), FP64 setup: one CTA per pair (a >= b) of S_k, A_ij -= A_ik W_kj.  The
+// outputs of the block lie flat over the threads: a DFMA warp instruction holds its scheduler for 64 cycles whatever its
+// lanes do and shared-memory loads are free beside it, so full warps count, not register tiles (32 x 32 tiles
+// padded the 18-unknown blocks of a 4,720-unknown plate threefold: 59 ms per setup).
+constexpr int UPD64_T = 128;
+__device__ __forceinline__ void upd64_cp(double2 *dst, const double2 *src)
 {
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    constexpr int TS = 16 * U;
-    S acc[U][U];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int v = 0; v < U; ++v) acc[u][v] = czero(S());
-    for (int q0 = 0; q0 < nk; q0 += QC) {
-        const int nq = min(QC, nk - q0);
-        stage_copy<4>(
-            TS * nq, [&](int e) { return e % TS < ni ? Aik[e % TS + (int64_t)(q0 + e / TS) * Mk] : czero(S()); },
-            [&](int e, S v) { As[e / TS][e % TS] = v; });
-        stage_copy<4>(
-            nq * TS, [&](int e) { return e / nq < nj ? Wkj[(q0 + e % nq) + (int64_t)(e / nq) * nk] : czero(S()); },
-            [&](int e, S v) { Ws[e % nq][e / nq] = v; });
-        __syncthreads();
-        for (int q = 0; q < nq; ++q) {
-            S av[U], wv[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) av[u] = As[q][tx + 16 * u];
-#pragma unroll
-            for (int v = 0; v < U; ++v) wv[v] = Ws[q][ty + 16 * v];
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-#pragma unroll
-                for (int v = 0; v < U; ++v) acc[u][v] = cfma(av[u], wv[v], acc[u][v]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int v = 0; v < U; ++v) {
-            const int r = tx + 16 * u, c = ty + 16 * v;
-            if (r < ni && c < nj) {
-                S *p = C + r + (int64_t)c * ldc;
-                S o = *p;
-                o.x -= acc[u][v].x;
-                o.y -= acc[u][v].y;
-                *p = o;
-            }
-        }
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
 }
-
-template <class S>
-__global__ void __launch_bounds__(256) k_update(int k, int ns, const int *size, const int *sptr, const int *sidx,
-                                                const int *srow, const int *M, const int64_t *coff,
-                                                const int64_t *doff, const S *W, S *A, S *Ad)
+__global__ void __launch_bounds__(UPD64_T) k_update64(int k, int ns, const int *size, const int *sptr, const int *sidx,
+                                                      const int *srow, const int *M, const int64_t *coff,
+                                                      const int64_t *doff, const double2 *W, double2 *A, double2 *Ad)
 {
-    constexpr int QC = sizeof(S) == 16 ? 16 : 32;
-    __shared__ S As[QC][65];   // As[q][r] = A_ik[r, q0+q]
-    __shared__ S Ws[QC][65];   // Ws[q][c] = W_kj[q0+q, c]
+    extern __shared__ double2 upd64_sm[];
     // triangular index -> (a, b), a >= b (integer arithmetic only)
     const long t = blockIdx.x;
     int a = (int)sqrtf(2.0f * (float)t);
     while ((long)(a + 1) * (a + 2) / 2 <= t) ++a;
     while ((long)a * (a + 1) / 2 > t) --a;
-    int b = (int)(t - (long)a * (a + 1) / 2);
+    const int b = (int)(t - (long)a * (a + 1) / 2);
     if (a >= ns) return;
     const int e0 = sptr[k];
     const int i = sidx[e0 + a], j = sidx[e0 + b];
     const int nk = size[k], ni = size[i], nj = size[j];
     const int Mk = M[k];
-    const S *Aik = A + coff[k] + srow[e0 + a];                 // ld Mk
-    const S *Wkj = W + coff[k] + (int64_t)srow[e0 + b] * nk;   // ld nk
-    S *C;
+    const double2 *Aik = A + coff[k] + srow[e0 + a];                 // ld Mk
+    const double2 *Wkj = W + coff[k] + (int64_t)srow[e0 + b] * nk;   // ld nk
+    double2 *C;
     int ldc;
     if (i == j) {
         C = Ad + doff[i];
         ldc = ni;
     } else {
         int r = find_row(sptr, sidx, srow, j, i);
-        if (r < 0) return;   // cannot happen when S is the symbolic fill (i in S_j)
+        if (r < 0) return;   // a dropped update of the elimination without fill (else i is in S_j)
         C = A + coff[j] + r;
         ldc = M[j];
     }
-    if (ni <= 32 && nj <= 32)
-        update_tile<S, QC, 2>(As, Ws, Aik, Mk, Wkj, nk, ni, nj, C, ldc);
-    else
-        update_tile<S, QC, 4>(As, Ws, Aik, Mk, Wkj, nk, ni, nj, C, ldc);
+    double2 *As = upd64_sm, *Ws = As + ni * nk;                      // As[q * ni + r] = A_ik[r, q], Ws[c * nk + q] = W_kj[q, c]
+    for (int e = threadIdx.x; e < ni * nk; e += UPD64_T) upd64_cp(As + e, Aik + e % ni + (int64_t)(e / ni) * Mk);
+    for (int e = threadIdx.x; e < nk * nj; e += UPD64_T) upd64_cp(Ws + e, Wkj + e);
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncthreads();
+    for (int e = threadIdx.x; e < ni * nj; e += UPD64_T) {
+        const int r = e % ni, c = e / ni;
+        double2 *p = C + r + (int64_t)c * ldc;
+        const double2 old = *p;
+        double2 acc = make_double2(0.0, 0.0);
+        for (int q = 0; q < nk; ++q) acc = cfma(As[q * ni + r], Ws[c * nk + q], acc);
+        *p = make_double2(old.x - acc.x, old.y - acc.y);
+    }
 }
 
 // Grouped Schur updates of step k for the complex-FP32 setup.  CTA -> (a, g): row block a
 // of S_k and the column blocks b = g*gb .. min(a, g*gb + gb - 1).  For each, C_ij -= A_ik W_kj
-// with the thread layout and q order of update_tile, so the result is bitwise that of
-// k_update, on a tile fitted to the block in steps of 16 rows and columns (update_tile pads
-// to 32 x 32 or 64 x 64: up to 5x the useful FMAs for uneven pairs).  A_ik is staged once
+// on a tile fitted to the block in steps of 16 rows and columns (tiles of 32 x 32 or 64 x 64
+// take up to 5x the useful FMAs for uneven pairs).  A_ik is staged once
 // per CTA, the W_kj blocks stream through two cp.async buffers (the copy of the next overlaps
 // the product of the current) and each C block's old values are loaded before its product,
 // so their latency hides behind the FMAs.
@@ -444,7 +379,7 @@ __device__ __forceinline__ void upd_cp(float2 *dst, const float2 *src)
 }
 
 // C (ni x nj) -= A W on a (16 UR) x (16 UC) tile, UR = ceil(ni / 16), UC = ceil(nj / 16):
-// thread (tx, ty) owns rows tx + 16u and columns ty + 16v, as in update_tile.
+// thread (tx, ty) owns rows tx + 16u and columns ty + 16v.
 template <int UR, int UC>
 __device__ __forceinline__ void upd_product(const float2 (*As)[UPD_LD], const float2 (*Ws)[UPD_LD], int nk, int ni,
                                             int nj, float2 *C, int ldc)
@@ -652,37 +587,49 @@ static int upd_group(int ns, int nsm)
     return gb;
 }
 
-// one pivot block on a cluster of h->pivot_cl CTAs (2, 4 or 8)
-template <class S>
-static cudaError_t pivot_cluster(hm_ctx *h, int k, int nk, const S *Ad, float2 *Dinv32)
+// count pivot blocks from k on, of at most nk unknowns, each on CL CTAs
+template <class S, int CL>
+static cudaError_t pivot_launch(hm_ctx *h, int k, int count, int nk, const S *Ad, float2 *Dinv32)
 {
-    const int C = h->pivot_cl;
-    const int nloc = (nk + C - 1) / C;
+    const size_t smem = sizeof(double2) * 2 * (size_t)nk * ((nk + CL - 1) / CL);
+    static DeviceOnce attr;
+    if (attr.need()) {
+        const cudaError_t e = cudaFuncSetAttribute(k_pivot_inverse<S, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(sizeof(double2) * 2 * 64 * (64 / CL)));
+        if (e) return e;
+        attr.done();
+    }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)C, 1, 1);
-    cfg.blockDim = dim3(128, 1, 1);
-    cfg.dynamicSmemBytes = sizeof(double2) * ((size_t)nk * (nloc + 1) + nloc);
+    cfg.gridDim = dim3((unsigned)(CL * count), 1, 1);
+    cfg.blockDim = dim3(128, 1, 1);   // one warp per scheduler
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = h->stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.x = CL;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = CL > 1 ? 1 : 0;
     cudaError_t e = cudaSuccess;
-    const int *sz = h->d_size;
-    const int64_t *dof = h->d_doff;
-    double2 *Dinv = h->d_Dinv;
-    int *err = h->d_err;
-    if (C == 2)
-        HM_LAUNCH(h, K_PIVOT, e = cudaLaunchKernelEx(&cfg, k_pivot_inverse_cl<S, 2>, k, sz, dof, Ad, Dinv, Dinv32, err));
-    else if (C == 4)
-        HM_LAUNCH(h, K_PIVOT, e = cudaLaunchKernelEx(&cfg, k_pivot_inverse_cl<S, 4>, k, sz, dof, Ad, Dinv, Dinv32, err));
-    else
-        HM_LAUNCH(h, K_PIVOT, e = cudaLaunchKernelEx(&cfg, k_pivot_inverse_cl<S, 8>, k, sz, dof, Ad, Dinv, Dinv32, err));
-    if (e) return e;
-    return cudaGetLastError();
+    HM_LAUNCH(h, K_PIVOT,
+              e = cudaLaunchKernelEx(&cfg, k_pivot_inverse<S, CL>, k, (const int *)h->d_size, (const int64_t *)h->d_doff, Ad,
+                                     h->d_Dinv, Dinv32, h->d_err));
+    return e ? e : cudaGetLastError();
+}
+
+// One pivot block on h->pivot_cl CTAs.  By default on two up to 28 unknowns, where the pushes to more CTAs cost what
+// their schedulers save (4,720-unknown plate, blocks of 18: 11.7 / 10.2 / 11.7 / 14.8 ms per setup on 1 / 2 /
+// 4 / 8; 29,800-unknown plate, 29: 101 / 70 / 71 / 91), on four above (1,920-unknown sphere, 34: 11.5 / 7.2 /
+// 5.1 / 6.6 ms; 30,720-unknown sphere: 175 / 113 / 83 / 105 ms).
+template <class S> static cudaError_t pivot_step(hm_ctx *h, int k, int nk, const S *Ad, float2 *Dinv32)
+{
+    switch (h->pivot_cl ? h->pivot_cl : nk <= 28 ? 2 : 4) {
+    case 2: return pivot_launch<S, 2>(h, k, 1, nk, Ad, Dinv32);
+    case 4: return pivot_launch<S, 4>(h, k, 1, nk, Ad, Dinv32);
+    case 8: return pivot_launch<S, 8>(h, k, 1, nk, Ad, Dinv32);
+    default: return pivot_launch<S, 1>(h, k, 1, nk, Ad, Dinv32);
+    }
 }
 
 template <class S>
@@ -700,15 +647,14 @@ static cudaError_t setup_typed(hm_ctx *h, S *A, S *Ad, S *W, S *DinvS, float2 *D
                   (int)h->near_t.size(), h->d_near_t, h->d_near_s, h->d_near_off, h->d_near, h->d_leaf_ptr, h->d_pos,
                   h->d_sptr, h->d_sidx, h->d_srow, h->d_M, h->d_coff, h->d_doff, A, Ad, h->d_err));
     if ((e = cudaGetLastError())) return e;
-    const size_t inv_smem = sizeof(double2) * (64 * 65 + 128);
-    const size_t panel_smem = sizeof(S) * (2 * 64 * 65);
-    if ((e = cudaFuncSetAttribute(k_pivot_inverse<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_smem)))
-        return e;
-    if ((e = cudaFuncSetAttribute(k_panel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem)))
+    if ((e = cudaFuncSetAttribute(k_panel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem<S>(64))))
         return e;
     if ((e = cudaFuncSetAttribute(k_update_grp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UPD_SMEM))) return e;
     int dev = 0, nsm = 0;
     if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev))) return e;
+    const int maxn = *std::max_element(P.size.begin(), P.size.end());
+    if ((e = cudaFuncSetAttribute(k_update64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(double2) * 2 * 64 * 64)))
+        return e;
     if (sizeof(S) == 8 && h->update_kind == 2) {
         if (!h->d_ucum) {   // tensor-core update tasks: per row a of S_k, 64-column pieces of W_k
             std::vector<int> uc(std::max<size_t>(P.sidx.size(), 1));
@@ -731,18 +677,13 @@ static cudaError_t setup_typed(hm_ctx *h, S *A, S *Ad, S *W, S *DinvS, float2 *D
     }
     for (int k = 0; k < P.nb; ++k) {
         int nk = P.size[k];
-        if (h->pivot_cl > 1) {
-            if ((e = pivot_cluster<S>(h, k, nk, Ad, Dinv32))) return e;
-        } else
-            HM_LAUNCH(h, K_PIVOT,
-                      k_pivot_inverse<S><<<1, 256, sizeof(double2) * (nk * (nk + 1) + 2 * nk), st>>>(
-                          k, h->d_size, h->d_doff, Ad, h->d_Dinv, Dinv32, h->d_err));
+        if ((e = pivot_step<S>(h, k, nk, Ad, Dinv32))) return e;
         int ns = P.sptr[k + 1] - P.sptr[k];
         if (ns > 0) {
             int Mk = P.M[k];
             HM_LAUNCH(h, K_PANEL,
-                      k_panel<S><<<(Mk + 63) / 64, 256, panel_smem, st>>>(k, h->d_size, h->d_M, h->d_coff, h->d_doff,
-                                                                          DinvS, A, W));
+                      k_panel<S><<<(Mk + PANEL_COLS<S> - 1) / PANEL_COLS<S>, 256, panel_smem<S>(nk), st>>>(
+                          k, h->d_size, h->d_M, h->d_coff, h->d_doff, DinvS, A, W));
             if (h->opts.compress_in_setup && (e = compress_step<S>(h, k, W))) return e;
             if constexpr (sizeof(S) == 8) {
                 if (h->update_kind == 2) {
@@ -761,9 +702,8 @@ static cudaError_t setup_typed(hm_ctx *h, S *A, S *Ad, S *W, S *DinvS, float2 *D
             } else {
                 long nt = (long)ns * (ns + 1) / 2;
                 HM_LAUNCH(h, K_UPDATE,
-                          k_update<S><<<(unsigned)nt, 256, 0, st>>>(k, ns, h->d_size, h->d_sptr, h->d_sidx,
-                                                                    h->d_srow, h->d_M, h->d_coff, h->d_doff, W, A,
-                                                                    Ad));
+                          k_update64<<<(unsigned)nt, UPD64_T, sizeof(double2) * 2 * maxn * nk, st>>>(
+                              k, ns, h->d_size, h->d_sptr, h->d_sidx, h->d_srow, h->d_M, h->d_coff, h->d_doff, W, A, Ad));
             }
         }
         if ((e = cudaGetLastError())) return e;
@@ -791,13 +731,8 @@ cudaError_t block_jacobi_setup(hm_ctx *h, int *bad_block)
                   (int)h->near_t.size(), h->d_near_t, h->d_near_s, h->d_near_off, h->d_near, h->d_leaf_ptr, h->d_pos,
                   h->d_sptr, h->d_sidx, h->d_srow, h->d_M, h->d_coff, h->d_doff, (double2 *)nullptr, h->d_Ad, h->d_err,
                   true));
-    const size_t inv_smem = sizeof(double2) * (64 * 65 + 128);
-    if ((e = cudaFuncSetAttribute(k_pivot_inverse<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)inv_smem)))
+    if ((e = pivot_launch<double2, 1>(h, 0, P.nb, *std::max_element(P.size.begin(), P.size.end()), h->d_Ad, nullptr)))
         return e;
-    HM_LAUNCH(h, K_PIVOT,
-              k_pivot_inverse<double2><<<P.nb, 256, inv_smem, st>>>(0, h->d_size, h->d_doff, h->d_Ad, h->d_Dinv,
-                                                                    nullptr, h->d_err));
     if ((e = cudaGetLastError())) return e;
     int herr = 0;
     if ((e = cudaMemcpyAsync(&herr, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, st))) return e;

@@ -414,7 +414,7 @@ def hm_set_update_schedule(h, kind=0):
 
 def hm_set_pivot_schedule(h, ctas=0):
     """CTAs per FP64 pivot inversion in precond_setup: 1, or a cluster of 2, 4 or 8 (bitwise
-    the same inverses); 0 = the default (8)."""
+    the same inverses); 0 = the default (2 or 4 by the block's size)."""
     h.check(load().hm_set_pivot_schedule(h.ptr, ctas), "hm_set_pivot_schedule")
 
 
