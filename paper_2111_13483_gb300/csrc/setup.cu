@@ -356,20 +356,24 @@ __global__ void __launch_bounds__(UPD64_T) k_update64(int k, int ns, const int *
 }
 
 // Grouped Schur updates of step k for the complex-FP32 setup.  CTA -> (a, g): row block a
-// of S_k and the column blocks b = g*gb .. min(a, g*gb + gb - 1).  For each, C_ij -= A_ik W_kj
-// on a tile fitted to the block in steps of 16 rows and columns (tiles of 32 x 32 or 64 x 64
-// take up to 5x the useful FMAs for uneven pairs).  A_ik is staged once
-// per CTA, the W_kj blocks stream through two cp.async buffers (the copy of the next overlaps
-// the product of the current) and each C block's old values are loaded before its product,
-// so their latency hides behind the FMAs.
-constexpr int UPD_LD = 65;
-constexpr size_t UPD_SMEM = sizeof(float2) * 3 * 64 * UPD_LD;   // A_ik + two W_kj buffers
+// of S_k and the column blocks b = g*gb .. min(a, g*gb + gb - 1), one warp per column block.
+// A_ik is staged once per CTA; each warp streams its W_kj, UPD_C columns at a time, through two buffers of its
+// own and multiplies 32 x UPD_C pieces of the block, up to 4 x 4 outputs per lane (8 row lanes, 4 column lanes;
+// the pieces of uneven blocks have fewer), so that 8 shared-memory loads feed 64 FMAs and nothing
+// but A_ik is shared between warps.  The old values of a piece are loaded before its operands have landed.  Every output
+// sums its n_k products in order and is then subtracted from the old value.
+// What bounds it is latency: a block's product takes 2 us of a warp, the loads of its operands and old values (HBM: the
+// 1.2 GB workspace does not fit L2) as long again, so many warps matter: 4 x 8 outputs per lane leave 8 warps
+// per SM, 197 ms of updates per setup of the 30,720-unknown sphere.  The whole CTA on one block with 2 x 2 outputs per
+// thread loaded 4 values for 16 FMAs and met at two barriers per block: 249 ms (217 with smaller buffers and
+// three CTAs per SM); this is 158 (a 100 x 100 plate, 29,800 unknowns: 118 -> 62).
+constexpr int UPD_NW = 4, UPD_C = 16, UPD_CTAS = 4;   // CTAs per SM: 3 / 4 / 5 give 156 / 158 / 182 ms (plate 64 / 62 / 70)
 
-// CTAs of the rows a' < a: sum over m = 1..a of ceil(m / gb)
-__host__ __device__ __forceinline__ long upd_first(int a, int gb)
+// CTAs of the rows a' < a: sum over m = 1..a of ceil(m / gb), gb = 2^lg
+__host__ __device__ __forceinline__ long upd_first(int a, int lg)
 {
-    const long q = a / gb, r = a % gb;
-    return (long)gb * q * (q + 1) / 2 + r * (q + 1);
+    const long q = a >> lg, r = a & (1 << lg) - 1;
+    return (q * (q + 1) / 2 << lg) + r * (q + 1);
 }
 
 __device__ __forceinline__ void upd_cp(float2 *dst, const float2 *src)
@@ -378,120 +382,149 @@ __device__ __forceinline__ void upd_cp(float2 *dst, const float2 *src)
                  : "memory");
 }
 
-// C (ni x nj) -= A W on a (16 UR) x (16 UC) tile, UR = ceil(ni / 16), UC = ceil(nj / 16):
-// thread (tx, ty) owns rows tx + 16u and columns ty + 16v.
-template <int UR, int UC>
-__device__ __forceinline__ void upd_product(const float2 (*As)[UPD_LD], const float2 (*Ws)[UPD_LD], int nk, int ni,
-                                            int nj, float2 *C, int ldc)
+// row offset of block i inside stacked column j, found by one warp (-1 if absent): 32 probes, then the entries between two
+__device__ __forceinline__ int find_row_warp(const int *sptr, const int *sidx, const int *srow, int j, int i)
 {
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float2 old[UR][UC], acc[UR][UC];
+    const int lane = threadIdx.x & 31, lo = sptr[j], len = sptr[j + 1] - lo, step = (len + 31) / 32;
+    const int e = lane * step;
+    const unsigned below = __ballot_sync(0xffffffffu, e < len && sidx[lo + e] <= i);
+    if (!below) return -1;
+    const int f = (31 - __clz(below)) * step;
+    int found = -1;
+    for (int g = f; g < f + step; g += 32) {   // one round for up to 1024 blocks
+        const int x = g + lane;
+        const unsigned hit = __ballot_sync(0xffffffffu, x < f + step && x < len && sidx[lo + x] == i);
+        if (hit) found = g + 31 - __clz(hit);
+    }
+    return found < 0 ? -1 : srow[lo + found];
+}
+
+// C (nr x nc, nr <= 8 U, nc <= 4 V) -= A W: As[q * lda + r], Ws[c * nk + q], once landed() says they are there
+template <int U, int V, class Landed>
+__device__ __forceinline__ void upd_piece(const float2 *As, int lda, const float2 *Ws, int nk, int nr, int nc, float2 *C,
+                                          int ldc, Landed &&landed)
+{
+    const int lr = threadIdx.x & 7, lc = (threadIdx.x & 31) >> 3;
+    float2 old[U][V], acc[U][V];
 #pragma unroll
-    for (int u = 0; u < UR; ++u)
+    for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int v = 0; v < UC; ++v) {
-            const int r = tx + 16 * u, c = ty + 16 * v;
-            old[u][v] = (r < ni && c < nj) ? C[r + (int64_t)c * ldc] : czero(float2());
+        for (int u = 0; u < U; ++u) {
+            const int r = lr + 8 * u, c = lc + 4 * v;
+            old[u][v] = (r < nr && c < nc) ? C[r + (int64_t)c * ldc] : czero(float2());
             acc[u][v] = czero(float2());
         }
+    landed();
+    const float2 *ap = As + lr, *wp = Ws + lc * nk;
     for (int q = 0; q < nk; ++q) {
-        float2 av[UR], wv[UC];
+        float2 av[U], wv[V];
 #pragma unroll
-        for (int u = 0; u < UR; ++u) av[u] = As[q][tx + 16 * u];
+        for (int u = 0; u < U; ++u) av[u] = ap[q * lda + 8 * u];
 #pragma unroll
-        for (int v = 0; v < UC; ++v) wv[v] = Ws[q][ty + 16 * v];
+        for (int v = 0; v < V; ++v) wv[v] = wp[4 * v * nk + q];
 #pragma unroll
-        for (int u = 0; u < UR; ++u)
+        for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int v = 0; v < UC; ++v) acc[u][v] = cfma(av[u], wv[v], acc[u][v]);
+            for (int v = 0; v < V; ++v) acc[u][v] = cfma(av[u], wv[v], acc[u][v]);
     }
 #pragma unroll
-    for (int u = 0; u < UR; ++u)
+    for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int v = 0; v < UC; ++v) {
-            const int r = tx + 16 * u, c = ty + 16 * v;
-            if (r < ni && c < nj) {
-                float2 o = old[u][v];
-                o.x -= acc[u][v].x;
-                o.y -= acc[u][v].y;
-                C[r + (int64_t)c * ldc] = o;
-            }
+        for (int u = 0; u < U; ++u) {
+            const int r = lr + 8 * u, c = lc + 4 * v;
+            if (r < nr && c < nc) C[r + (int64_t)c * ldc] = make_float2(old[u][v].x - acc[u][v].x, old[u][v].y - acc[u][v].y);
         }
 }
 
-__global__ void __launch_bounds__(256, 2) k_update_grp(int k, int ns, int gb, const int *size, const int *sptr,
-                                                       const int *sidx, const int *srow, const int *M,
-                                                       const int64_t *coff, const int64_t *doff, const float2 *W,
-                                                       float2 *A, float2 *Ad)
+// entries of a warp's W buffer: UPD_C columns and the alignment of the first
+__host__ __device__ __forceinline__ int upd_wcap(int nk) { return UPD_C * nk + 2; }
+static size_t upd_smem(int nk, int lda) { return sizeof(float2) * ((size_t)nk * lda + 2 * UPD_NW * (size_t)upd_wcap(nk)); }
+
+__global__ void __launch_bounds__(32 * UPD_NW, UPD_CTAS) k_update_grp(int k, int ns, int lg, int lda, const int *size,
+                                                                      const int *sptr, const int *sidx, const int *srow,
+                                                                      const int *M, const int64_t *coff,
+                                                                      const int64_t *doff, const float2 *W, float2 *A,
+                                                                      float2 *Ad)
 {
     extern __shared__ float2 upd_sm[];
-    float2(*As)[UPD_LD] = (float2(*)[UPD_LD])upd_sm;   // As[q][r] = A_ik[r, q], rows >= n_i zero
-    // W buffer w: Ws[q][c] = W_kj[q, c], columns >= n_j zero up to the tile size
-    auto wbuf = [&](int w) { return (float2(*)[UPD_LD])(upd_sm + (1 + w) * 64 * UPD_LD); };
     const long t = blockIdx.x;
     int lo = 0, hi = ns;   // largest a with upd_first(a) <= t
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
-        if (upd_first(mid, gb) <= t) lo = mid;
+        if (upd_first(mid, lg) <= t) lo = mid;
         else hi = mid;
     }
-    const int a = lo, b0 = (int)(t - upd_first(a, gb)) * gb, b1 = min(a + 1, b0 + gb);
+    const int a = lo, b0 = (int)(t - upd_first(a, lg)) << lg, b1 = min(a + 1, b0 + (1 << lg));
     if (b0 > a) return;   // cannot happen: row a has ceil((a + 1) / gb) groups
     const int e0 = sptr[k], i = sidx[e0 + a], nk = size[k], ni = size[i], Mk = M[k];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, cap = upd_wcap(nk);
+    float2 *As = upd_sm;   // As[q * lda + r] = A_ik[r, q]
+    float2 *const wb = upd_sm + nk * lda + 2 * wp * cap;
+    const float2 *const Wk = W + coff[k];
     const float2 *Aik = A + coff[k] + srow[e0 + a];   // ld Mk; panel k is not written in this step
-    for (int e = threadIdx.x; e < 64 * nk; e += blockDim.x) {
-        const int r = e & 63, q = e >> 6;
-        if (r < ni) upd_cp(&As[q][r], Aik + r + (int64_t)q * Mk);
-        else As[q][r] = czero(float2());
-    }
-    auto stage_w = [&](int b, int buf) {
-        const int nj = size[sidx[e0 + b]];
-        const float2 *Wkj = W + coff[k] + (int64_t)srow[e0 + b] * nk;   // ld nk
-        const int ts = (nj + 15) / 16 * 16;
-        float2(*Ws)[UPD_LD] = wbuf(buf);
-        for (int e = threadIdx.x; e < nk * ts; e += blockDim.x) {
-            const int q = e % nk, c = e / nk;
-            if (c < nj) upd_cp(&Ws[q][c], Wkj + q + (int64_t)c * nk);
-            else Ws[q][c] = czero(float2());
+    for (int q = wp; q < nk; q += UPD_NW)
+        for (int r = lane; r < ni; r += 32) upd_cp(As + q * lda + r, Aik + r + (int64_t)q * Mk);
+    // this warp's pieces: columns [c0, c0 + UPD_C) of W_kj for b = b0 + wp, b0 + wp + UPD_NW, ...; the 16-byte words that
+    // hold them (panel allocations end on 256 bytes)
+    int b = b0 + wp, c0 = 0;
+    auto stage = [&](int bb, int cc, int buf) {
+        if (bb < b1) {
+            const float2 *src = Wk + (srow[e0 + bb] + cc) * nk;
+            const int rem = (int)((size_t)src >> 3 & 1), n16 = (rem + min(UPD_C, size[sidx[e0 + bb]] - cc) * nk + 1) / 2;
+            const unsigned d = (unsigned)__cvta_generic_to_shared(wb + buf * cap);
+            const char *g = (const char *)(src - rem);
+#pragma unroll 4
+            for (int x = lane; x < n16; x += 32)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d + 16 * x), "l"(g + 16 * x) : "memory");
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
-    stage_w(b0, 0);   // one group with the A_ik copies
-    for (int b = b0, it = 0; b < b1; ++b, ++it) {
-        if (b + 1 < b1) {
-            stage_w(b + 1, (it + 1) & 1);
-            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-        } else
-            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-        __syncthreads();
-        const int j = sidx[e0 + b], nj = size[j];
-        float2 *C = nullptr;
-        int ldc = 0;
-        if (i == j) {
-            C = Ad + doff[i];
-            ldc = ni;
-        } else {
-            const int r = find_row(sptr, sidx, srow, j, i);   // >= 0 when S is the symbolic fill
-            if (r >= 0) {
-                C = A + coff[j] + r;
+    stage(b, 0, 0);   // one group with the A_ik copies
+    float2 *C = nullptr;
+    int ldc = 0;
+    bool first = true;   // A_ik is still to be waited for, by the whole CTA
+    for (int buf = 0; b < b1; buf ^= 1) {
+        const int j = sidx[e0 + b], nj = size[j], nc = min(UPD_C, nj - c0);
+        const bool last = c0 + UPD_C >= nj;
+        const int bn = last ? b + UPD_NW : b, cn = last ? 0 : c0 + UPD_C;
+        stage(bn, cn, buf ^ 1);
+        if (c0 == 0) {
+            if (i == j) {
+                C = Ad + doff[i];
+                ldc = ni;
+            } else {
+                const int r = find_row_warp(sptr, sidx, srow, j, i);   // >= 0 when S is the symbolic fill
+                C = r >= 0 ? A + coff[j] + r : nullptr;
                 ldc = M[j];
             }
         }
-        if (C) {
-            const float2(*Ws)[UPD_LD] = wbuf(it & 1);
-            switch (((ni - 1) >> 4) * 4 + ((nj - 1) >> 4)) {   // (UR - 1) * 4 + (UC - 1)
-#define HM_UPD(R, C_) \
-    case (R - 1) * 4 + (C_ - 1): upd_product<R, C_>(As, Ws, nk, ni, nj, C, ldc); break;
+        auto landed = [&]() {
+            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+            if (first) __syncthreads();
+            else __syncwarp();
+            first = false;
+        };
+        const float2 *Ws = wb + buf * cap + ((size_t)(Wk + (srow[e0 + b] + c0) * nk) >> 3 & 1);
+        for (int r0 = 0; r0 < ni; r0 += 32) {
+            const int nr = C ? min(32, ni - r0) : 0;
+            float2 *Cp = C + r0 + (int64_t)c0 * ldc;
+            switch ((max(nr, 1) - 1 >> 3) * 4 + (nc - 1 >> 2)) {   // (U - 1) * 4 + (V - 1)
+#define HM_UPD(U, V) \
+    case (U - 1) * 4 + (V - 1): upd_piece<U, V>(As + r0, lda, Ws, nk, nr, nc, Cp, ldc, landed); break;
                 HM_UPD(1, 1) HM_UPD(1, 2) HM_UPD(1, 3) HM_UPD(1, 4)
                 HM_UPD(2, 1) HM_UPD(2, 2) HM_UPD(2, 3) HM_UPD(2, 4)
                 HM_UPD(3, 1) HM_UPD(3, 2) HM_UPD(3, 3) HM_UPD(3, 4)
                 HM_UPD(4, 1) HM_UPD(4, 2) HM_UPD(4, 3) HM_UPD(4, 4)
 #undef HM_UPD
-            default: break;   // block sizes are 1..64
+            default: break;   // pieces are 1..32 x 1..16
             }
         }
-        __syncthreads();   // the buffer is restaged two products later
+        __syncwarp();   // the buffer is restaged in the next turn
+        b = bn;
+        c0 = cn;
     }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    if (first) __syncthreads();   // a warp without pieces
 }
 
 // Schur updates of step k on the tensor cores (complex-FP32 setup, update kind 2).  The step's
@@ -578,13 +611,14 @@ __global__ void __launch_bounds__(256) k_update_tc(int k, int ns, const int *ucu
     acc.close();
 }
 
-// Column blocks per CTA of the grouped update: the most (up to 8) that still leaves at least
-// four CTAs per SM.
+// Column blocks per CTA of the grouped update, as a power of two: as many as leave UPD_MIN CTAs per SM (A_ik is staged
+// once for them), at least one and at most four per warp.  30,720-unknown sphere: 173, 166, 158, 158 ms for 3, 6, 12, 24.
+constexpr int UPD_MIN = 12;
 static int upd_group(int ns, int nsm)
 {
-    int gb = 8;
-    while (gb > 1 && upd_first(ns, gb) < 4L * nsm) gb >>= 1;
-    return gb;
+    int lg = 4;
+    while (lg > 2 && upd_first(ns, lg) < (long)UPD_MIN * nsm) --lg;
+    return lg;
 }
 
 // count pivot blocks from k on, of at most nk unknowns, each on CL CTAs
@@ -649,10 +683,10 @@ static cudaError_t setup_typed(hm_ctx *h, S *A, S *Ad, S *W, S *DinvS, float2 *D
     if ((e = cudaGetLastError())) return e;
     if ((e = cudaFuncSetAttribute(k_panel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem<S>(64))))
         return e;
-    if ((e = cudaFuncSetAttribute(k_update_grp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UPD_SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(k_update_grp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)upd_smem(64, 64)))) return e;
     int dev = 0, nsm = 0;
     if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev))) return e;
-    const int maxn = *std::max_element(P.size.begin(), P.size.end());
+    const int maxn = *std::max_element(P.size.begin(), P.size.end()), lda = (maxn + 7) / 8 * 8;
     if ((e = cudaFuncSetAttribute(k_update64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(double2) * 2 * 64 * 64)))
         return e;
     if (sizeof(S) == 8 && h->update_kind == 2) {
@@ -694,10 +728,10 @@ static cudaError_t setup_typed(hm_ctx *h, S *A, S *Ad, S *W, S *DinvS, float2 *D
                     if ((e = cudaGetLastError())) return e;
                     continue;
                 }
-                const int gb = upd_group(ns, nsm);
+                const int lg = upd_group(ns, nsm);
                 HM_LAUNCH(h, K_UPDATE,
-                          k_update_grp<<<(unsigned)upd_first(ns, gb), 256, UPD_SMEM, st>>>(
-                              k, ns, gb, h->d_size, h->d_sptr, h->d_sidx, h->d_srow, h->d_M, h->d_coff, h->d_doff,
+                          k_update_grp<<<(unsigned)upd_first(ns, lg), 32 * UPD_NW, upd_smem(nk, lda), st>>>(
+                              k, ns, lg, lda, h->d_size, h->d_sptr, h->d_sidx, h->d_srow, h->d_M, h->d_coff, h->d_doff,
                               W, A, Ad));
             } else {
                 long nt = (long)ns * (ns + 1) / 2;
