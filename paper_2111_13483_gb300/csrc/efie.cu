@@ -35,7 +35,8 @@
 // Jacobi SVD of R_U R_V^T (in shared memory up to rank 64, in global scratch above), truncation
 // to the smallest rank whose singular-value tail is <= eps times the Frobenius norm; a block
 // whose truncated factors are not smaller than the block (r (m + n) >= m n) is filled densely.
-// Dense blocks are cut into tiles of at most 128 x 64 RWG functions, one CTA each.
+// Dense blocks are cut into tiles of at most 128 x 64 RWG functions; neighbours with the same rows share one of up to
+// 256 columns.  One kernel integrates the pairs of all tiles, one assembles their entries.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -56,7 +57,9 @@ constexpr int RC_SMALL = 64;   // ranks re-compressed with their work arrays in 
 constexpr int NT = 256;        // threads per CTA
 constexpr size_t CHUNK_BYTES = size_t(1) << 30;   // default device scratch per launch
 constexpr int NONE = 0x7fffffff;
-constexpr int FILL_TR = 128, FILL_TC = 64;   // largest dense tile (RWG rows x columns) of one CTA
+constexpr int FILL_TR = 128, FILL_TC = 64;   // tiles (RWG rows x columns) that a dense block is cut into
+constexpr int FILL_TC_MAX = 256;             // columns of a tile of several blocks
+constexpr int FILL_ITEM = NT;                // pairs, or entries, of one CTA (512 and 1024: the same times)
 
 __constant__ double c_qw[NQ];
 
@@ -104,6 +107,7 @@ struct V3 {
     double x, y, z;
 };
 __device__ __forceinline__ V3 ld3(const double *p) { return V3{p[0], p[1], p[2]}; }
+__device__ __forceinline__ V3 operator+(V3 a, V3 b) { return V3{a.x + b.x, a.y + b.y, a.z + b.z}; }
 __device__ __forceinline__ V3 operator-(V3 a, V3 b) { return V3{a.x - b.x, a.y - b.y, a.z - b.z}; }
 __device__ __forceinline__ V3 operator*(double s, V3 a) { return V3{s * a.x, s * a.y, s * a.z}; }
 __device__ __forceinline__ double dot(V3 a, V3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
@@ -114,6 +118,10 @@ __device__ __forceinline__ V3 cross(V3 a, V3 b)
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 csc(double s, double2 a) { return make_double2(s * a.x, s * a.y); }
 
+// ---------------------------------------------------------------------------------------
+// Integrals of the ACA.  On a regular mesh its pivot search meets moduli that are equal but for rounding, and which of
+// them wins decides the factors; so it keeps one fixed sequence of roundings, while the dense blocks below use the
+// cheaper one.
 // S0 = int_T 1/|r - r'| ds' and Sv = int_T (r' - rho)/|r - r'| ds' over the flat triangle P
 // (unit normal n), rho the projection of r on its plane.  Per edge a -> b with unit tangent l
 // and in-plane outward normal u = l x n, h = n.(r - P0): l+- = (b|a - rho).l,
@@ -211,13 +219,6 @@ __device__ void point_terms(const Mesh &M, int p, int q, int a, bool close, doub
     o[7] = cadd(o[7], csc(wa, dv));
 }
 
-__device__ void pair_values(const Mesh &M, int p, int q, double2 o[NPV])
-{
-    for (int v = 0; v < NPV; ++v) o[v] = make_double2(0.0, 0.0);
-    const bool close = close_pair(M, p, q);
-    for (int a = 0; a < NQ; ++a) point_terms(M, p, q, a, close, o);
-}
-
 // Z(m, n) of Eq. 7 from the pair values (point_terms summed over the test points) of
 // (T_s of m, T_t of n): pv(s, t, v) returns value v
 template <class PV> __device__ double2 assemble(const Mesh &M, int m, int n, PV pv)
@@ -249,34 +250,328 @@ template <class PV> __device__ double2 assemble(const Mesh &M, int m, int n, PV 
 }
 
 // ---------------------------------------------------------------------------------------
-// dense tiles: one CTA per tile x of B (at most FILL_TR x FILL_TC RWG functions), its pair
-// scratch at pairs + poff[x] (NPV x ntr x ntc, value-major), its entry (i, j) at
-// out[ooff[x] + i + j ld[x]] (a column-major piece of its block)
-__global__ void __launch_bounds__(NT, 2) k_efie_fill(Mesh M, Blocks B, int ntile, const int64_t *poff, double2 *pairs,
-                                                     const int64_t *ooff, const int *ld, double2 *out)
+// Integrals of the dense blocks
+constexpr int GEO = 6;   // per quadrature point x of a triangle with centroid c: k x and w (x - c), w the rule's weight
+constexpr int EDG = 10;  // per edge a -> b of a triangle: a, unit tangent l, in-plane outward normal l x n, length
+
+// Geometry of the dense blocks.  Moments and free vertices are relative to the triangle's centroid: about the origin the
+// four products of (r - v_m).(r' - v_n) cancel to the square of the edge length (3e-13 of a 7-wide plate's entries).
+struct Geometry {
+    double *tg;     // [nt][NQ][GEO]
+    double *tq;     // [nt][NQ][3] quadrature points
+    double *te;     // [nt][3][EDG]
+    double *tn;     // [nt][3] unit normal
+    double *ta;     // [nt] area
+    double *bfree;  // [nb][2][3] free vertex less the centroid of T+, T-
+    double *blen;   // [nb] edge length
+};
+
+// thread t takes triangle t and RWG function t; tc, th and btri of M are there
+__global__ void k_geometry(int nt, int nb, Mesh M, const double *V, const int *T, const int *fv, const double *bary,
+                           Geometry G)
 {
-    const int b = blockIdx.x;
-    if (b >= ntile) return;
-    const int m = (int)(B.rptr[b + 1] - B.rptr[b]), n = (int)(B.cptr[b + 1] - B.cptr[b]);
-    const int ntr = (int)(B.trptr[b + 1] - B.trptr[b]), ntc = (int)(B.tcptr[b + 1] - B.tcptr[b]);
-    const int *Tr = B.tridx + B.trptr[b], *Tc = B.tcidx + B.tcptr[b];
-    const int64_t P = (int64_t)ntr * ntc;
-    double2 *pb = pairs + poff[b];
-    for (int64_t i = threadIdx.x; i < P; i += blockDim.x) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    auto put = [](double *d, V3 v) { d[0] = v.x, d[1] = v.y, d[2] = v.z; };
+    if (t < nt) {
+        const V3 P[3] = {ld3(V + 3 * (size_t)T[3 * t]), ld3(V + 3 * (size_t)T[3 * t + 1]), ld3(V + 3 * (size_t)T[3 * t + 2])};
+        const V3 c = ld3(M.tc + 3 * (size_t)t), nn = cross(P[1] - P[0], P[2] - P[0]);
+        const double an = sqrt(dot(nn, nn));
+        const V3 n{nn.x / an, nn.y / an, nn.z / an};
+        G.ta[t] = 0.5 * an;
+        put(G.tn + 3 * (size_t)t, n);
+        for (int i = 0; i < 3; ++i) {
+            const V3 e = P[(i + 1) % 3] - P[i];
+            const double le = sqrt(dot(e, e));
+            const V3 l = (1.0 / le) * e;
+            double *E = G.te + ((size_t)t * 3 + i) * EDG;
+            put(E, P[i]);
+            put(E + 3, l);
+            put(E + 6, cross(l, n));
+            E[9] = le;
+        }
+        for (int a = 0; a < NQ; ++a) {
+            const double *b = bary + 3 * a;
+            const V3 x = b[0] * P[0] + b[1] * P[1] + b[2] * P[2];
+            put(G.tq + ((size_t)t * NQ + a) * 3, x);
+            put(G.tg + ((size_t)t * NQ + a) * GEO, M.k * x);
+            put(G.tg + ((size_t)t * NQ + a) * GEO + 3, c_qw[a] * (b[0] * (P[0] - c) + b[1] * (P[1] - c) + b[2] * (P[2] - c)));
+        }
+    }
+    if (t < nb) {
+        for (int s = 0; s < 2; ++s)
+            put(G.bfree + 6 * (size_t)t + 3 * s, ld3(V + 3 * (size_t)fv[2 * t + s]) - ld3(M.tc + 3 * (size_t)M.btri[2 * t + s]));
+        // the edge: the first two vertices of T+ other than its free vertex
+        const int *tt = T + 3 * (size_t)M.btri[2 * t];
+        V3 ev[2] = {V3{0, 0, 0}, V3{0, 0, 0}};
+        for (int i = 0, c = 0; i < 3; ++i)
+            if (tt[i] != fv[2 * t]) {
+                if (c == 0) ev[0] = ld3(V + 3 * (size_t)tt[i]);
+                if (c == 1) ev[1] = ld3(V + 3 * (size_t)tt[i]);
+                ++c;
+            }
+        const V3 e = ev[1] - ev[0];
+        G.blen[t] = sqrt(dot(e, e));
+    }
+}
+
+// S0 = int_T 1/|r - r'| ds' and Sv = int_T (r' - rho)/|r - r'| ds' over the flat triangle q
+// (unit normal n), rho the projection of r on its plane.  Per edge a -> b with unit tangent l
+// and in-plane outward normal u = l x n, h = n.(r - P0): l+- = (b|a - rho).l,
+// p0 = (a - rho).u, R0^2 = p0^2 + h^2, R+- = sqrt(l+-^2 + R0^2) the distances to the vertices,
+// f = log((R+ + l+)/(R- + l-)), each factor that cancels replaced by R0^2 over its conjugate:
+//   S0 = sum p0 f - |h| Omega,    Sv = sum u (R0^2 f + l+ R+ - l- R-) / 2,
+// Omega the solid angle of the triangle, tan(Omega / 2) = 2 A |h| / (R1 R2 R3 + R1 r2.r3 + R2 r3.r1 +
+// R3 r1.r2) (van Oosterom and Strackee, IEEE Trans. Biomed. Eng. 1983), one arctangent instead of the six
+// of the per-edge form.
+__device__ __forceinline__ void potential(const Geometry &G, int q, V3 r, double &S0, V3 &Sv, V3 &rho)
+{
+    const double *E = G.te + (size_t)q * 3 * EDG;
+    V3 d[3];
+    double R[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        d[i] = ld3(E + EDG * i) - r;
+        R[i] = sqrt(dot(d[i], d[i]));
+    }
+    const V3 n = ld3(G.tn + 3 * (size_t)q);
+    const double h = -dot(n, d[0]), ah = fabs(h), h2 = h * h;
+    rho = r - h * n;
+    S0 = 0.0;
+    Sv = V3{0.0, 0.0, 0.0};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const double *e = E + EDG * i;
+        const V3 l = ld3(e + 3), u = ld3(e + 6);
+        const double le = e[9];
+        const double lm = dot(d[i], l), lp = lm + le, p0 = dot(d[i], u);
+        const double R02 = p0 * p0 + h2, Rm = R[i], Rp = R[(i + 1) % 3];
+        const double sp = Rp + fabs(lp), sm = Rm + fabs(lm);   // l- <= l+
+        double num = sp, den = sm;
+        if (lp <= 0.0) {
+            num = sm;
+            den = sp;
+        } else if (lm < 0.0) {
+            num = sp * sm;
+            den = R02;
+        }
+        const double f = R02 > 1e-24 * le * le ? log(num / den) : 0.0;   // 0: rho is on the edge's line
+        S0 += p0 * f;
+        const double g = 0.5 * (R02 * f + lp * Rp - lm * Rm);
+        Sv = V3{Sv.x + g * u.x, Sv.y + g * u.y, Sv.z + g * u.z};
+    }
+    if (ah > 0.0) {
+        const double D = R[0] * (R[1] * R[2] + dot(d[1], d[2])) + R[1] * dot(d[2], d[0]) + R[2] * dot(d[0], d[1]);
+        S0 -= 2.0 * ah * atan2(2.0 * G.ta[q] * ah, D);
+    }
+}
+
+// sin x and off + cos x (off 0 or -1, the latter without cancellation) for x >= 0: reduction by multiples of pi/2 in
+// two parts (Cody and Waite), then the Taylor series on |r| <= pi/4, the terms from r^12 on (1e-10 of the sum) in
+// FP32: a warp's FP64 operation holds its scheduler for 64 cycles, so the 20 that are left are the price.
+__device__ __forceinline__ void sin_cos(double x, double off, double &sn, double &cs)
+{
+    if (!(x < 1e5)) {
+        sn = sin(x);
+        cs = cos(x) + off;
+        return;
+    }
+    const double magic = 6755399441055744.0;   // 1.5 2^52: its low bits are the rounded multiple
+    const double qm = fma(x, 0.63661977236758134308, magic);
+    const int qi = __double2loint(qm);
+    const double q = qm - magic;
+    const double r = fma(-q, 6.123233995736766036e-17, fma(-q, 1.5707963267948965580, x));
+    const double z = r * r;
+    const float zf = (float)z;
+    const double ts = (double)fmaf(zf, fmaf(zf, 2.8114573e-15f, -7.6471637e-13f), 1.6059044e-10f);   // 1/17!, 1/15!, 1/13!
+    const double tc = (double)fmaf(zf, fmaf(zf, 4.7794773e-14f, -1.1470746e-11f), 2.0876757e-9f);    // 1/16!, 1/14!, 1/12!
+    double ps = fma(z, ts, -1.0 / 39916800), pc = fma(z, tc, -1.0 / 3628800);
+    ps = fma(z, ps, 1.0 / 362880);
+    pc = fma(z, pc, 1.0 / 40320);
+    ps = fma(z, ps, -1.0 / 5040);
+    pc = fma(z, pc, -1.0 / 720);
+    ps = fma(z, ps, 1.0 / 120);
+    pc = fma(z, pc, 1.0 / 24);
+    ps = fma(z, ps, -1.0 / 6);
+    pc = fma(z, pc, -0.5);
+    const double s = fma(r * z, ps, r), m = z * pc;   // sin r, cos r - 1
+    // quadrants 0, 1, 2, 3: sin x = s, 1 + m, -s, -1 - m; cos x = 1 + m, -s, -1 - m, s
+    const bool odd = qi & 1;
+    sn = odd ? 1.0 + m : s;
+    if (qi & 2) sn = -sn;
+    const double a = odd ? s : m, sg = (qi + 1 & 2) ? -a : a;
+    cs = sg + (odd ? off : (qi & 2) ? off - 1.0 : off + 1.0);
+}
+
+// o[v] += the terms of one test point from the sums over the source (scaled by 1/k)
+__device__ __forceinline__ void add_point(double k, const double *ga, double wa, double2 s0, double2 sx, double2 sy,
+                                          double2 sz, double2 o[NPV])
+{
+    const double w = k * wa, x = k * ga[3], y = k * ga[4], z = k * ga[5];
+    auto add = [](double2 &d, double c, double2 v) { d = make_double2(fma(c, v.x, d.x), fma(c, v.y, d.y)); };
+    add(o[0], w, s0);
+    add(o[1], x, s0);
+    add(o[2], y, s0);
+    add(o[3], z, s0);
+    add(o[4], w, sx);
+    add(o[5], w, sy);
+    add(o[6], w, sz);
+    add(o[7], x, sx);
+    add(o[7], y, sy);
+    add(o[7], z, sz);
+}
+
+// Point a of test triangle p against the 7 points of source triangle q: o[v] += w_a times the integral over q, divided by
+// its area, of G, G r_a, G r', G r_a.r' (value order I0, Ir, Irp, Irr; r_a and r' from their centroids), G less 1/R on a
+// close pair.  The sum over a is the pair's integral divided by both areas.
+// FP64 arithmetic bounds it (2 operations a cycle and SM): with the points scaled by k the reciprocal root gives kR and
+// 1/kR at once, so a point pair takes 6 operations for its distance, the root, 22 for the phase and 8 for the sums: 1,700
+// a triangle pair, where the ACA's sequence (root, two divisions, the library's sine and cosine) takes 5,000.
+__device__ __forceinline__ void rule_terms(const Geometry &G, double k, int p, int q, int a, bool close, double2 o[NPV])
+{
+    const double *ga = G.tg + ((size_t)p * NQ + a) * GEO, *gb = G.tg + (size_t)q * NQ * GEO;
+    const V3 ra = ld3(ga);
+    const double off = close ? -1.0 : 0.0;
+    double2 s0 = make_double2(0.0, 0.0), sx = s0, sy = s0, sz = s0;
+    for (int b = 0; b < NQ; ++b, gb += GEO) {
+        const V3 d = ra - ld3(gb);
+        const double r2 = dot(d, d);
+        double2 g;
+        if (close && r2 < 1e-28 * k * k) {   // the limit of (e^{-jkR} - 1)/kR
+            g = make_double2(0.0, -1.0);
+        } else {
+            const double ri = rsqrt(r2);
+            double sn, cs;
+            sin_cos(r2 * ri, off, sn, cs);
+            g = make_double2(cs * ri, -sn * ri);
+        }
+        const V3 wr = ld3(gb + 3);
+        const double wb = c_qw[b];
+        s0 = make_double2(fma(wb, g.x, s0.x), fma(wb, g.y, s0.y));
+        sx = make_double2(fma(wr.x, g.x, sx.x), fma(wr.x, g.y, sx.y));
+        sy = make_double2(fma(wr.y, g.x, sy.x), fma(wr.y, g.y, sy.y));
+        sz = make_double2(fma(wr.z, g.x, sz.x), fma(wr.z, g.y, sz.y));
+    }
+    add_point(k, ga, c_qw[a], s0, sx, sy, sz, o);
+}
+
+// the 1/R part of a close pair in closed form, test point a, added to the same values
+__device__ __forceinline__ void close_terms(const Geometry &G, V3 cq, int p, int q, int a, double2 o[NPV])
+{
+    double S0;
+    V3 Sv, rho;
+    potential(G, q, ld3(G.tq + ((size_t)p * NQ + a) * 3), S0, Sv, rho);
+    const double *ga = G.tg + ((size_t)p * NQ + a) * GEO;
+    const double c = 1.0 / G.ta[q], wa = c_qw[a];
+    S0 *= c;
+    const V3 s = c * Sv + S0 * (rho - cq);
+    o[0].x = fma(wa, S0, o[0].x);
+    o[1].x = fma(ga[3], S0, o[1].x);
+    o[2].x = fma(ga[4], S0, o[2].x);
+    o[3].x = fma(ga[5], S0, o[3].x);
+    o[4].x = fma(wa, s.x, o[4].x);
+    o[5].x = fma(wa, s.y, o[5].x);
+    o[6].x = fma(wa, s.z, o[6].x);
+    o[7].x += dot(ld3(ga + 3), s);
+}
+
+// Z(m, n) of Eq. 7 from the pair values of (T_s of m, T_t of n): pv(s, t, v) returns value v
+template <class PV>
+__device__ __forceinline__ double2 entry(const Geometry &G, double k, double eta0, int m, int n, PV pv)
+{
+    double2 z = make_double2(0.0, 0.0);
+    const double ik2 = -4.0 / (k * k);
+    auto add = [](double2 &d, double c, double2 v) { d = make_double2(fma(c, v.x, d.x), fma(c, v.y, d.y)); };
+    for (int s = 0; s < 2; ++s) {
+        const V3 vm = ld3(G.bfree + 6 * (size_t)m + 3 * s);
+        for (int t = 0; t < 2; ++t) {
+            const V3 vn = ld3(G.bfree + 6 * (size_t)n + 3 * t);
+            double2 d = pv(s, t, 7);
+            add(d, -vn.x, pv(s, t, 1));
+            add(d, -vn.y, pv(s, t, 2));
+            add(d, -vn.z, pv(s, t, 3));
+            add(d, -vm.x, pv(s, t, 4));
+            add(d, -vm.y, pv(s, t, 5));
+            add(d, -vm.z, pv(s, t, 6));
+            add(d, dot(vm, vn) + ik2, pv(s, t, 0));
+            z = (s == t) ? cadd(z, d) : make_double2(z.x - d.x, z.y - d.y);
+        }
+    }
+    const double c = k * eta0 / (16.0 * M_PI) * G.blen[m] * G.blen[n];
+    return make_double2(-c * z.y, c * z.x);   // j c z
+}
+
+// ---------------------------------------------------------------------------------------
+// Dense tiles: tile x of B (at most FILL_TR x FILL_TC_MAX RWG functions), its pair scratch at pairs + poff[x] (NPV x ntr
+// x ntc, value-major), its entry (i, j) at out[ooff[x] + i + j ld[x]].  The pairs of all tiles, then their
+// entries, are dealt out in items of FILL_ITEM, one CTA each (cum[x] items before tile x): with a tile per CTA a quarter
+// of the time went into the last wave.
+struct Tiles {
+    const int64_t *poff, *ooff;
+    const int *ld, *pcum, *ecum;   // [ntile + 1]
+    int ntile;
+};
+__device__ __forceinline__ int find_tile(const int *cum, int ntile, int item)
+{
+    int lo = 0, hi = ntile;   // largest x with cum[x] <= item; every tile has at least one item
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (cum[mid] <= item) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// FP64 arithmetic bounds it (pipe 87% busy): near field of a 72 x 72 plate 50 ms for 9.0 M pairs, 106 before with 9.8 M.
+// All pairs of the item by the regular rule, the close ones noted; then the closed-form part, one close pair per
+// thread: it costs as much again, and only one pair in six needs it.
+__global__ void __launch_bounds__(NT, 2) k_fill_pairs(Mesh M, Geometry G, Blocks B, Tiles S, double2 *pairs)
+{
+    __shared__ int s_close[FILL_ITEM], s_n;
+    const int x = find_tile(S.pcum, S.ntile, blockIdx.x);
+    const int ntr = (int)(B.trptr[x + 1] - B.trptr[x]), ntc = (int)(B.tcptr[x + 1] - B.tcptr[x]);
+    const int *Tr = B.tridx + B.trptr[x], *Tc = B.tcidx + B.tcptr[x];
+    const int P = ntr * ntc;   // at most 2 FILL_TR x 2 FILL_TC_MAX
+    const int i = (int)(blockIdx.x - S.pcum[x]) * FILL_ITEM + threadIdx.x;
+    double2 *pb = pairs + S.poff[x];
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    if (i < P) {
+        const int p = Tr[i % ntr], q = Tc[i / ntr];
+        const bool close = close_pair(M, p, q);
         double2 o[NPV];
-        pair_values(M, Tr[i % ntr], Tc[i / ntr], o);
-        for (int v = 0; v < NPV; ++v) pb[v * P + i] = o[v];
+        for (int v = 0; v < NPV; ++v) o[v] = make_double2(0.0, 0.0);
+        for (int a = 0; a < NQ; ++a) rule_terms(G, M.k, p, q, a, close, o);
+        for (int v = 0; v < NPV; ++v) pb[(int64_t)v * P + i] = o[v];
+        if (close) s_close[atomicAdd(&s_n, 1)] = i;   // their order is without effect
     }
     __syncthreads();
-    const int *R = B.ridx + B.rptr[b], *C = B.cidx + B.cptr[b];
-    const int *rl = B.rloc + 2 * B.rptr[b], *cl = B.cloc + 2 * B.cptr[b];
-    double2 *ob = out + ooff[b];
-    const int64_t ldo = ld[b];
-    for (int64_t e = threadIdx.x; e < (int64_t)m * n; e += blockDim.x) {
-        const int i = (int)(e % m), j = (int)(e / m);
+    if (threadIdx.x < s_n) {
+        const int j = s_close[threadIdx.x], p = Tr[j % ntr], q = Tc[j / ntr];
+        const V3 cq = ld3(M.tc + 3 * (size_t)q);
+        double2 o[NPV];
+        for (int v = 0; v < NPV; ++v) o[v] = make_double2(0.0, 0.0);
+        for (int a = 0; a < NQ; ++a) close_terms(G, cq, p, q, a, o);
+        for (int v = 0; v < NPV; ++v) pb[(int64_t)v * P + j].x += o[v].x;
+    }
+}
+
+__global__ void __launch_bounds__(NT) k_fill_entries(Mesh M, Geometry G, Blocks B, Tiles S, const double2 *pairs,
+                                                     double2 *out)
+{
+    const int x = find_tile(S.ecum, S.ntile, blockIdx.x);
+    const int m = (int)(B.rptr[x + 1] - B.rptr[x]), n = (int)(B.cptr[x + 1] - B.cptr[x]);
+    const int ntr = (int)(B.trptr[x + 1] - B.trptr[x]), P = ntr * (int)(B.tcptr[x + 1] - B.tcptr[x]);
+    const int *R = B.ridx + B.rptr[x], *C = B.cidx + B.cptr[x];
+    const int *rl = B.rloc + 2 * B.rptr[x], *cl = B.cloc + 2 * B.cptr[x];
+    const double2 *pb = pairs + S.poff[x];
+    double2 *ob = out + S.ooff[x];
+    const int64_t ldo = S.ld[x];
+    const int e = (int)(blockIdx.x - S.ecum[x]) * FILL_ITEM + threadIdx.x;
+    if (e < m * n) {
+        const int i = e % m, j = e / m;
         const int r0 = rl[2 * i], r1 = rl[2 * i + 1], c0 = cl[2 * j], c1 = cl[2 * j + 1];
-        ob[i + j * ldo] = assemble(M, R[i], C[j], [&](int s, int t, int v) {
-            return pb[v * P + (int64_t)(s ? r1 : r0) + (int64_t)ntr * (t ? c1 : c0)];
+        ob[i + j * ldo] = entry(G, M.k, M.eta0, R[i], C[j], [&](int s, int t, int v) {
+            return pb[(int64_t)v * P + (s ? r1 : r0) + ntr * (t ? c1 : c0)];
         });
     }
 }
@@ -368,14 +663,16 @@ __device__ __forceinline__ int aca_cap(int m, int n)
     return min(min(min(m, n), (int)((int64_t)m * n / (m + n)) + 1), ACA_RCAP);
 }
 
-// partially pivoted ACA of block b0 + blockIdx.x (Eqs. 9-10): U (m x cap), V (n x cap)
-__global__ void __launch_bounds__(NT, 2) k_efie_aca(Mesh M, Blocks B, int b0, int nchunk, double eps, AcaWork W)
+// partially pivoted ACA of block order[blockIdx.x] (Eqs. 9-10): U (m x cap), V (n x cap).  FP64 arithmetic bounds it; the
+// blocks start in the order of falling size: in the order of the tree the last, large ones left half of the chip idle
+// (far field of a 48 x 48 plate with its re-compression 124 -> 109 ms).
+__global__ void __launch_bounds__(NT, 2) k_efie_aca(Mesh M, Blocks B, const int *order, int nchunk, double eps, AcaWork W)
 {
     __shared__ double s_red[NT / 32], s_v[NT / 32];
     __shared__ int s_i[NT / 32];
     __shared__ double2 s_c[ACA_RCAP];
-    const int lb = blockIdx.x, b = b0 + lb;
-    if (lb >= nchunk) return;
+    if (blockIdx.x >= nchunk) return;
+    const int b = order[blockIdx.x];
     const int m = (int)(B.rptr[b + 1] - B.rptr[b]), n = (int)(B.cptr[b + 1] - B.cptr[b]);
     const int ntr = (int)(B.trptr[b + 1] - B.trptr[b]), ntc = (int)(B.tcptr[b + 1] - B.tcptr[b]);
     const int *R = B.ridx + B.rptr[b], *C = B.cidx + B.cptr[b];
@@ -602,13 +899,13 @@ __device__ void recompress(int b, int r, int m, int n, double eps, AcaWork &W, d
     if (threadIdx.x == 0) W.rank[b] = rr;
 }
 
-// blocks b0 + blockIdx.x of rank 1 .. 64, with their work arrays in shared memory
-__global__ void __launch_bounds__(NT) k_aca_recompress(int b0, int nchunk, const int64_t *rptr, const int64_t *cptr,
+// blocks order[blockIdx.x] of rank 1 .. 64, with their work arrays in shared memory
+__global__ void __launch_bounds__(NT) k_aca_recompress(const int *order, int nchunk, const int64_t *rptr, const int64_t *cptr,
                                                         double eps, AcaWork W, double2 *Uo, double2 *Vo)
 {
     extern __shared__ unsigned char smraw[];
-    const int lb = blockIdx.x, b = b0 + lb;
-    if (lb >= nchunk) return;
+    if (blockIdx.x >= nchunk) return;
+    const int b = order[blockIdx.x];
     const int r = W.rank[b];
     // a zero block (rank 0), the cap reached (-1), or a rank for k_aca_recompress_big
     if (r <= 0 || r > RC_SMALL) return;
@@ -656,12 +953,6 @@ struct DevBufs {
         *d = (T *)x;
         return cudaSuccess;
     }
-    template <class T> cudaError_t up(T **d, const std::vector<T> &v)
-    {
-        cudaError_t e = alloc(d, v.size());
-        if (e || v.empty()) return e;
-        return cudaMemcpy(*d, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice);
-    }
     // grow-only scratch
     template <class T> cudaError_t grow(T **d, size_t *have, size_t need)
     {
@@ -678,15 +969,34 @@ struct DevBufs {
     }
 };
 
-struct Ctx {
-    DevBufs mem;
-    Mesh M{};
-    Blocks B{};   // the call's blocks on the device (the ACA works on them)
-    int nblk = 0, nt = 0;
-    const int32_t *tri = nullptr;                   // host, the caller's (valid during the call)
-    std::vector<int64_t> rptr, cptr, trptr, tcptr;  // host copies
-    std::vector<int> ridx, cidx;
-    std::vector<unsigned char> sym;                 // per block: mirror the upper triangle
+// Host arrays that go to the device in one allocation and one copy: a small call is mostly such copies (8 us each).
+struct Pack {
+    struct Item {
+        void *dst;   // address of the device pointer
+        const void *src;
+        size_t bytes, off;
+    };
+    std::vector<Item> items;
+    size_t total = 0;
+    template <class T> void add(const T **dst, const T *src, size_t count)   // src stays valid until send
+    {
+        items.push_back(Item{(void *)dst, src, sizeof(T) * count, total});
+        total += (sizeof(T) * count + 255) & ~size_t(255);
+    }
+    template <class T> void add(const T **dst, const std::vector<T> &v) { add(dst, v.data(), v.size()); }
+    cudaError_t send(DevBufs &mem)
+    {
+        std::vector<char> h(total);
+        char *d = nullptr;
+        cudaError_t e = mem.alloc(&d, total);
+        if (e) return e;
+        for (const Item &x : items) {
+            if (x.bytes) std::memcpy(h.data() + x.off, x.src, x.bytes);
+            char *p = d + x.off;
+            std::memcpy(x.dst, &p, sizeof(p));
+        }
+        return total ? cudaMemcpy(d, h.data(), total, cudaMemcpyHostToDevice) : cudaSuccess;
+    }
 };
 
 int check_mesh(int nv, const double *V, int nt, const int32_t *T, int nb, const int32_t *tri, const int32_t *fv,
@@ -740,34 +1050,42 @@ void side_lists(int nt, int nblk, const int64_t *ptr, const int32_t *idx, const 
     }
 }
 
-template <class T> cudaError_t upload(DevBufs &mem, const T **dst, const std::vector<T> &v)
-{
-    T *d = nullptr;
-    cudaError_t e = mem.up(&d, v);
-    *dst = d;
-    return e;
-}
-
-// a set of blocks (RWG row and column lists) on the device with their distinct triangles
-cudaError_t upload_blocks(DevBufs &mem, int nt, const int32_t *tri, const std::vector<int64_t> &rptr,
-                          const std::vector<int> &ridx, const std::vector<int64_t> &cptr,
-                          const std::vector<int> &cidx, Blocks &B, std::vector<int64_t> &trptr,
-                          std::vector<int64_t> &tcptr)
-{
-    const int nblk = (int)rptr.size() - 1;
+// a set of blocks (RWG row and column lists) with their distinct triangles
+struct BlockLists {
     std::vector<int> tridx, tcidx, rloc, cloc;
-    side_lists(nt, nblk, rptr.data(), ridx.data(), tri, trptr, tridx, rloc);
-    side_lists(nt, nblk, cptr.data(), cidx.data(), tri, tcptr, tcidx, cloc);
-    cudaError_t e;
-    if ((e = upload(mem, &B.rptr, rptr)) || (e = upload(mem, &B.cptr, cptr)) || (e = upload(mem, &B.trptr, trptr)) ||
-        (e = upload(mem, &B.tcptr, tcptr)) || (e = upload(mem, &B.ridx, ridx)) || (e = upload(mem, &B.cidx, cidx)) ||
-        (e = upload(mem, &B.tridx, tridx)) || (e = upload(mem, &B.tcidx, tcidx)) || (e = upload(mem, &B.rloc, rloc)) ||
-        (e = upload(mem, &B.cloc, cloc)))
-        return e;
-    return cudaSuccess;
-}
+    void build(int nt, const int32_t *tri, const std::vector<int64_t> &rptr, const std::vector<int> &ridx,
+               const std::vector<int64_t> &cptr, const std::vector<int> &cidx, std::vector<int64_t> &trptr,
+               std::vector<int64_t> &tcptr)
+    {
+        const int nblk = (int)rptr.size() - 1;
+        side_lists(nt, nblk, rptr.data(), ridx.data(), tri, trptr, tridx, rloc);
+        side_lists(nt, nblk, cptr.data(), cidx.data(), tri, tcptr, tcidx, cloc);
+    }
+    void pack(Pack &K, Blocks &B, const std::vector<int64_t> &rptr, const std::vector<int> &ridx,
+              const std::vector<int64_t> &cptr, const std::vector<int> &cidx, const std::vector<int64_t> &trptr,
+              const std::vector<int64_t> &tcptr) const
+    {
+        K.add(&B.rptr, rptr), K.add(&B.cptr, cptr), K.add(&B.trptr, trptr), K.add(&B.tcptr, tcptr);
+        K.add(&B.ridx, ridx), K.add(&B.cidx, cidx), K.add(&B.tridx, tridx), K.add(&B.tcidx, tcidx);
+        K.add(&B.rloc, rloc), K.add(&B.cloc, cloc);
+    }
+};
 
-cudaError_t ctx_init(Ctx &X, const double *V, int nt, const int32_t *T, int nb, const int32_t *tri,
+struct Ctx {
+    DevBufs mem;
+    Mesh M{};
+    Blocks B{};   // the call's blocks on the device (the ACA works on them)
+    BlockLists lists;
+    int nblk = 0, nt = 0;
+    int nv = 0, nb = 0;
+    const double *V = nullptr;                      // host, the caller's (valid during the call)
+    const int32_t *T = nullptr, *tri = nullptr, *fv = nullptr;
+    std::vector<int64_t> rptr, cptr, trptr, tcptr;  // host copies
+    std::vector<int> ridx, cidx;
+    std::vector<unsigned char> sym;                 // per block: mirror the upper triangle
+};
+
+cudaError_t ctx_init(Ctx &X, int nv, const double *V, int nt, const int32_t *T, int nb, const int32_t *tri,
                      const int32_t *fv, double k, double eta0, double r_abs, double c_rel, int nblk,
                      const int64_t *rptr, const int32_t *ridx, const int64_t *cptr, const int32_t *cidx,
                      bool mirror)
@@ -776,32 +1094,69 @@ cudaError_t ctx_init(Ctx &X, const double *V, int nt, const int32_t *T, int nb, 
     radon_rule(w, bq);
     cudaError_t e;
     if ((e = cudaMemcpyToSymbol(c_qw, w, sizeof(w)))) return e;
-    std::vector<double> tv(9 * (size_t)nt), tn(3 * (size_t)nt), ta(nt), tc(3 * (size_t)nt), th(nt),
-        tq(3 * NQ * (size_t)nt), bfree(6 * (size_t)nb), blen(nb);
+    Mesh &M = X.M;
+    M.k = k;
+    M.eta0 = eta0;
+    M.r_abs = r_abs;
+    M.c_rel = c_rel;
+    // what decides which pairs are close, for both kinds of block
+    std::vector<double> tc(3 * (size_t)nt), th(nt);
+    for (int t = 0; t < nt; ++t) {
+        const double *P[3] = {V + 3 * (size_t)T[3 * t], V + 3 * (size_t)T[3 * t + 1], V + 3 * (size_t)T[3 * t + 2]};
+        double e1[3], e2[3], e3[3];
+        for (int j = 0; j < 3; ++j) e1[j] = P[1][j] - P[0][j], e2[j] = P[2][j] - P[0][j], e3[j] = P[2][j] - P[1][j];
+        auto len = [](const double *x) { return std::sqrt(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]); };
+        th[t] = std::max(len(e1), std::max(len(e2), len(e3)));
+        for (int j = 0; j < 3; ++j) tc[3 * t + j] = (P[0][j] + P[1][j] + P[2][j]) / 3.0;
+    }
+    Pack K;
+    K.add(&M.tc, tc), K.add(&M.th, th), K.add(&M.btri, tri, 2 * (size_t)nb);
+    if ((e = K.send(X.mem))) return e;
+    X.nv = nv;
+    X.nb = nb;
+    X.V = V;
+    X.T = T;
+    X.fv = fv;
+    X.nblk = nblk;
+    X.nt = nt;
+    X.tri = tri;
+    X.rptr.assign(rptr, rptr + nblk + 1);
+    X.cptr.assign(cptr, cptr + nblk + 1);
+    X.ridx.assign(ridx, ridx + rptr[nblk]);
+    X.cidx.assign(cidx, cidx + cptr[nblk]);
+    X.sym.assign(nblk, 0);
+    for (int b = 0; b < nblk && mirror; ++b)
+        X.sym[b] = rptr[b + 1] - rptr[b] == cptr[b + 1] - cptr[b] &&
+                   std::equal(ridx + rptr[b], ridx + rptr[b + 1], cidx + cptr[b]);
+    X.lists.build(nt, tri, X.rptr, X.ridx, X.cptr, X.cidx, X.trptr, X.tcptr);
+    return cudaSuccess;
+}
+
+// the tables and the blocks that the ACA reads
+cudaError_t aca_tables(Ctx &X)
+{
+    const int nt = X.nt, nb = X.nb;
+    const double *V = X.V;
+    const int32_t *T = X.T, *tri = X.tri, *fv = X.fv;
+    double w[NQ], bq[NQ][3];
+    radon_rule(w, bq);
+    std::vector<double> tv(9 * (size_t)nt), tn(3 * (size_t)nt), ta(nt), tq(3 * NQ * (size_t)nt), bfree(6 * (size_t)nb), blen(nb);
     for (int t = 0; t < nt; ++t) {
         double *P = &tv[9 * (size_t)t];
         for (int i = 0; i < 3; ++i)
             for (int j = 0; j < 3; ++j) P[3 * i + j] = V[3 * T[3 * t + i] + j];
-        double e1[3], e2[3], e3[3];
-        for (int j = 0; j < 3; ++j) e1[j] = P[3 + j] - P[j], e2[j] = P[6 + j] - P[j], e3[j] = P[6 + j] - P[3 + j];
+        double e1[3], e2[3];
+        for (int j = 0; j < 3; ++j) e1[j] = P[3 + j] - P[j], e2[j] = P[6 + j] - P[j];
         const double nn[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2],
                               e1[0] * e2[1] - e1[1] * e2[0]};
         const double an = std::sqrt(nn[0] * nn[0] + nn[1] * nn[1] + nn[2] * nn[2]);
-        auto len = [](const double *x) { return std::sqrt(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]); };
         ta[t] = 0.5 * an;
-        th[t] = std::max(len(e1), std::max(len(e2), len(e3)));
-        for (int j = 0; j < 3; ++j) {
-            tn[3 * t + j] = nn[j] / an;
-            tc[3 * t + j] = (P[j] + P[3 + j] + P[6 + j]) / 3.0;
-        }
+        for (int j = 0; j < 3; ++j) tn[3 * t + j] = nn[j] / an;
         for (int q = 0; q < NQ; ++q)
             for (int j = 0; j < 3; ++j)
                 tq[(t * NQ + q) * 3 + j] = bq[q][0] * P[j] + bq[q][1] * P[3 + j] + bq[q][2] * P[6 + j];
     }
-    std::vector<int> btri(2 * (size_t)nb);
     for (int n = 0; n < nb; ++n) {
-        btri[2 * n] = tri[2 * n];
-        btri[2 * n + 1] = tri[2 * n + 1];
         for (int s = 0; s < 2; ++s)
             for (int j = 0; j < 3; ++j) bfree[6 * n + 3 * s + j] = V[3 * fv[2 * n + s] + j];
         // the edge: the two vertices of T+ other than its free vertex
@@ -818,38 +1173,55 @@ cudaError_t ctx_init(Ctx &X, const double *V, int nt, const int32_t *T, int nb, 
         blen[n] = std::sqrt(d2);
     }
     Mesh &M = X.M;
-    M.k = k;
-    M.eta0 = eta0;
-    M.r_abs = r_abs;
-    M.c_rel = c_rel;
-    if ((e = upload(X.mem, &M.tv, tv)) || (e = upload(X.mem, &M.tn, tn)) || (e = upload(X.mem, &M.ta, ta)) ||
-        (e = upload(X.mem, &M.tc, tc)) || (e = upload(X.mem, &M.th, th)) || (e = upload(X.mem, &M.tq, tq)) ||
-        (e = upload(X.mem, &M.bfree, bfree)) || (e = upload(X.mem, &M.blen, blen)) ||
-        (e = upload(X.mem, &M.btri, btri)))
-        return e;
-    X.nblk = nblk;
-    X.nt = nt;
-    X.tri = tri;
-    X.rptr.assign(rptr, rptr + nblk + 1);
-    X.cptr.assign(cptr, cptr + nblk + 1);
-    X.ridx.assign(ridx, ridx + rptr[nblk]);
-    X.cidx.assign(cidx, cidx + cptr[nblk]);
-    X.sym.assign(nblk, 0);
-    for (int b = 0; b < nblk && mirror; ++b)
-        X.sym[b] = rptr[b + 1] - rptr[b] == cptr[b + 1] - cptr[b] &&
-                   std::equal(ridx + rptr[b], ridx + rptr[b + 1], cidx + cptr[b]);
-    return upload_blocks(X.mem, nt, tri, X.rptr, X.ridx, X.cptr, X.cidx, X.B, X.trptr, X.tcptr);
+    Pack K;
+    K.add(&M.tv, tv), K.add(&M.tn, tn), K.add(&M.ta, ta), K.add(&M.tq, tq), K.add(&M.bfree, bfree), K.add(&M.blen, blen);
+    X.lists.pack(K, X.B, X.rptr, X.ridx, X.cptr, X.cidx, X.trptr, X.tcptr);
+    return K.send(X.mem);
 }
 
-// dense blocks `list` of X into host memory, block list[x] at host + hoff[x].  A block is
-// cut into tiles of at most FILL_TR x FILL_TC RWG functions (one CTA each), so that a large
-// block is spread over the SMs; the tiles of a chunk of blocks get their own triangle lists.
+// the tables that the dense blocks read
+cudaError_t fill_tables(Ctx &X, Geometry &G)
+{
+    const size_t nt = X.nt, nb = X.nb;
+    double w[NQ], bq[NQ][3];
+    radon_rule(w, bq);
+    const double *d_V, *d_b;
+    const int *d_T, *d_fv;
+    Pack K;
+    K.add(&d_V, X.V, 3 * (size_t)X.nv), K.add(&d_T, X.T, 3 * nt), K.add(&d_fv, X.fv, 2 * nb), K.add(&d_b, &bq[0][0], 3 * NQ);
+    double *g;
+    cudaError_t e;
+    if ((e = K.send(X.mem)) ||
+        (e = X.mem.alloc(&g, (GEO * NQ + 3 * NQ + 3 * EDG + 4) * nt + 7 * nb)))
+        return e;
+    G.tg = g;
+    G.tq = G.tg + GEO * NQ * nt;
+    G.te = G.tq + 3 * NQ * nt;
+    G.tn = G.te + 3 * EDG * nt;
+    G.ta = G.tn + 3 * nt;
+    G.bfree = G.ta + nt;
+    G.blen = G.bfree + 6 * nb;
+    k_geometry<<<(unsigned)(std::max(nt, nb) + 63) / 64, 64>>>(X.nt, X.nb, X.M, d_V, d_T, d_fv, d_b, G);
+    return cudaGetLastError();
+}
+
+bool same_rows(const Ctx &X, int a, int b)
+{
+    return X.rptr[a + 1] - X.rptr[a] == X.rptr[b + 1] - X.rptr[b] &&
+           std::equal(X.ridx.begin() + X.rptr[a], X.ridx.begin() + X.rptr[a + 1], X.ridx.begin() + X.rptr[b]);
+}
+
+// dense blocks `list` of X into host memory, block list[x] at host + hoff[x].  A block of more than FILL_TR x FILL_TC RWG
+// functions is cut into tiles, smaller ones with the same rows share a tile; the tiles of a chunk of blocks
+// get their own triangle lists.
 cudaError_t fill_dense(Ctx &X, const std::vector<int> &list, const std::vector<int64_t> &hoff, hm_c128 *host,
                        size_t chunk_bytes)
 {
     cudaError_t e;
     double2 *d_pairs = nullptr, *d_out = nullptr;
     size_t h_pairs = 0, h_out = 0;
+    Geometry G{};
+    if ((e = fill_tables(X, G))) return e;
     size_t x0 = 0;
     while (x0 < list.size()) {
         std::vector<int64_t> trp(1, 0), tcp(1, 0), ooff, pofs, soff;
@@ -868,16 +1240,24 @@ cudaError_t fill_dense(Ctx &X, const std::vector<int> &list, const std::vector<i
                 soff.push_back(out_len);
                 sm.push_back((int)m);
             }
-            for (int64_t c0 = 0; c0 < n; c0 += FILL_TC)
-                for (int64_t r0 = 0; r0 < m; r0 += FILL_TR) {
-                    const int64_t r1 = std::min(m, r0 + FILL_TR), c1 = std::min(n, c0 + FILL_TC);
-                    tr.insert(tr.end(), R + r0, R + r1);
-                    tc.insert(tc.end(), C + c0, C + c1);
-                    trp.push_back((int64_t)tr.size());
-                    tcp.push_back((int64_t)tc.size());
-                    ooff.push_back(out_len + r0 + c0 * m);
-                    lds.push_back((int)m);
-                }
+            // a block with the rows of the one before it: its column triangles are largely the same, too
+            const bool join = x1 > x0 && m <= FILL_TR && (int64_t)tc.size() - tcp[tcp.size() - 2] + n <= FILL_TC_MAX &&
+                              same_rows(X, list[x1 - 1], b);
+            if (join) {   // the block is the next columns of the last tile
+                tc.insert(tc.end(), C, C + n);
+                tcp.back() = (int64_t)tc.size();
+            } else {
+                for (int64_t c0 = 0; c0 < n; c0 += FILL_TC)
+                    for (int64_t r0 = 0; r0 < m; r0 += FILL_TR) {
+                        const int64_t r1 = std::min(m, r0 + FILL_TR), c1 = std::min(n, c0 + FILL_TC);
+                        tr.insert(tr.end(), R + r0, R + r1);
+                        tc.insert(tc.end(), C + c0, C + c1);
+                        trp.push_back((int64_t)tr.size());
+                        tcp.push_back((int64_t)tc.size());
+                        ooff.push_back(out_len + r0 + c0 * m);
+                        lds.push_back((int)m);
+                    }
+            }
             pofs.push_back(out_len);
             out_len += m * n;
             bytes += nbytes;
@@ -886,17 +1266,30 @@ cudaError_t fill_dense(Ctx &X, const std::vector<int> &list, const std::vector<i
         DevBufs tmem;   // the chunk's tiles
         Blocks TB{};
         std::vector<int64_t> ttrp, ttcp;
-        if ((e = upload_blocks(tmem, X.nt, X.tri, trp, tr, tcp, tc, TB, ttrp, ttcp))) return e;
+        BlockLists TL;
+        TL.build(X.nt, X.tri, trp, tr, tcp, tc, ttrp, ttcp);
         const int ntile = (int)ooff.size();
         std::vector<int64_t> po(ntile + 1, 0);
         for (int t = 0; t < ntile; ++t) po[t + 1] = po[t] + NPV * (ttrp[t + 1] - ttrp[t]) * (ttcp[t + 1] - ttcp[t]);
-        const int64_t *d_po, *d_oo, *d_so;
-        const int *d_ld, *d_sm;
-        if ((e = X.mem.grow(&d_pairs, &h_pairs, (size_t)po.back())) || (e = X.mem.grow(&d_out, &h_out, (size_t)out_len)) ||
-            (e = upload(tmem, &d_po, po)) || (e = upload(tmem, &d_oo, ooff)) || (e = upload(tmem, &d_ld, lds)) ||
-            (e = upload(tmem, &d_so, soff)) || (e = upload(tmem, &d_sm, sm)))
+        Tiles S{};
+        S.ntile = ntile;
+        std::vector<int> pc(ntile + 1, 0), ec(ntile + 1, 0);
+        for (int t = 0; t < ntile; ++t) {
+            const int64_t np = (po[t + 1] - po[t]) / NPV, ne = (trp[t + 1] - trp[t]) * (tcp[t + 1] - tcp[t]);
+            pc[t + 1] = pc[t] + (int)((np + FILL_ITEM - 1) / FILL_ITEM);
+            ec[t + 1] = ec[t] + (int)((ne + FILL_ITEM - 1) / FILL_ITEM);
+        }
+        const int64_t *d_so;
+        const int *d_sm;
+        Pack K;
+        TL.pack(K, TB, trp, tr, tcp, tc, ttrp, ttcp);
+        K.add(&S.poff, po), K.add(&S.ooff, ooff), K.add(&S.ld, lds), K.add(&S.pcum, pc), K.add(&S.ecum, ec);
+        K.add(&d_so, soff), K.add(&d_sm, sm);
+        if ((e = X.mem.grow(&d_pairs, &h_pairs, (size_t)po.back())) ||
+            (e = X.mem.grow(&d_out, &h_out, (size_t)out_len)) || (e = K.send(tmem)))
             return e;
-        k_efie_fill<<<ntile, NT>>>(X.M, TB, ntile, d_po, d_pairs, d_oo, d_ld, d_out);
+        k_fill_pairs<<<(unsigned)pc.back(), NT>>>(X.M, G, TB, S, d_pairs);
+        k_fill_entries<<<(unsigned)ec.back(), NT>>>(X.M, G, TB, S, d_pairs, d_out);
         if (!soff.empty()) k_mirror<<<(unsigned)soff.size(), NT>>>((int)soff.size(), d_so, d_sm, d_out);
         if ((e = cudaGetLastError()) || (e = cudaDeviceSynchronize())) return e;
         // copy out, one copy per run of blocks adjacent in the host layout
@@ -949,7 +1342,7 @@ extern "C" int hm_efie_fill(int32_t nv, const double *V, int32_t nt, const int32
     cudaError_t e;
     if ((e = cudaSetDevice(device))) return status(e, "hm_efie_fill");
     Ctx X;
-    if ((e = ctx_init(X, V, nt, T, nb, tri, free_v, k, eta0, r_abs, c_rel, nblk, rptr, ridx, cptr, cidx,
+    if ((e = ctx_init(X, nv, V, nt, T, nb, tri, free_v, k, eta0, r_abs, c_rel, nblk, rptr, ridx, cptr, cidx,
                       mirror != 0)))
         return status(e, "hm_efie_fill");
     std::vector<int> list(nblk);
@@ -975,8 +1368,9 @@ extern "C" int hm_efie_far(int32_t nv, const double *V, int32_t nt, const int32_
     cudaError_t e;
     if ((e = cudaSetDevice(device))) return status(e, "hm_efie_far");
     Ctx X;
-    if ((e = ctx_init(X, V, nt, T, nb, tri, free_v, k, eta0, r_abs, c_rel, nblk, rptr, ridx, cptr, cidx, false)))
+    if ((e = ctx_init(X, nv, V, nt, T, nb, tri, free_v, k, eta0, r_abs, c_rel, nblk, rptr, ridx, cptr, cidx, false)))
         return status(e, "hm_efie_far");
+    if ((e = aca_tables(X))) return status(e, "hm_efie_far");
     const size_t smem = sizeof(double2) * 2 * RC_SMALL * RC_SMALL;
     if ((e = cudaFuncSetAttribute(k_aca_recompress, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
         return status(e, "hm_efie_far");
@@ -1007,10 +1401,19 @@ extern "C" int hm_efie_far(int32_t nv, const double *V, int32_t nt, const int32_
         chunk.push_back(nblk);
         cneed_p.push_back(sp), cneed_u.push_back(su), cneed_v.push_back(sv), cneed_f.push_back(sf);
     }
+    // the blocks of a chunk by falling size (their triangles): the last wave then holds the small ones
+    std::vector<int> order(nblk);
+    for (int b = 0; b < nblk; ++b) order[b] = b;
+    for (size_t ci = 0; ci + 1 < chunk.size(); ++ci)
+        std::stable_sort(order.begin() + chunk[ci], order.begin() + chunk[ci + 1], [&](int a, int b) {
+            return X.trptr[a + 1] - X.trptr[a] + X.tcptr[a + 1] - X.tcptr[a] >
+                   X.trptr[b + 1] - X.trptr[b] + X.tcptr[b + 1] - X.tcptr[b];
+        });
+    const int *d_order;
     AcaWork W{};
-    if ((e = upload(X.mem, &W.poff, wp)) || (e = upload(X.mem, &W.uoff, wu)) || (e = upload(X.mem, &W.voff, wv)) ||
-        (e = upload(X.mem, &W.foff, wf)) || (e = X.mem.alloc(&W.rank, nblk)))
-        return status(e, "hm_efie_far");
+    Pack K;
+    K.add(&d_order, order), K.add(&W.poff, wp), K.add(&W.uoff, wu), K.add(&W.voff, wv), K.add(&W.foff, wf);
+    if ((e = K.send(X.mem)) || (e = X.mem.alloc(&W.rank, nblk))) return status(e, "hm_efie_far");
     double2 *Uo = nullptr, *Vo = nullptr, *d_cu = nullptr, *d_cv = nullptr, *d_big = nullptr;
     int64_t *d_so = nullptr, *d_do = nullptr, *d_len = nullptr;
     int *d_blist = nullptr;
@@ -1026,14 +1429,14 @@ extern "C" int hm_efie_far(int32_t nv, const double *V, int32_t nt, const int32_
             (e = X.mem.grow(&W.V, &hv, cneed_v[ci])) || (e = X.mem.grow(&W.flags, &hf, cneed_f[ci])) ||
             (e = X.mem.grow(&Uo, &huo, cneed_u[ci])) || (e = X.mem.grow(&Vo, &hvo, cneed_v[ci])))
             return status(e, "hm_efie_far");
-        k_efie_aca<<<nc, NT>>>(X.M, X.B, b0, nc, eps, W);
+        k_efie_aca<<<nc, NT>>>(X.M, X.B, d_order + b0, nc, eps, W);
         if ((e = cudaGetLastError()) || (e = cudaDeviceSynchronize()) ||
             (e = cudaMemcpy(rank + b0, W.rank + b0, sizeof(int) * nc, cudaMemcpyDeviceToHost)))
             return status(e, "hm_efie_far");
         std::vector<int> big;   // ACA ranks above what the shared-memory re-compression holds
         for (int b = b0; b < b1; ++b)
             if (rank[b] > RC_SMALL) big.push_back(b);
-        k_aca_recompress<<<nc, NT, smem>>>(b0, nc, X.B.rptr, X.B.cptr, eps, W, Uo, Vo);
+        k_aca_recompress<<<nc, NT, smem>>>(d_order + b0, nc, X.B.rptr, X.B.cptr, eps, W, Uo, Vo);
         for (size_t x0 = 0; x0 < big.size(); x0 += BIG_BATCH) {
             const int nbl = (int)std::min<size_t>(BIG_BATCH, big.size() - x0);
             if ((e = X.mem.grow(&d_big, &hbig, (size_t)nbl * 2 * ACA_RCAP * ACA_RCAP)) ||
