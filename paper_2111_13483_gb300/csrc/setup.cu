@@ -11,8 +11,8 @@
 //   Dinv + doff[k]      D_k^{-1} for the Eq. 28 preconditioner.
 // Step k: pivot inverse, panel, Schur updates
 // A_ij -= A_ik W_kj for i >= j in S_k (Eq. 19; diagonal blocks in full; one CTA per block
-// pair in FP64, one CTA per row block and group of up to 8 column blocks in FP32).  Stream
-// order gives the step dependencies.
+// pair in FP64, one CTA per row block and group of up to 16 column blocks in FP32).  Stream
+// order and the two events of the look-ahead give the step dependencies.
 //
 // S is the storage and arithmetic type of A, the diagonal blocks and W: complex FP64, or
 // complex FP32 in the mixed-precision setup, where the pivot blocks are still inverted in
@@ -305,13 +305,16 @@ __global__ void __launch_bounds__(256) k_panel(int k, const int *size, const int
 // outputs of the block lie flat over the threads: a DFMA warp instruction holds its scheduler for 64 cycles whatever its
 // lanes do and shared-memory loads are free beside it, so full warps count, not register tiles (32 x 32 tiles
 // padded the 18-unknown blocks of a 4,720-unknown plate threefold: 59 ms per setup).
+// The updates of a step come in one launch (UPD_ALL), or in two: the blocks of the first column of S_k, which the next
+// pivot block may be waiting for (UPD_FIRST, ns CTAs), and those of the other ns columns (UPD_REST, ns one less).
+constexpr int UPD_ALL = 0, UPD_FIRST = 1, UPD_REST = 2;
 constexpr int UPD64_T = 128;
 __device__ __forceinline__ void upd64_cp(double2 *dst, const double2 *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
 }
-__global__ void __launch_bounds__(UPD64_T) k_update64(int k, int ns, const int *size, const int *sptr, const int *sidx,
+__global__ void __launch_bounds__(UPD64_T) k_update64(int k, int ns, int part, const int *size, const int *sptr, const int *sidx,
                                                       const int *srow, const int *M, const int64_t *coff,
                                                       const int64_t *doff, const double2 *W, double2 *A, double2 *Ad)
 {
@@ -321,9 +324,13 @@ __global__ void __launch_bounds__(UPD64_T) k_update64(int k, int ns, const int *
     int a = (int)sqrtf(2.0f * (float)t);
     while ((long)(a + 1) * (a + 2) / 2 <= t) ++a;
     while ((long)a * (a + 1) / 2 > t) --a;
-    const int b = (int)(t - (long)a * (a + 1) / 2);
+    int b = (int)(t - (long)a * (a + 1) / 2);
+    if (part == UPD_FIRST) {
+        a = (int)t;
+        b = 0;
+    }
     if (a >= ns) return;
-    const int e0 = sptr[k];
+    const int e0 = sptr[k] + (part == UPD_REST);
     const int i = sidx[e0 + a], j = sidx[e0 + b];
     const int nk = size[k], ni = size[i], nj = size[j];
     const int Mk = M[k];
@@ -440,7 +447,7 @@ __device__ __forceinline__ void upd_piece(const float2 *As, int lda, const float
 __host__ __device__ __forceinline__ int upd_wcap(int nk) { return UPD_C * nk + 2; }
 static size_t upd_smem(int nk, int lda) { return sizeof(float2) * ((size_t)nk * lda + 2 * UPD_NW * (size_t)upd_wcap(nk)); }
 
-__global__ void __launch_bounds__(32 * UPD_NW, UPD_CTAS) k_update_grp(int k, int ns, int lg, int lda, const int *size,
+__global__ void __launch_bounds__(32 * UPD_NW, UPD_CTAS) k_update_grp(int k, int ns, int part, int lg, int lda, const int *size,
                                                                       const int *sptr, const int *sidx, const int *srow,
                                                                       const int *M, const int64_t *coff,
                                                                       const int64_t *doff, const float2 *W, float2 *A,
@@ -454,9 +461,12 @@ __global__ void __launch_bounds__(32 * UPD_NW, UPD_CTAS) k_update_grp(int k, int
         if (upd_first(mid, lg) <= t) lo = mid;
         else hi = mid;
     }
-    const int a = lo, b0 = (int)(t - upd_first(a, lg)) << lg, b1 = min(a + 1, b0 + (1 << lg));
-    if (b0 > a) return;   // cannot happen: row a has ceil((a + 1) / gb) groups
-    const int e0 = sptr[k], i = sidx[e0 + a], nk = size[k], ni = size[i], Mk = M[k];
+    // UPD_FIRST: CTA = row, the warps share its block of column 0 (UPD_NW UPD_C = 64 columns at most)
+    const bool one = part == UPD_FIRST;
+    const int a = one ? (int)t : lo, b0 = one ? 0 : (int)(t - upd_first(a, lg)) << lg;
+    const int b1 = one ? 1 : min(a + 1, b0 + (1 << lg));
+    if (b0 > a || a >= ns) return;   // cannot happen: row a has ceil((a + 1) / gb) groups
+    const int e0 = sptr[k] + (part == UPD_REST), i = sidx[e0 + a], nk = size[k], ni = size[i], Mk = M[k];
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, cap = upd_wcap(nk);
     float2 *As = upd_sm;   // As[q * lda + r] = A_ik[r, q]
     float2 *const wb = upd_sm + nk * lda + 2 * wp * cap;
@@ -466,7 +476,8 @@ __global__ void __launch_bounds__(32 * UPD_NW, UPD_CTAS) k_update_grp(int k, int
         for (int r = lane; r < ni; r += 32) upd_cp(As + q * lda + r, Aik + r + (int64_t)q * Mk);
     // this warp's pieces: columns [c0, c0 + UPD_C) of W_kj for b = b0 + wp, b0 + wp + UPD_NW, ...; the 16-byte words that
     // hold them (panel allocations end on 256 bytes)
-    int b = b0 + wp, c0 = 0;
+    const int cstart = one ? wp * UPD_C : 0, cstep = one ? UPD_NW * UPD_C : UPD_C;
+    int b = one ? (cstart < size[sidx[e0]] ? 0 : 1) : b0 + wp, c0 = cstart;
     auto stage = [&](int bb, int cc, int buf) {
         if (bb < b1) {
             const float2 *src = Wk + (srow[e0 + bb] + cc) * nk;
@@ -479,16 +490,16 @@ __global__ void __launch_bounds__(32 * UPD_NW, UPD_CTAS) k_update_grp(int k, int
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
-    stage(b, 0, 0);   // one group with the A_ik copies
+    stage(b, c0, 0);   // one group with the A_ik copies
     float2 *C = nullptr;
     int ldc = 0;
     bool first = true;   // A_ik is still to be waited for, by the whole CTA
     for (int buf = 0; b < b1; buf ^= 1) {
         const int j = sidx[e0 + b], nj = size[j], nc = min(UPD_C, nj - c0);
-        const bool last = c0 + UPD_C >= nj;
-        const int bn = last ? b + UPD_NW : b, cn = last ? 0 : c0 + UPD_C;
+        const bool last = c0 + cstep >= nj;
+        const int bn = last ? b + UPD_NW : b, cn = last ? cstart : c0 + cstep;
         stage(bn, cn, buf ^ 1);
-        if (c0 == 0) {
+        if (c0 == cstart) {
             if (i == j) {
                 C = Ad + doff[i];
                 ldc = ni;
@@ -623,7 +634,7 @@ static int upd_group(int ns, int nsm)
 
 // count pivot blocks from k on, of at most nk unknowns, each on CL CTAs
 template <class S, int CL>
-static cudaError_t pivot_launch(hm_ctx *h, int k, int count, int nk, const S *Ad, float2 *Dinv32)
+static cudaError_t pivot_launch(hm_ctx *h, cudaStream_t st, int k, int count, int nk, const S *Ad, float2 *Dinv32)
 {
     const size_t smem = sizeof(double2) * 2 * (size_t)nk * ((nk + CL - 1) / CL);
     static DeviceOnce attr;
@@ -637,7 +648,7 @@ static cudaError_t pivot_launch(hm_ctx *h, int k, int count, int nk, const S *Ad
     cfg.gridDim = dim3((unsigned)(CL * count), 1, 1);
     cfg.blockDim = dim3(128, 1, 1);   // one warp per scheduler
     cfg.dynamicSmemBytes = smem;
-    cfg.stream = h->stream;
+    cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = CL;
@@ -656,15 +667,41 @@ static cudaError_t pivot_launch(hm_ctx *h, int k, int count, int nk, const S *Ad
 // their schedulers save (4,720-unknown plate, blocks of 18: 11.7 / 10.2 / 11.7 / 14.8 ms per setup on 1 / 2 /
 // 4 / 8; 29,800-unknown plate, 29: 101 / 70 / 71 / 91), on four above (1,920-unknown sphere, 34: 11.5 / 7.2 /
 // 5.1 / 6.6 ms; 30,720-unknown sphere: 175 / 113 / 83 / 105 ms).
-template <class S> static cudaError_t pivot_step(hm_ctx *h, int k, int nk, const S *Ad, float2 *Dinv32)
+template <class S>
+static cudaError_t pivot_step(hm_ctx *h, cudaStream_t st, int k, int nk, const S *Ad, float2 *Dinv32)
 {
     switch (h->pivot_cl ? h->pivot_cl : nk <= 28 ? 2 : 4) {
-    case 2: return pivot_launch<S, 2>(h, k, 1, nk, Ad, Dinv32);
-    case 4: return pivot_launch<S, 4>(h, k, 1, nk, Ad, Dinv32);
-    case 8: return pivot_launch<S, 8>(h, k, 1, nk, Ad, Dinv32);
-    default: return pivot_launch<S, 1>(h, k, 1, nk, Ad, Dinv32);
+    case 2: return pivot_launch<S, 2>(h, st, k, 1, nk, Ad, Dinv32);
+    case 4: return pivot_launch<S, 4>(h, st, k, 1, nk, Ad, Dinv32);
+    case 8: return pivot_launch<S, 8>(h, st, k, 1, nk, Ad, Dinv32);
+    default: return pivot_launch<S, 1>(h, st, k, 1, nk, Ad, Dinv32);
     }
 }
+
+// The stream of the pivots that run ahead.  Its work is over before the object is, on every way out.
+struct Ahead {
+    cudaStream_t st = nullptr;
+    cudaEvent_t upd = nullptr, pan = nullptr;   // the next pivot's inputs are final; its panel is
+    cudaError_t open()
+    {
+        int lo = 0, hi = 0;
+        cudaError_t e;
+        if ((e = cudaDeviceGetStreamPriorityRange(&lo, &hi)) ||
+            (e = cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, hi)) ||
+            (e = cudaEventCreateWithFlags(&upd, cudaEventDisableTiming)))
+            return e;
+        return cudaEventCreateWithFlags(&pan, cudaEventDisableTiming);
+    }
+    ~Ahead()
+    {
+        if (st) {
+            cudaStreamSynchronize(st);
+            cudaStreamDestroy(st);
+        }
+        if (upd) cudaEventDestroy(upd);
+        if (pan) cudaEventDestroy(pan);
+    }
+};
 
 template <class S>
 static cudaError_t setup_typed(hm_ctx *h, S *A, S *Ad, S *W, S *DinvS, float2 *Dinv32, int *bad_block)
@@ -709,38 +746,64 @@ static cudaError_t setup_typed(hm_ctx *h, S *A, S *Ad, S *W, S *DinvS, float2 *D
         if ((e = cudaFuncSetAttribute(k_update_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::SMEM_BYTES)))
             return e;
     }
-    for (int k = 0; k < P.nb; ++k) {
-        int nk = P.size[k];
-        if ((e = pivot_step<S>(h, k, nk, Ad, Dinv32))) return e;
-        int ns = P.sptr[k + 1] - P.sptr[k];
-        if (ns > 0) {
-            int Mk = P.M[k];
+    // Look-ahead: the pivot and panel of block k + 1 run on a stream of their own once the first column of the updates
+    // of step k is done, beside the others.  They occupy a few SMs for 85 us a step, the updates up to all of them:
+    // 345 -> 302 ms per mixed setup of the 30,720-unknown sphere, 162 -> 130 of a 29,800-unknown plate, 35 -> 31 per FP64
+    // setup of a 4,720-unknown plate.
+    // Off where a launch is timed, where the panel is compressed before its updates and for the tensor-core updates.
+    Ahead ahead;
+    const bool on = P.nb > 1 && !h->prof.on && !h->opts.compress_in_setup && !(sizeof(S) == 8 && h->update_kind == 2);
+    if (on && (e = ahead.open())) return e;
+    const cudaStream_t ps = on ? ahead.st : st;
+    auto factor = [&](int k) -> cudaError_t {   // pivot block k and its panel
+        cudaError_t e2;
+        if (on && ((e2 = cudaEventRecord(ahead.upd, st)) || (e2 = cudaStreamWaitEvent(ps, ahead.upd, 0)))) return e2;
+        if ((e2 = pivot_step<S>(h, ps, k, P.size[k], Ad, Dinv32))) return e2;
+        if (P.sptr[k + 1] > P.sptr[k])
             HM_LAUNCH(h, K_PANEL,
-                      k_panel<S><<<(Mk + PANEL_COLS<S> - 1) / PANEL_COLS<S>, 256, panel_smem<S>(nk), st>>>(
+                      k_panel<S><<<(P.M[k] + PANEL_COLS<S> - 1) / PANEL_COLS<S>, 256, panel_smem<S>(P.size[k]), ps>>>(
                           k, h->d_size, h->d_M, h->d_coff, h->d_doff, DinvS, A, W));
-            if (h->opts.compress_in_setup && (e = compress_step<S>(h, k, W))) return e;
-            if constexpr (sizeof(S) == 8) {
-                if (h->update_kind == 2) {
-                    HM_LAUNCH(h, K_UPDATE,
-                              k_update_tc<<<(unsigned)h->utot[k], 256, tc::SMEM_BYTES, st>>>(
-                                  k, ns, h->d_ucum, h->d_size, h->d_sptr, h->d_sidx, h->d_srow, h->d_M, h->d_coff,
-                                  h->d_doff, W, A, Ad, h->d_err, WAIT_NS_DEFAULT));
-                    if ((e = cudaGetLastError())) return e;
-                    continue;
-                }
-                const int lg = upd_group(ns, nsm);
-                HM_LAUNCH(h, K_UPDATE,
-                          k_update_grp<<<(unsigned)upd_first(ns, lg), 32 * UPD_NW, upd_smem(nk, lda), st>>>(
-                              k, ns, lg, lda, h->d_size, h->d_sptr, h->d_sidx, h->d_srow, h->d_M, h->d_coff, h->d_doff,
-                              W, A, Ad));
-            } else {
-                long nt = (long)ns * (ns + 1) / 2;
-                HM_LAUNCH(h, K_UPDATE,
-                          k_update64<<<(unsigned)nt, UPD64_T, sizeof(double2) * 2 * maxn * nk, st>>>(
-                              k, ns, h->d_size, h->d_sptr, h->d_sidx, h->d_srow, h->d_M, h->d_coff, h->d_doff, W, A, Ad));
-            }
+        if ((e2 = cudaGetLastError())) return e2;
+        return on ? cudaEventRecord(ahead.pan, ps) : cudaSuccess;
+    };
+    auto update = [&](int k, int ns, int part) -> cudaError_t {
+        if (ns <= 0) return cudaSuccess;
+        const int nk = P.size[k];
+        if constexpr (sizeof(S) == 8) {
+            const int lg = upd_group(ns, nsm);
+            HM_LAUNCH(h, K_UPDATE,
+                      k_update_grp<<<(unsigned)(part == UPD_FIRST ? ns : upd_first(ns, lg)), 32 * UPD_NW, upd_smem(nk, lda), st>>>(
+                          k, ns, part, lg, lda, h->d_size, h->d_sptr, h->d_sidx, h->d_srow, h->d_M, h->d_coff, h->d_doff,
+                          W, A, Ad));
+        } else {
+            const long nt = part == UPD_FIRST ? ns : (long)ns * (ns + 1) / 2;
+            HM_LAUNCH(h, K_UPDATE,
+                      k_update64<<<(unsigned)nt, UPD64_T, sizeof(double2) * 2 * maxn * nk, st>>>(
+                          k, ns, part, h->d_size, h->d_sptr, h->d_sidx, h->d_srow, h->d_M, h->d_coff, h->d_doff, W, A, Ad));
         }
-        if ((e = cudaGetLastError())) return e;
+        return cudaGetLastError();
+    };
+    if ((e = factor(0))) return e;
+    for (int k = 0; k < P.nb; ++k) {
+        const int ns = P.sptr[k + 1] - P.sptr[k];
+        if (on) {
+            const bool next = ns > 0 && P.sidx[P.sptr[k]] == k + 1;
+            if ((e = cudaStreamWaitEvent(st, ahead.pan, 0))) return e;
+            if (next && (e = update(k, ns, UPD_FIRST))) return e;
+            if (k + 1 < P.nb && (e = factor(k + 1))) return e;
+            if ((e = next ? update(k, ns - 1, UPD_REST) : update(k, ns, UPD_ALL))) return e;
+            continue;
+        }
+        if (ns > 0 && h->opts.compress_in_setup && (e = compress_step<S>(h, k, W))) return e;
+        if constexpr (sizeof(S) == 8) {
+            if (ns > 0 && h->update_kind == 2)
+                HM_LAUNCH(h, K_UPDATE,
+                          k_update_tc<<<(unsigned)h->utot[k], 256, tc::SMEM_BYTES, st>>>(
+                              k, ns, h->d_ucum, h->d_size, h->d_sptr, h->d_sidx, h->d_srow, h->d_M, h->d_coff, h->d_doff,
+                              W, A, Ad, h->d_err, WAIT_NS_DEFAULT));
+        }
+        if (!(sizeof(S) == 8 && h->update_kind == 2) && (e = update(k, ns, UPD_ALL))) return e;
+        if (k + 1 < P.nb && (e = factor(k + 1))) return e;
     }
     int herr = 0;
     if ((e = cudaMemcpyAsync(&herr, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, st))) return e;
@@ -765,7 +828,7 @@ cudaError_t block_jacobi_setup(hm_ctx *h, int *bad_block)
                   (int)h->near_t.size(), h->d_near_t, h->d_near_s, h->d_near_off, h->d_near, h->d_leaf_ptr, h->d_pos,
                   h->d_sptr, h->d_sidx, h->d_srow, h->d_M, h->d_coff, h->d_doff, (double2 *)nullptr, h->d_Ad, h->d_err,
                   true));
-    if ((e = pivot_launch<double2, 1>(h, 0, P.nb, *std::max_element(P.size.begin(), P.size.end()), h->d_Ad, nullptr)))
+    if ((e = pivot_launch<double2, 1>(h, st, 0, P.nb, *std::max_element(P.size.begin(), P.size.end()), h->d_Ad, nullptr)))
         return e;
     if ((e = cudaGetLastError())) return e;
     int herr = 0;
