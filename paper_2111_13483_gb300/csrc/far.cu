@@ -348,6 +348,184 @@ __global__ void __launch_bounds__(256) k_far_y(int nl, const int *leaf_ptr, cons
     tile_store(acc, part + (size_t)pp * n * nrhs + cl2new[a], 1, n, ni, nrhs, nrt, ntiles);
 }
 
+// ---- complex FP32, more than 16 columns ----------------------------------------------------
+// The same two phases for wide batches.  A warp owns a patch of 16 rows x 32 columns, a lane 4 x 4 outputs of it: rows
+// 2 (l % 4) + {0, 1, 8, 9} and columns 4 (l / 4) + {0 .. 3}, so that a contraction step is four conflict-free 16-byte
+// shared-memory loads for 64 FMAs; the CTA has as many warps as the block has patches.  Staging goes one contraction row
+// (or factor column) per warp turn, without divisions, the vector rows in 16-byte words when nrhs is even.
+// Issue slots bound it: 2 x 4 outputs per lane of a 256-thread CTA with element-wise staging spent as many on addresses
+// and loads as on FMAs (64 columns of the 30,720-unknown sphere: 1.04 + 1.98 ms, now
+// 0.68 + 1.52; 23 columns of a 22,500-unknown plate: 0.25 + 0.42, now 0.24 + 0.29).  A ring of four chunks leaves fewer CTAs
+// per SM (phase 2 of 23 columns 0.95 -> 1.11 ms), patches of 32 rows waste more of the 28-row leaves (1.64 for 1.52).
+constexpr int F32_ROWS = 16, F32_COLS = 32;   // patch of a warp
+constexpr int F32_KC = 16, F32_RING = 3;      // contraction entries of a chunk, chunks in shared memory
+__host__ __device__ __forceinline__ int f32_np(int no) { return (no + F32_ROWS - 1) / F32_ROWS; }
+__host__ __device__ __forceinline__ int f32_nc(int nrhs) { return (nrhs + F32_COLS - 1) / F32_COLS; }
+// row strides of the staged blocks: whole patches; even, for 16-byte loads
+__host__ __device__ __forceinline__ int f32_ldw(int np) { return np * F32_ROWS + 2; }
+
+__device__ __forceinline__ void far_cp16(float2 *dst, const float2 *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+// one vector row of nrhs <= 64 entries; v16: nrhs is even and the vectors start on 16 bytes, so every row does
+__device__ __forceinline__ void f32_row(float2 *dst, const float2 *src, int nrhs, bool v16)
+{
+    const int lane = threadIdx.x & 31;
+    if (v16) {
+        if (2 * lane < nrhs) far_cp16(dst + 2 * lane, src + 2 * lane);
+    } else
+        for (int r = lane; r < nrhs; r += 32) far_cp(dst + r, src + r);
+}
+// acc += the staged step, terms in ascending order (the order of tile_mac)
+__device__ __forceinline__ void f32_mac(float2 (&acc)[4][4], const float2 *wp, int ldw, const float2 *yp, int ldr, int nc)
+{
+#pragma unroll 2
+    for (int q = 0; q < nc; ++q, wp += ldw, yp += ldr) {
+        const float4 w0 = *(const float4 *)wp, w1 = *(const float4 *)(wp + 8), y0 = *(const float4 *)yp,
+                     y1 = *(const float4 *)(yp + 2);
+        const float2 w[4] = {make_float2(w0.x, w0.y), make_float2(w0.z, w0.w), make_float2(w1.x, w1.y),
+                             make_float2(w1.z, w1.w)};
+        const float2 y[4] = {make_float2(y0.x, y0.y), make_float2(y0.z, y0.w), make_float2(y1.x, y1.y),
+                             make_float2(y1.z, y1.w)};
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[a][c] = cfma(w[a], y[c], acc[a][c]);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_far_t32(const int *task_lo, const int *task_hi, const int *task_ptr,
+                                                 const int64_t *item_off, const int *item_ld, const int *item_rank,
+                                                 const int *item_row, const int *item_isv, const float2 *U, const float2 *V,
+                                                 const float2 *u, int nrhs, float2 *t, float2 *s, bool v16)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ int s_item[64], s_l[64];
+    __shared__ const float2 *s_src[64];
+    const int task = blockIdx.x;
+    const int lo = task_lo[task], hi = task_hi[task], i0 = task_ptr[task], i1 = task_ptr[task + 1];
+    const int R = far_items(i0, i1, item_off, item_ld, item_rank, item_isv, U, V, s_item, s_l, s_src);
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int ncol = f32_nc(nrhs), ldw = f32_ldw(4), ldr = ncol * F32_COLS;
+    const int prow = wp / ncol, row0 = prow * F32_ROWS + 2 * (lane & 3), col0 = wp % ncol * F32_COLS + 4 * (lane >> 2);
+    float2 *const ring = (float2 *)smraw;
+    float2 acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[a][c] = make_float2(0.f, 0.f);
+    const int nch = (hi - lo + F32_KC - 1) / F32_KC;
+    // chunk c: Ws[qq * ldw + rr], then Ys[qq * ldr + r]; half a warp per factor column
+    auto stage = [&](int c) {
+        const int c0 = lo + c * F32_KC, ch = min(F32_KC, hi - c0), qh = lane & 15;
+        float2 *Ws = ring + c % F32_RING * F32_KC * (ldw + ldr), *Ys = Ws + F32_KC * ldw;
+        if (c < nch) {
+            if (qh < ch)
+                for (int rr = 2 * wp + (lane >> 4); rr < R; rr += 2 * nw) far_cp(Ws + qh * ldw + rr, s_src[rr] + (c0 - lo + qh));
+            for (int qq = wp; qq < ch; qq += nw) f32_row(Ys + qq * ldr, u + (int64_t)(c0 + qq) * nrhs, nrhs, v16);
+        }
+        cp_async_commit();
+    };
+    stage(0);
+    stage(1);
+    for (int c = 0; c < nch; ++c) {
+        cp_async_wait<1>();
+        __syncthreads();   // chunk c has landed, chunk c - 1 is consumed
+        stage(c + 2);
+        const float2 *Ws = ring + c % F32_RING * F32_KC * (ldw + ldr);
+        if (prow * F32_ROWS < R)
+            f32_mac(acc, Ws + row0, ldw, Ws + F32_KC * ldw + col0, ldr, min(F32_KC, hi - lo - c * F32_KC));
+    }
+    cp_async_wait<0>();
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const int row = row0 + (a & 1) + 8 * (a >> 1);
+        if (row >= R) continue;
+        const int it = s_item[row];
+        float2 *dst = (item_isv[it] ? t : s) + (int64_t)(item_row[it] + s_l[row]) * nrhs;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (col0 + c < nrhs) dst[col0 + c] = acc[a][c];
+    }
+}
+
+// phase 2 (see k_far_y); np: patches that cover the rows of the largest leaf
+__global__ void __launch_bounds__(256) k_far_y32(int nl, const int *leaf_ptr, const int *part_ptr, const int *kcum,
+                                                 const FarSegD *segs, const float2 *U, const float2 *V, const float2 *t,
+                                                 const float2 *s, const float2 *u, const int *cl2new, int n, int nrhs,
+                                                 float2 *part, int np, bool v16)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int l = blockIdx.x / FAR_PARTS, pp = blockIdx.x % FAR_PARTS;
+    if (l >= nl) return;
+    const int a0 = leaf_ptr[l], ni = leaf_ptr[l + 1] - a0;
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int ncol = f32_nc(nrhs), ldw = f32_ldw(np), ldr = ncol * F32_COLS;
+    const int prow = wp / ncol, row0 = prow * F32_ROWS + 2 * (lane & 3), col0 = wp % ncol * F32_COLS + 4 * (lane >> 2);
+    float2 *const ring = (float2 *)smraw;
+    float2 acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[a][c] = make_float2(0.f, 0.f);
+    const int p0 = part_ptr[blockIdx.x], w1 = part_ptr[blockIdx.x + 1];
+    const int k0 = p0 < w1 ? kcum[p0] : 0, K = p0 < w1 ? kcum[w1] - k0 : 0, nch = (K + F32_KC - 1) / F32_KC;
+    // the part's stacked contraction entries, one per warp turn; a warp follows the segments in order, with the next
+    // segment's descriptor on its way
+    int q = p0, qlo = 0, qhi = 0;
+    FarSegD g = {}, gn = {};
+    int hn = 0;   // end of the next segment
+    if (K > 0) {
+        gn = segs[p0];
+        hn = kcum[p0 + 1] - k0;
+    }
+    const float2 *F = nullptr, *Yb = nullptr;
+    auto stage = [&](int c) {
+        float2 *Ws = ring + c % F32_RING * F32_KC * (ldw + ldr), *Ys = Ws + F32_KC * ldw;
+        const int ke = min(K, (c + 1) * F32_KC);
+        for (int kk = c * F32_KC + wp; kk < ke; kk += nw) {
+            while (kk >= qhi) {
+                g = gn;
+                qlo = qhi;
+                qhi = hn;
+                ++q;
+                if (q < w1) {
+                    gn = segs[q];
+                    hn = kcum[q + 1] - k0;
+                }
+                F = ((g.src & 1) ? V : U) + g.foff;
+                const int ys = g.src >> 1;
+                Yb = (ys == 0 ? t : (ys == 1 ? s : u)) + g.yrow * nrhs;
+            }
+            const float2 *f = F + (int64_t)(kk - qlo) * g.fk;
+            const int o = kk - c * F32_KC;
+            for (int i = lane; i < ni; i += 32) far_cp(Ws + o * ldw + i, f + (int64_t)i * g.fi);
+            f32_row(Ys + o * ldr, Yb + (int64_t)(kk - qlo) * nrhs, nrhs, v16);
+        }
+        cp_async_commit();
+    };
+    stage(0);
+    stage(1);
+    for (int c = 0; c < nch; ++c) {
+        cp_async_wait<1>();
+        __syncthreads();   // chunk c has landed, chunk c - 1 is consumed
+        stage(c + 2);
+        const float2 *Ws = ring + c % F32_RING * F32_KC * (ldw + ldr);
+        if (prow * F32_ROWS < ni) f32_mac(acc, Ws + row0, ldw, Ws + F32_KC * ldw + col0, ldr, min(F32_KC, K - c * F32_KC));
+    }
+    cp_async_wait<0>();
+    float2 *out = part + (size_t)pp * n * nrhs + cl2new[a0];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int row = row0 + (a & 1) + 8 * (a >> 1);
+            if (row < ni && col0 + c < nrhs) out[row + (int64_t)(col0 + c) * n] = acc[a][c];
+        }
+}
+
 // complex FP64, phase 2 (see f64_mac): the segments of the far list and, with nearp, those of the leaf's
 // near-field blocks (zpart / zkcum / zsegs), which gives Z u in one pass
 template <int NU>
@@ -775,14 +953,50 @@ cudaError_t far_product64(hm_ctx *h, const double2 *U, const double2 *V, double2
     return far64_run<16, 16>(h, U, V, t, s, ucl, y, nrhs, near);
 }
 
+// complex FP32, 17 to 64 columns
+static cudaError_t far32_run(hm_ctx *h, const float2 *U, const float2 *V, float2 *t, float2 *s, const float2 *ucl,
+                             float2 *y, int nrhs)
+{
+    const FarPlan &F = h->fplan;
+    const int n = h->plan.n, np = f32_np(h->max_leaf), nc = f32_nc(nrhs), ldr = nc * F32_COLS;
+    const size_t smt = sizeof(float2) * F32_RING * F32_KC * (size_t)(f32_ldw(4) + ldr);
+    const size_t smy = sizeof(float2) * F32_RING * F32_KC * (size_t)(f32_ldw(np) + ldr);
+    static DeviceOnce attr;
+    if (attr.need()) {   // 64 rows and 64 columns
+        const int smax = (int)(sizeof(float2) * F32_RING * F32_KC * (f32_ldw(4) + 64));
+        cudaError_t e;
+        if ((e = cudaFuncSetAttribute(k_far_t32, cudaFuncAttributeMaxDynamicSharedMemorySize, smax)) ||
+            (e = cudaFuncSetAttribute(k_far_y32, cudaFuncAttributeMaxDynamicSharedMemorySize, smax)))
+            return e;
+        attr.done();
+    }
+    const bool v16 = nrhs % 2 == 0 && (((uintptr_t)t | (uintptr_t)s | (uintptr_t)ucl) & 15) == 0;
+    const int ntask = (int)F.p1_lo.size();
+    if (ntask > 0)
+        HM_LAUNCH(h, K_FAR1,
+                  k_far_t32<<<ntask, 32 * 4 * nc, smt, h->stream>>>(h->d_p1_lo, h->d_p1_hi, h->d_p1_ptr, h->d_p1_off,
+                                                                    h->d_p1_ld, h->d_p1_rank, h->d_p1_row, h->d_p1_isv, U,
+                                                                    V, ucl, nrhs, t, s, v16));
+    float2 *part = (float2 *)h->d_farpart;
+    HM_LAUNCH(h, K_FAR2,
+              k_far_y32<<<h->nl * FAR_PARTS, 32 * np * nc, smy, h->stream>>>(
+                  h->nl, h->d_leaf_ptr, h->d_part_ptr, h->d_seg_kcum, h->d_segs, U, V, t, s, ucl, h->d_cl2new, n, nrhs,
+                  part, np, v16));
+    const int64_t len = (int64_t)n * nrhs;
+    HM_LAUNCH(h, K_FAR2, k_far_sum<float2><<<nblk(len, 256), 256, 0, h->stream>>>(len, part, y));
+    return cudaGetLastError();
+}
+
 cudaError_t far_product32(hm_ctx *h, const float2 *U, const float2 *V, float2 *t, float2 *s, const float2 *ucl, float2 *y,
                           int nrhs)
 {
     h->prof.cols[K_FAR1] += nrhs;
     h->prof.cols[K_FAR2] += nrhs;
     if (h->far_kind == 2) return far_tc_launch(h, U, V, t, s, ucl, y, nrhs);
+    // the wide kernels from 17 columns on: their warps cover 32 (at 16 columns half of the lanes would be idle)
+    if (nrhs > 16) return far32_run(h, U, V, t, s, ucl, y, nrhs);
     FarLaunch<float2> f{h, U, V, t, s, ucl, y, nrhs};
-    return tile_dispatch<float2>(nrhs, f);
+    return nrhs <= 4 ? f.run<1, 1, 1>(4) : f.run<2, 2, 1>(16);
 }
 
 }  // namespace hm

@@ -133,3 +133,27 @@ def test_products_and_solves_of_uneven_blocks(sizes):
     I, its, rr, code = hm.solve(h, B, tol=1e-10, restart=20)
     assert code == 0
     assert np.all(np.linalg.norm(B - Z @ I, axis=0) <= 2e-10 * np.linalg.norm(B, axis=0))
+
+
+@pytest.mark.parametrize("sizes", [MIXED, [32] * 9, [33] * 9, [1, 64, 2, 33, 5, 6, 7, 8, 9, 10]])
+def test_far_field_widths(sizes):
+    """The complex-FP32 far field where its kernels change (16 / 17 columns, even and odd widths, blocks of one and of two
+    row patches): the bits of every column at every width, and 1e-5 (600 terms, sqrt(600) u 5) of the exact product."""
+    P, N, Z = problem(sizes, 3)
+    h = hm.hmat_create(P, ordering=1, precision=1)
+    hm.precond_setup(h)
+    rng = np.random.default_rng(2)
+    X = rng.standard_normal((64, P.n)) + 1j * rng.standard_normal((64, P.n))
+    p = np.asarray(hm.hm_get_index_map(h))
+    F = (Z - N)[np.ix_(p, p)]
+    np.fill_diagonal(F, 0)
+    ref = None
+    for w in (64, 4, 16, 17, 18, 23, 32, 33, 48, 49, 63):
+        x = torch.from_numpy(X[:w]).cuda()
+        y = torch.empty_like(x)
+        hm.hm_apply(h, H.OP32 + H.OP_ZF, x, y)
+        y = y.cpu().numpy()
+        ref = y if ref is None else ref
+        assert np.array_equal(y, ref[:w])
+    want = X @ F.T
+    assert np.max(np.abs(ref - want)) <= 1e-5 * np.max(np.abs(want))
