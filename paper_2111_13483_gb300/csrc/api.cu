@@ -251,7 +251,7 @@ int hmat_create(const hm_desc *d, const hm_opts *opts, hm_handle *out)
     if ((e = h->arena.alloc((void **)&h->d_err, sizeof(int) * ERR_WORDS)) ||
         (e = h->arena.alloc((void **)&h->d_ticket, sizeof(int))) ||
         (e = cudaMemcpy(h->d_err, err_init, sizeof(err_init), cudaMemcpyHostToDevice)) ||
-        (h->opts.precision == 1 && (e = make_fp32_copies(h))) || (e = cudaStreamSynchronize(h->stream))) {
+        (e = far64_prepare(h)) || (h->opts.precision == 1 && (e = make_fp32_copies(h))) || (e = cudaStreamSynchronize(h->stream))) {
         int s = cuda_fail(h, e, "hmat_create");
         h->arena.release_all();
         if (h->own_stream) cudaStreamDestroy(h->stream);

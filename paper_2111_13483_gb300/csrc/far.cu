@@ -8,7 +8,8 @@
 // Phase 1 (k_far_t): the rank vectors t_b = V_b^T u[c-range] and s_b = U_b^T u[r-range].
 // Factor columns that contract over the same index range are stacked (up to 64 per task),
 // so one CTA stages each piece of u once for all of them (cp.async, double buffered) and
-// runs a register-tiled product (tile.cuh); t and s are stored interleaved like u.
+// runs a register-tiled product (tile.cuh; complex FP64: integer digits on the tensor cores); t and s are stored
+// interleaved like u.
 // Phase 2 (k_far_y): one CTA per leaf accumulates, in the order of the leaf's list of
 // covering far blocks, U_b t_b (row side), V_b s_b (column side), B u (dense row side) and
 // B^T u (dense column side) for the leaf's rows; the host plan cuts the list into
@@ -18,6 +19,7 @@
 // one fixed order, so results are deterministic and do not depend on how many right-hand
 // sides share the launch.
 #include <algorithm>
+#include <cstdint>
 
 #include "cplx.cuh"
 #include "hm_internal.h"
@@ -137,107 +139,378 @@ __global__ void __launch_bounds__(256) k_far_t(const int *task_lo, const int *ta
 }
 
 // ---- complex FP64 ---------------------------------------------------------------------------
-// GB300 issues a DFMA for two lanes per SM and clock: one warp instruction holds its scheduler for 64
-// cycles whatever its lanes do, and shared-memory loads are free beside it.  So the outputs are laid flat
-// over the lanes (28 rows x 16 columns are 14 full warps; 2 x 2 register tiles left an eighth of the
-// lanes idle), and the contraction is split F64_NK ways (entry kk of the whole contraction to
-// way kk mod F64_NK, partial sums added in order), so that one column keeps all four schedulers busy
-// too.  The split does not depend on the columns: a column's bits are the same in any batch.
-// The near-field blocks of a leaf join its phase-2 segments where Z itself is applied.
-// Measured at 64 columns on the 30,720-unknown sphere: phase 1 23.5 -> 22.8 ms, phase 2 38.6 and the near field
-// 34.6 (a CTA of its own per leaf) -> 47.2 ms together; one column: 0.64 -> 0.46 and 1.37 + 0.80 -> 1.42 ms.
-// Phase 2 runs at the DFMA rate (0.63 T/s measured by a chain of FMAs).
-constexpr int F64_NK = 4, F64_NH = 2;   // ways the contraction and the outputs are split over the warps
-constexpr int F64_T = 32 * F64_NK * F64_NH;
+// GB300 has two DFMA lanes per SM and clock, so the FP64 products run on the tensor cores, split into integer digits
+// (Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 2012).  With e the largest exponent of a coefficient row, and of
+// a vector column, an entry x is the integer v = x 2^(1084 - e), |v| < 2^62, truncated below 1, in eight signed
+// digits of 8 bits.  Products of digits i + j <= 7 are summed by mma.sync m16n8k16 (FP16 digits, FP32 sums): every sum of
+// 64 entries stays within 2^24 and is exact, and goes into 64-bit integers.  So a result is the exact sum of
+// truncated integers, in any order and at any width, with an error of about 2^-62 of (row maximum x column maximum)
+// per term: 2^-9 of an FP64 rounding, which leaves room for entries far below the maxima.  A row or column with
+// an infinity or a NaN gives NaN.
+constexpr int OZ_KC = 16, OZ_FOLD = 4;   // chunk = one step of the MMA; steps between foldings
+constexpr int OZ_ROWS = 32;               // rows of a CTA
 
-// acc[u] += sum over this warp's kk of Ws[kk * ldw + i] Ys[kk * ldr + c], output e = lane + 32 (F64_NH u + half) = c * no + i
-template <int NU>
-__device__ __forceinline__ void f64_mac(double2 (&acc)[NU], const double2 *Ws, int ldw, const double2 *Ys, int ldr, int k0,
-                                        int klen, int no, int len)
+// |x| < 2^(e - 1022): bytes of the result less 128 are the signed digits of the modulus, the first in the highest byte
+__device__ __forceinline__ uint2 oz_bytes(double x, int e)
 {
-    const int w = (threadIdx.x >> 5) - k0 & F64_NK - 1;   // the chunk starts at entry k0
-    const int e0 = (threadIdx.x & 31) + 32 * (threadIdx.x >> 7), di = 32 * F64_NH % no, dc = 32 * F64_NH / no;
-    for (int kk = w; kk < klen; kk += F64_NK) {
-        const double2 *wp = Ws + kk * ldw, *yp = Ys + kk * ldr;
-        int i = e0 % no, c = e0 / no;
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t mh = hi & 0xfffff | 0x100000, a = __funnelshift_l(lo, mh, 9), b = lo << 9;
+    const uint32_t r = (uint32_t)(e - (int)(hi >> 20 & 0x7ff));   // e >= 64 (oz_exp): a zero is shifted out
+    uint32_t l, h, l2;   // (a : b) >> r
+    asm("shr.u32 %0, %1, %2;" : "=r"(h) : "r"(a), "r"(r));        // shifts of 32 and more give 0
+    l = __funnelshift_rc(b, a, r);
+    asm("shr.u32 %0, %1, %2;" : "=r"(l2) : "r"(l), "r"((uint32_t)max((int)r - 32, 0)));
+    const uint64_t w = ((uint64_t)h << 32 | l2) + 0x8080808080808080ull;
+    return make_uint2((uint32_t)w, (uint32_t)(w >> 32));
+}
+// digits i of two entries as a pair of FP16 numbers: 1024 + byte - 1152 with the entry's sign
+__device__ __forceinline__ void oz_pair(double x0, double x1, int e, uint32_t (&d)[8])
+{
+    const uint2 w0 = oz_bytes(x0, e), w1 = oz_bytes(x1, e);
+    const uint32_t sg = __byte_perm((uint32_t)__double2hiint(x0), (uint32_t)__double2hiint(x1), 0x7632) & 0x80008000u;
+    const uint32_t one = sg | 0x3c003c00u, off = sg ^ 0xe480e480u;   // +-1, -+1152
 #pragma unroll
-        for (int u = 0; u < NU; ++u) {
-            const int e = e0 + 32 * F64_NH * u;
-            if (e - (int)(threadIdx.x & 31) >= len) break;
-            if (e < len) acc[u] = cfma(wp[i], yp[c], acc[u]);
-            i += di;
-            c += dc;
-            if (i >= no) i -= no, ++c;
-        }
+    for (int i = 0; i < 8; ++i) {
+        const int b = 3 - (i & 3);   // byte of the word
+        const uint32_t p = __byte_perm(i < 4 ? w0.y : w0.x, i < 4 ? w1.y : w1.x, b | b << 4 | (4 + b) << 8 | (4 + b) << 12);
+        const uint32_t q = p & 0x00ff00ffu | 0x64006400u;
+        asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d[i]) : "r"(q), "r"(one), "r"(off));
     }
 }
-
-// the warps' partial sums through shared memory: put(e, sum) for every output e < len
-template <int NU, class Put> __device__ __forceinline__ void f64_reduce(const double2 (&acc)[NU], double2 *sm, int len, Put &&put)
+__device__ __forceinline__ void oz_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
-    const int e0 = (threadIdx.x & 31) + 32 * (threadIdx.x >> 7), w = threadIdx.x >> 5 & F64_NK - 1;
-#pragma unroll
-    for (int u = 0; u < NU; ++u) {
-        const int e = e0 + 32 * F64_NH * u;
-        if (e < len) sm[w * len + e] = acc[u];
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < len; e += F64_T) {
-        double2 v = sm[e];
-        for (int q = 1; q < F64_NK; ++q) {
-            v.x += sm[q * len + e].x;
-            v.y += sm[q * len + e].y;
-        }
-        put(e, v);
-    }
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ int oz_exp(double2 v)
+{
+    return max(64, max(__double2hiint(v.x) >> 20 & 0x7ff, __double2hiint(v.y) >> 20 & 0x7ff));
 }
 
-// phase 1, tasks as in k_far_t
-template <int NU>
-__global__ void __launch_bounds__(F64_T) k_far_t64(const int *task_lo, const int *task_hi, const int *task_ptr,
-                                                   const int64_t *item_off, const int *item_ld, const int *item_rank,
-                                                   const int *item_row, const int *item_isv, const double2 *U,
-                                                   const double2 *V, const double2 *u, int nrhs, double2 *t, double2 *s,
-                                                   int half)
+// A CTA takes 32 rows x NT column tiles of 8 right-hand sides, one warp per 16 x 8 outputs.  Per chunk of 16 contraction
+// entries: the raw entries land in one of two buffers (cp.async), the warps turn them into digit fragments in
+// shared memory, once for all warps that use them, and then each runs its 144 MMAs.  Up to four columns (NARROW) the real and
+// the imaginary parts of the vectors share one tile, columns 0 .. 3 and 4 .. 7: 72 MMAs.  The integers of all forms are the
+// same, so a column's bits do not depend on the width.
+// Bound by latency and issue slots: 12 warps per SM issue in 40% of the cycles, the tensor pipe is a third busy, a pair of
+// entries takes 50 instructions to split.  Z on 64 columns of the 30,720-unknown sphere, phases 1 + 2: DFMA 22.8 + 47.2 ms
+// (its rate), with the digits in each warp's registers (225 of them, six warps per SM) 8.2 + 21.1, now 4.7 + 13.2; on one
+// column 0.46 + 1.43 by DFMA and 0.46 + 1.54 now, four 1.53 + 3.44 and 0.48 + 1.56.  Error of Z x against 64-bit-mantissa
+// products (2-norm, relative): 1.1e-16, by FP64 FMAs 1e-15.
+template <bool NARROW> struct Oz {
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int nct, ldr;                  // column tiles; row stride of the raw vector entries
+    double2 *raw;                  // [2][OZ_KC * (ldw + ldr)]
+    uint4 *ad;                     // [2 row tiles][2 parts][8 digits][32 lanes]
+    uint4 *bd;                     // [nct][8][32]: real (two words), imaginary part
+    int64_t *sum;                  // [nw][16][32]: of this lane, (part * 4 + output) * 2 + {high, low}
+    float c[2][8][4];              // sums of digit products of weight i + j
+    int steps = 0;
+    static constexpr int ldw = OZ_ROWS | 1;
+    static __host__ __device__ int tiles(int nrhs) { return NARROW ? 1 : (nrhs + 7) / 8; }
+    static size_t smem(int nrhs)
+    {
+        const int nt = tiles(nrhs);
+        return sizeof(double2) * 2 * OZ_KC * (size_t)(ldw + (nt * 8 | 1)) + (NARROW ? 8 * 32 * 8 : 16 * 32 * 8 * (size_t)(4 + nt)) + 8 * 16 * 32 * (size_t)(2 * nt);
+    }
+    __device__ __forceinline__ Oz(unsigned char *sm, int nrhs) : nct(tiles(nrhs)), ldr(nct * 8 | 1)
+    {
+        ad = (uint4 *)sm;
+        bd = ad + (NARROW ? 0 : 4 * 8 * 32);
+        sum = (int64_t *)(bd + nct * 8 * (NARROW ? 16 : 32));
+        raw = (double2 *)(sum + nw * 16 * 32);
+        sum += wp * 16 * 32 + lane;
+#pragma unroll
+        for (int x = 0; x < 16; ++x) sum[32 * x] = 0;
+        clear();
+    }
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int z = 0; z < 2; ++z)
+#pragma unroll
+            for (int w = 0; w < 8; ++w)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) c[z][w][x] = 0.f;
+        steps = 0;
+    }
+    __device__ __forceinline__ double2 *ws(int ch) const { return raw + (ch & 1) * OZ_KC * (ldw + ldr); }
+    __device__ __forceinline__ double2 *ys(int ch) const { return ws(ch) + OZ_KC * ldw; }
+    __device__ __forceinline__ int row0() const { return NARROW ? 16 * wp : 16 * (wp / nct); }
+    __device__ __forceinline__ int col0() const { return NARROW ? 0 : 8 * (wp % nct); }
+    // digits of chunk ch: rows r < rows, exponents re(row) and ce(column)
+    template <class RE, class CE> __device__ __forceinline__ void split(int ch, int rows, RE &&re, CE &&ce)
+    {
+        const int g = lane >> 2, k = 2 * (lane & 3);
+        const double2 *Ws = ws(ch), *Ys = ys(ch);
+        if constexpr (NARROW) {   // two warps, a word of the vector fragments (entries + 8 word) each; by column real or imaginary part
+            uint32_t d[8];
+            const double *y0 = (const double *)(Ys + (k + 8 * wp) * ldr + (g & 3)) + (g >> 2);
+            oz_pair(y0[0], y0[2 * ldr], ce(g & 3), d);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) ((uint32_t *)bd)[(i * 32 + lane) * 2 + wp] = d[i];
+        } else {   // 8 halves of coefficient fragments, then 2 of each column tile's, dealt out to the warps
+            for (int x = wp; x < 8 + 2 * nct; x += nw) {
+                uint32_t d[2][8];
+                uint2 *dst;
+                if (x < 8) {   // words q: rows + 8 q of entries + 8 (x & 1)
+                    const int r = 16 * (x >> 2) + g;
+                    if (r - g >= rows) continue;
+                    const double *w0 = (const double *)(Ws + (k + 8 * (x & 1)) * ldw + r) + (x >> 1 & 1);
+                    oz_pair(w0[0], w0[2 * ldw], re(r), d[0]);
+                    oz_pair(w0[16], w0[2 * ldw + 16], re(r + 8), d[1]);
+                    dst = (uint2 *)(ad + (x >> 1) * 8 * 32 + lane) + (x & 1);
+                } else {   // words q: entries + 8 q of one part
+                    const int t = x - 8 >> 1, part = x & 1, e = ce(8 * t + g);
+                    const double *y0 = (const double *)(Ys + k * ldr + 8 * t + g) + part;
+                    oz_pair(y0[0], y0[2 * ldr], e, d[0]);
+                    oz_pair(y0[16 * ldr], y0[18 * ldr], e, d[1]);
+                    dst = (uint2 *)(bd + t * 8 * 32 + lane) + part;
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) dst[64 * i] = make_uint2(d[0][i], d[1][i]);
+            }
+        }
+    }
+    // NARROW: a warp is alone with its rows and splits them into its registers
+    template <class RE> __device__ __forceinline__ void multiply_own(int ch, RE &&re)
+    {
+        const int g = lane >> 2, k = 2 * (lane & 3);
+        const uint2 *B = (const uint2 *)bd + lane;
+        uint32_t b[8][2];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const uint2 v = B[32 * j];
+            b[j][0] = v.x;
+            b[j][1] = v.y;
+        }
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {
+            uint32_t d[4][8];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int r = row0() + g + 8 * (q & 1);
+                const double *w0 = (const double *)(ws(ch) + (k + 8 * (q >> 1)) * ldw + r) + part;
+                oz_pair(w0[0], w0[2 * ldw], re(r), d[q]);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t a[4] = {d[0][i], d[1][i], d[2][i], d[3][i]};
+#pragma unroll
+                for (int j = 0; j < 8 - i; ++j) oz_mma(c[part][i + j], a, b[j][0], b[j][1]);
+            }
+        }
+        if (++steps == OZ_FOLD) fold();
+    }
+    __device__ __forceinline__ void multiply()
+    {
+        const uint4 *B = bd + wp % nct * 8 * 32 + lane, *A = ad + (row0() >> 4) * 2 * 8 * 32 + lane;
+        uint4 b[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) b[j] = B[32 * j];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint4 vr = A[32 * i], vi = A[32 * (8 + i)];
+            const uint32_t ar[4] = {vr.x, vr.y, vr.z, vr.w}, ai[4] = {vi.x, vi.y, vi.z, vi.w};
+            const uint32_t an[4] = {ai[0] ^ 0x80008000u, ai[1] ^ 0x80008000u, ai[2] ^ 0x80008000u, ai[3] ^ 0x80008000u};
+#pragma unroll
+            for (int j = 0; j < 8 - i; ++j) {
+                oz_mma(c[0][i + j], ar, b[j].x, b[j].y);
+                oz_mma(c[1][i + j], ar, b[j].z, b[j].w);
+                oz_mma(c[0][i + j], an, b[j].z, b[j].w);
+                oz_mma(c[1][i + j], ai, b[j].x, b[j].y);
+            }
+        }
+        if (++steps == OZ_FOLD) fold();
+    }
+    __device__ __forceinline__ void fold()
+    {
+#pragma unroll
+        for (int z = 0; z < 2; ++z)
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                int64_t h = sum[32 * (8 * z + 2 * x)], l = sum[32 * (8 * z + 2 * x + 1)];
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    h += (int64_t)__float2int_rn(c[z][w][x]) * (1 << 8 * (3 - w));
+                    l += (int64_t)__float2int_rn(c[z][4 + w][x]) * (1 << 8 * (3 - w));
+                }
+                sum[32 * (8 * z + 2 * x)] = h;
+                sum[32 * (8 * z + 2 * x + 1)] = l;
+            }
+        clear();
+    }
+    // the chunks 0 .. nch - 1 that stage(c) copies (one commit each, also past the end); every thread calls it
+    template <class Stage, class RE, class CE>
+    __device__ __forceinline__ void run(int nch, int rows, Stage &&stage, RE &&re, CE &&ce)
+    {
+        stage(0);
+        stage(1);
+        for (int ch = 0; ch < nch; ++ch) {
+            if (NARROW && ch) asm volatile("cp.async.wait_group 0;\n" ::: "memory");   // its stage was the last one
+            else asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+            __syncthreads();   // chunk ch has landed, the digits of the one before are consumed
+            split(ch, rows, re, ce);
+            __syncthreads();   // its raw buffer is free, the digits are there
+            if (NARROW) {   // the raw coefficients are still read: the next barrier frees them
+                if (ch) stage(ch + 1);
+                if (row0() < rows) multiply_own(ch, re);
+            } else {
+                stage(ch + 2);
+                if (row0() < rows) multiply();
+            }
+        }
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        __syncthreads();
+    }
+    // put(row, column, value) for the outputs of the warp (rows, columns of the CTA); whole warps call it
+    template <class RE, class CE, class Put>
+    __device__ __forceinline__ void store(int rows, int nrhs, RE &&re, CE &&ce, Put &&put)
+    {
+        if (row0() >= rows) return;
+        fold();
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const int row = row0() + (lane >> 2) + 8 * (x >> 1), col = col0() + 2 * (lane & 3) + (x & 1);
+            int64_t v[2][2];
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                v[0][p] = sum[32 * (2 * x + p)];
+                v[1][p] = sum[32 * (8 + 2 * x + p)];
+                if (NARROW) {   // real x real, real x imaginary two lanes on; imaginary x the same
+                    const int64_t r2 = __shfl_down_sync(0xffffffffu, v[0][p], 2), i2 = __shfl_down_sync(0xffffffffu, v[1][p], 2);
+                    v[0][p] -= i2;
+                    v[1][p] += r2;
+                }
+            }
+            if (row >= rows || col >= nrhs) continue;
+            const int ea = re(row), eb = ce(col), e = ea + eb - 2112, eh = e / 2;
+            double2 y = make_double2(nan(""), nan(""));
+            if (ea != 0x7ff && eb != 0x7ff) {   // in two steps: 2^e alone may be below the smallest power of two
+                const double s0 = __hiloint2double(eh + 1023 << 20, 0), s1 = __hiloint2double(e - eh + 1023 << 20, 0);
+                y.x = fma((double)v[0][0], 4294967296.0, (double)v[0][1]) * s0 * s1;
+                y.y = fma((double)v[1][0], 4294967296.0, (double)v[1][1]) * s0 * s1;
+            }
+            put(row, col, y);
+        }
+    }
+};
+
+// a staged vector entry, zero past the contraction's end
+__device__ __forceinline__ void oz_cp(double2 *dst, const double2 *src, bool ok)
 {
-    extern __shared__ unsigned char smraw[];
-    __shared__ int s_item[64], s_l[64];
+    if (ok) far_cp(dst, src);
+    else *dst = make_double2(0.0, 0.0);
+}
+
+// phase 1, tasks as in k_far_t, blockIdx.y: which 32 of its factor columns; rexp: exponents of the factor columns, of V
+// (tlen), then of U; cexp: of the columns of u (read), then of t and s (written)
+template <bool NARROW>
+__global__ void __launch_bounds__(NARROW ? 64 : 128, NARROW ? 6 : 3) k_far_t64(const int *task_lo, const int *task_hi, const int *task_ptr,
+                                                    const int64_t *item_off, const int *item_ld, const int *item_rank,
+                                                    const int *item_row, const int *item_isv, const double2 *U,
+                                                    const double2 *V, const double2 *u, int nrhs, double2 *t, double2 *s,
+                                                    const int *rexp, int64_t tlen, int *cexp)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ int s_item[64], s_l[64], s_cmax[16], s_re[OZ_ROWS], s_ce[16];
     __shared__ const double2 *s_src[64];
-    const int task = blockIdx.x;
+    const int task = blockIdx.x, f0 = OZ_ROWS * blockIdx.y;
     const int lo = task_lo[task], hi = task_hi[task], i0 = task_ptr[task], i1 = task_ptr[task + 1];
-    const int R = far_items(i0, i1, item_off, item_ld, item_rank, item_isv, U, V, s_item, s_l, s_src), len = R * nrhs, ldw = R | 1;
-    double2 *const bufs[2] = {(double2 *)smraw, (double2 *)smraw + half};
-    double2 acc[NU];
-#pragma unroll
-    for (int q = 0; q < NU; ++q) acc[q] = make_double2(0.0, 0.0);
-    auto stage = [&](int c0, int which) {   // as in k_far_t: Ws[qq * ldw + rr], then Ys[qq * nrhs + r]
-        const int ch = min(FAR_T1, hi - c0);
-        double2 *Ws = bufs[which], *Ys = Ws + ch * ldw;
-        for (int rr = threadIdx.x / FAR_T1; rr < R; rr += F64_T / FAR_T1) {
-            const int qq = threadIdx.x % FAR_T1;
-            if (qq < ch) far_cp(Ws + qq * ldw + rr, s_src[rr] + (c0 - lo + qq));
+    const int R = far_items(i0, i1, item_off, item_ld, item_rank, item_isv, U, V, s_item, s_l, s_src) - f0;
+    if (R <= 0) return;
+    const int rows = min(R, OZ_ROWS);
+    auto dest = [&](int row) {
+        const int it = s_item[f0 + row];
+        return (item_isv[it] ? 0 : tlen) + item_row[it] + s_l[f0 + row];
+    };
+    if (threadIdx.x < 16) {
+        s_cmax[threadIdx.x] = 0;
+        s_ce[threadIdx.x] = threadIdx.x < nrhs ? cexp[threadIdx.x] : 64;
+    }
+    if (threadIdx.x < OZ_ROWS) s_re[threadIdx.x] = threadIdx.x < rows ? rexp[dest(threadIdx.x)] : 64;
+    Oz<NARROW> oz(smraw, nrhs);
+    const int nch = (hi - lo + OZ_KC - 1) / OZ_KC;
+    auto stage = [&](int c) {   // factor column rr of row c0 + qq, half a warp each; then the vector rows
+        if (c < nch) {
+            const int c0 = lo + c * OZ_KC, ch = min(OZ_KC, hi - c0), qh = oz.lane & 15;
+            double2 *Ws = oz.ws(c), *Ys = oz.ys(c);
+            if (qh < ch)
+                for (int rr = 2 * oz.wp + (oz.lane >> 4); rr < rows; rr += 2 * oz.nw)
+                    far_cp(Ws + qh * oz.ldw + rr, s_src[f0 + rr] + (c0 - lo + qh));
+            const double2 *uc = u + (int64_t)c0 * nrhs;
+            if (NARROW) {
+                const int qq = threadIdx.x >> 2, r = threadIdx.x & 3;   // 64 threads, 16 rows of at most 4
+                if (r < nrhs) oz_cp(Ys + qq * oz.ldr + r, uc + qq * nrhs + r, qq < ch);
+            } else
+                for (int qq = oz.wp; qq < OZ_KC; qq += oz.nw)
+                    if (oz.lane < nrhs) oz_cp(Ys + qq * oz.ldr + oz.lane, uc + qq * nrhs + oz.lane, qq < ch);
         }
-        const double2 *uc = u + (int64_t)c0 * nrhs;
-        for (int e = threadIdx.x; e < ch * nrhs; e += F64_T) far_cp(Ys + e, uc + e);
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
-    if (lo < hi) stage(lo, 0);
-    for (int c0 = lo, it = 0; c0 < hi; c0 += FAR_T1, ++it) {
-        const int ch = min(FAR_T1, hi - c0);
-        if (c0 + FAR_T1 < hi) {
-            stage(c0 + FAR_T1, (it + 1) & 1);
-            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-        } else
-            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-        __syncthreads();
-        const double2 *Ws = bufs[it & 1];
-        f64_mac<NU>(acc, Ws, ldw, Ws + ch * ldw, nrhs, c0 - lo, ch, R, len);
-        __syncthreads();
-    }
-    f64_reduce<NU>(acc, (double2 *)smraw, len, [&](int e, double2 v) {
-        const int rr = e % R, r = e / R, it = s_item[rr];
-        (item_isv[it] ? t : s)[(int64_t)(item_row[it] + s_l[rr]) * nrhs + r] = v;
+    auto re = [&](int row) { return s_re[row]; };
+    auto ce = [&](int col) { return s_ce[col]; };
+    oz.run(nch, rows, stage, re, ce);
+    oz.store(rows, nrhs, re, ce, [&](int row, int col, double2 v) {
+        const int64_t d = dest(row);
+        (d < tlen ? t + d * nrhs : s + (d - tlen) * nrhs)[col] = v;
+        atomicMax(&s_cmax[col], oz_exp(v));
     });
+    __syncthreads();
+    if (threadIdx.x < nrhs) atomicMax(&cexp[16 + threadIdx.x], s_cmax[threadIdx.x]);
+}
+
+// exponents of the factor columns (see k_far_t64): task as there, one warp per factor column
+__global__ void k_far_rexp1(const int *task_lo, const int *task_hi, const int *task_ptr, const int64_t *item_off,
+                            const int *item_ld, const int *item_rank, const int *item_row, const int *item_isv,
+                            const double2 *U, const double2 *V, int *rexp, int64_t tlen)
+{
+    __shared__ int s_item[64], s_l[64];
+    __shared__ const double2 *s_src[64];
+    const int task = blockIdx.x, lane = threadIdx.x & 31;
+    const int R = far_items(task_ptr[task], task_ptr[task + 1], item_off, item_ld, item_rank, item_isv, U, V, s_item, s_l, s_src);
+    for (int rr = threadIdx.x >> 5; rr < R; rr += blockDim.x >> 5) {
+        int e = 0;
+        for (int q = lane; q < task_hi[task] - task_lo[task]; q += 32) e = max(e, oz_exp(s_src[rr][q]));
+        e = __reduce_max_sync(0xffffffffu, e);
+        const int it = s_item[rr];
+        if (lane == 0) rexp[(item_isv[it] ? 0 : tlen) + item_row[it] + s_l[rr]] = e;
+    }
+}
+// exponents of the coefficient rows of a leaf (one CTA): over its far segments (F0 = U, F1 = V) or its near ones
+__global__ void k_far_rexp2(const int *leaf_ptr, const int *part_ptr, const FarSegD *segs, const double2 *F0,
+                            const double2 *F1, int *rexp)
+{
+    __shared__ int s_e[64];
+    const int l = blockIdx.x, a = leaf_ptr[l], ni = leaf_ptr[l + 1] - a, i = threadIdx.x & 63;
+    if (threadIdx.x < 64) s_e[threadIdx.x] = 0;
+    __syncthreads();
+    int e = 0;
+    for (int q = part_ptr[l * FAR_PARTS]; q < part_ptr[(l + 1) * FAR_PARTS] && i < ni; ++q) {
+        const FarSegD g = segs[q];
+        const double2 *F = ((g.src & 1) ? F1 : F0) + g.foff + (int64_t)i * g.fi;
+        for (int kk = threadIdx.x >> 6; kk < g.len; kk += blockDim.x >> 6) e = max(e, oz_exp(F[(int64_t)kk * g.fk]));
+    }
+    atomicMax(&s_e[i], e);
+    __syncthreads();
+    if (threadIdx.x < ni) rexp[a + threadIdx.x] = s_e[threadIdx.x];
+}
+// u[i * nrhs + r] = x[idx[i] + r * n] and the exponents of its columns, cexp[r] (cexp is zero before)
+__global__ void k_far_gather64(int n, int nrhs, const int *idx, const double2 *x, double2 *u, int *cexp)
+{
+    __shared__ int s_e[16];
+    if (threadIdx.x < 16) s_e[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e < (int64_t)n * nrhs) {
+        const int i = (int)(e / nrhs), r = (int)(e - (int64_t)i * nrhs);
+        const double2 v = x[idx[i] + (int64_t)r * n];
+        u[e] = v;
+        atomicMax(&s_e[r], oz_exp(v));
+    }
+    __syncthreads();
+    if (threadIdx.x < nrhs) atomicMax(&cexp[threadIdx.x], s_e[threadIdx.x]);
 }
 
 // Phase 2: one CTA per leaf over the leaf's segments (FarSegD, list order, len <= 32).
@@ -526,96 +799,89 @@ __global__ void __launch_bounds__(256) k_far_y32(int nl, const int *leaf_ptr, co
         }
 }
 
-// complex FP64, phase 2 (see f64_mac): the segments of the far list and, with nearp, those of the leaf's
-// near-field blocks (zpart / zkcum / zsegs), which gives Z u in one pass
-template <int NU>
-__global__ void __launch_bounds__(F64_T) k_far_y64(int nl, const int *leaf_ptr, const int *part_ptr, const int *kcum,
-                                                   const FarSegD *segs, const int *zpart, const int *zkcum,
-                                                   const FarSegD *zsegs, const double2 *U, const double2 *V,
-                                                   const double2 *nearp, const double2 *t, const double2 *s,
-                                                   const double2 *u, const int *cl2new, int n, int nrhs, double2 *part,
-                                                   int half)
+// complex FP64, phase 2: the segments of the far list and, with nearp, those of the leaf's near-field blocks (zpart /
+// zkcum / zsegs), which gives Z u in one pass; blockIdx.y: which 32 of the leaf's rows; rexp: exponents of the far rows (n),
+// then of the near rows
+template <bool NARROW>
+__global__ void __launch_bounds__(NARROW ? 64 : 128, NARROW ? 6 : 3) k_far_y64(int nl, const int *leaf_ptr, const int *part_ptr, const int *kcum,
+                                                    const FarSegD *segs, const int *zpart, const int *zkcum,
+                                                    const FarSegD *zsegs, const double2 *U, const double2 *V,
+                                                    const double2 *nearp, const double2 *t, const double2 *s,
+                                                    const double2 *u, const int *cl2new, int n, int nrhs, double2 *part,
+                                                    const int *rexp, const int *cexp)
 {
-    extern __shared__ unsigned char smraw[];
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ int s_re[OZ_ROWS], s_ce[16];
     const int l = blockIdx.x / FAR_PARTS, pp = blockIdx.x % FAR_PARTS;
     if (l >= nl) return;
-    const int a = leaf_ptr[l], ni = leaf_ptr[l + 1] - a, len = ni * nrhs, ldw = ni | 1;
-    const int kmax = half / (ldw + nrhs);   // >= 32
-    double2 *const bufs[2] = {(double2 *)smraw, (double2 *)smraw + half};
-    double2 acc[NU];
-#pragma unroll
-    for (int q = 0; q < NU; ++q) acc[q] = make_double2(0.0, 0.0);
+    const int r0 = OZ_ROWS * blockIdx.y, a = leaf_ptr[l] + r0, rows = min(leaf_ptr[l + 1] - a, OZ_ROWS);
+    if (rows <= 0) return;
+    if (threadIdx.x < OZ_ROWS) {
+        int e = 64;
+        if (threadIdx.x < rows) e = nearp ? max(rexp[a + threadIdx.x], rexp[n + a + threadIdx.x]) : rexp[a + threadIdx.x];
+        s_re[threadIdx.x] = e;
+    }
+    if (threadIdx.x < 16) s_ce[threadIdx.x] = threadIdx.x < nrhs ? max(cexp[threadIdx.x], cexp[16 + threadIdx.x]) : 64;
+    Oz<NARROW> oz(smraw, nrhs);
+    auto re = [&](int row) { return s_re[row]; };
+    auto ce = [&](int col) { return s_ce[col]; };
     for (int tab = 0; tab < (nearp ? 2 : 1); ++tab) {
-        const int *pt = tab ? zpart : part_ptr, *kc = tab ? zkcum : kcum;
+        const int *kc = tab ? zkcum : kcum;
         const FarSegD *sg = tab ? zsegs : segs;
         const double2 *F0 = tab ? nearp : U, *F1 = tab ? nearp : V;
-        const int w1 = pt[blockIdx.x + 1];
-        auto chunk_count = [&](int p) {   // segments from p on whose stacked length fits kmax
-            const int q = p + threadIdx.x;
-            return __syncthreads_count(q < w1 && kc[q + 1] - kc[p] <= kmax);
-        };
-        auto stage = [&](int p, int cnt, double2 *buf) {   // as in k_far_y
-            const int k0 = kc[p], klen = kc[p + cnt] - k0;
-            double2 *Wst = buf, *Yst = buf + kmax * ldw;
-            int q = -1, qlo = 0, qhi = 0;
-            const double2 *F = nullptr;
-            int64_t fi = 0, fk = 0;
-            for (int e = threadIdx.x; e < klen * ni; e += F64_T) {
-                const int kk = e / ni, i = e - kk * ni;
-                while (kk >= qhi) {
-                    ++q;
-                    qlo = kc[p + q] - k0;
-                    qhi = kc[p + q + 1] - k0;
-                    const FarSegD g = sg[p + q];
-                    F = ((g.src & 1) ? F1 : F0) + g.foff;
-                    fi = g.fi;
-                    fk = g.fk;
+        const int p0 = (tab ? zpart : part_ptr)[blockIdx.x], w1 = (tab ? zpart : part_ptr)[blockIdx.x + 1];
+        const int k0 = p0 < w1 ? kc[p0] : 0, K = p0 < w1 ? kc[w1] - k0 : 0, nch = (K + OZ_KC - 1) / OZ_KC;
+        // lane o and o + 16 of every warp follow contraction entry o of the chunks through the segments, with the next
+        // segment's descriptor on its way
+        int q = p0, qlo = 0, qhi = 0, hn = 0;
+        FarSegD gn = {};
+        if (K > 0) {
+            gn = sg[p0];
+            hn = kc[p0 + 1] - k0;
+        }
+        const double2 *F = nullptr, *Yb = nullptr;
+        int fi = 0, fk = 0;
+        auto stage = [&](int c) {
+            if (c < nch) {
+                double2 *Ws = oz.ws(c), *Ys = oz.ys(c);
+                const int o = oz.lane & 15, kk = c * OZ_KC + o;
+                while (kk < K && kk >= qhi) {
+                    F = ((gn.src & 1) ? F1 : F0) + gn.foff + (int64_t)r0 * gn.fi;
+                    const int ys = gn.src >> 1;
+                    Yb = (ys == 0 ? t : (ys == 1 ? s : u)) + gn.yrow * nrhs;
+                    fi = gn.fi;
+                    fk = gn.fk;
+                    qlo = qhi;
+                    qhi = hn;
+                    if (++q < w1) {
+                        gn = sg[q];
+                        hn = kc[q + 1] - k0;
+                    }
                 }
-                cp_async_el(Wst + kk * ldw + i, F + (int64_t)i * fi + (int64_t)(kk - qlo) * fk);
-            }
-            q = -1;
-            qhi = 0;
-            const double2 *Yb = nullptr;
-            for (int e = threadIdx.x; e < klen * nrhs; e += F64_T) {
-                const int kk = e / nrhs, r = e - kk * nrhs;
-                while (kk >= qhi) {
-                    ++q;
-                    qlo = kc[p + q] - k0;
-                    qhi = kc[p + q + 1] - k0;
-                    const FarSegD g = sg[p + q];
-                    const int ys = g.src >> 1;
-                    Yb = (ys == 0 ? t : (ys == 1 ? s : u)) + g.yrow * nrhs;
+                const bool in = kk < K;
+                const uint64_t f = in ? (uint64_t)(F + (int64_t)(kk - qlo) * fk) : 0, y = (uint64_t)(Yb + (int64_t)(kk - qlo) * nrhs);
+#pragma unroll 4
+                for (int x = oz.wp; x < OZ_KC; x += oz.nw) {
+                    const double2 *fx = (const double2 *)__shfl_sync(0xffffffffu, f, x);
+                    const int fix = __shfl_sync(0xffffffffu, fi, x);
+                    if (fx && oz.lane < rows) far_cp(Ws + x * oz.ldw + oz.lane, fx + (int64_t)oz.lane * fix);
                 }
-                cp_async_el(Yst + e, Yb + (int64_t)(kk - qlo) * nrhs + r);
+                if (NARROW) {
+                    for (int r = 2 * oz.wp + (oz.lane >> 4); r < nrhs; r += 2 * oz.nw)
+                        oz_cp(Ys + o * oz.ldr + r, (const double2 *)y + r, in);
+                } else
+#pragma unroll 4
+                    for (int x = oz.wp; x < OZ_KC; x += oz.nw) {
+                        const double2 *yx = (const double2 *)__shfl_sync(0xffffffffu, y, x);
+                        if (oz.lane < nrhs) oz_cp(Ys + x * oz.ldr + oz.lane, yx + oz.lane, c * OZ_KC + x < K);
+                    }
             }
             cp_async_commit();
-            return klen;
         };
-        const int p0 = pt[blockIdx.x];
-        int p = p0;
-        if (p >= w1) continue;
-        int cnt = chunk_count(p), klen = stage(p, cnt, bufs[0]);
-        for (int it = 0;; ++it) {
-            const int pn = p + cnt;
-            int cntn = 0, klenn = 0;
-            if (pn < w1) {
-                cntn = chunk_count(pn);
-                klenn = stage(pn, cntn, bufs[(it + 1) & 1]);
-                cp_async_wait<1>();
-            } else
-                cp_async_wait<0>();
-            __syncthreads();
-            const double2 *buf = bufs[it & 1];
-            f64_mac<NU>(acc, buf, ldw, buf + kmax * ldw, nrhs, kc[p] - kc[p0], klen, ni, len);
-            __syncthreads();
-            if (pn >= w1) break;
-            p = pn;
-            cnt = cntn;
-            klen = klenn;
-        }
+        oz.run(nch, rows, stage, re, ce);
     }
-    double2 *out = part + (size_t)pp * n * nrhs + cl2new[a];
-    f64_reduce<NU>(acc, (double2 *)smraw, len, [&](int e, double2 v) { out[e % ni + (int64_t)(e / ni) * n] = v; });
+    double2 *out = part + (size_t)pp * n * nrhs + cl2new[leaf_ptr[l]] + r0;
+    oz.store(rows, nrhs, re, ce, [&](int row, int col, double2 v) { out[row + (int64_t)col * n] = v; });
 }
 
 // ---- complex FP32 on the tensor cores ------------------------------------------------------
@@ -823,9 +1089,11 @@ __global__ void __launch_bounds__(256, 2) k_far_y_tc(int nl, const int *leaf_ptr
 }
 
 // y = sum of the FAR_PARTS partial products, added in part order
-template <class T> __global__ void k_far_sum(int64_t len, const T *part, T *y)
+// (the column exponents of the FP64 product are cleared here, for its next call)
+template <class T> __global__ void k_far_sum(int64_t len, const T *part, T *y, int *cexp = nullptr)
 {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (cexp && e < 32) cexp[e] = 0;
     if (e >= len) return;
     T v = part[e];
     for (int p = 1; p < FAR_PARTS; ++p) {
@@ -908,49 +1176,68 @@ static cudaError_t far_tc_launch(hm_ctx *h, const float2 *U, const float2 *V, fl
     return cudaGetLastError();
 }
 
-// complex FP64: y = Z_F u, or Z u with the near-field segments.  NU: outputs per lane of the largest block (64 rank
-// rows in phase 1, the largest leaf in phase 2).
-template <int NT, int NY>
-static cudaError_t far64_run(hm_ctx *h, const double2 *U, const double2 *V, double2 *t, double2 *s, const double2 *ucl,
-                             double2 *y, int nrhs, bool near)
+// exponents of the coefficient rows for the FP64 products, once per handle (h->d_rexp: V columns, U columns, far rows,
+// near rows)
+cudaError_t far64_prepare(hm_ctx *h)
 {
     const FarPlan &F = h->fplan;
-    const int n = h->plan.n, maxn = h->max_leaf;
-    const int ht = std::max(FAR_T1 * (65 + nrhs), (F64_NK * 64 * nrhs + 1) / 2);
-    const int hy = std::max(32 * ((maxn | 1) + nrhs), (F64_NK * maxn * nrhs + 1) / 2);
-    static DeviceOnce attr;
-    if (attr.need()) {   // nrhs <= 16, blocks of up to 64 rows
-        const int smax = (int)(sizeof(double2) * 2 * 32 * (65 + 16));
-        cudaError_t e;
-        if ((e = cudaFuncSetAttribute(k_far_t64<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax)) ||
-            (e = cudaFuncSetAttribute(k_far_y64<NY>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax)))
-            return e;
-        attr.done();
-    }
+    const int64_t tlen = F.tlen, n = h->n;
+    cudaError_t e;
+    if ((e = h->arena.alloc((void **)&h->d_rexp, sizeof(int) * (size_t)(2 * tlen + 2 * n + 32)))) return e;
+    h->d_cexp = h->d_rexp + 2 * tlen + 2 * n;
+    if ((e = cudaMemsetAsync(h->d_rexp, 0, sizeof(int) * (size_t)(2 * tlen + 2 * n + 32), h->stream))) return e;
     const int ntask = (int)F.p1_lo.size();
     if (ntask > 0)
-        HM_LAUNCH(h, K_FAR1,
-                  k_far_t64<NT><<<ntask, F64_T, sizeof(double2) * 2 * ht, h->stream>>>(
-                      h->d_p1_lo, h->d_p1_hi, h->d_p1_ptr, h->d_p1_off, h->d_p1_ld, h->d_p1_rank, h->d_p1_row,
-                      h->d_p1_isv, U, V, ucl, nrhs, t, s, ht));
-    double2 *part = (double2 *)h->d_farpart;
-    HM_LAUNCH(h, K_FAR2,
-              k_far_y64<NY><<<h->nl * FAR_PARTS, F64_T, sizeof(double2) * 2 * hy, h->stream>>>(
-                  h->nl, h->d_leaf_ptr, h->d_part_ptr, h->d_seg_kcum, h->d_segs, h->d_zpart, h->d_zkcum, h->d_zsegs, U, V,
-                  near ? h->d_near : nullptr, t, s, ucl, h->d_cl2new, n, nrhs, part, hy));
-    const int64_t len = (int64_t)n * nrhs;
-    HM_LAUNCH(h, K_FAR2, k_far_sum<double2><<<nblk(len, 256), 256, 0, h->stream>>>(len, part, y));
+        k_far_rexp1<<<ntask, 256, 0, h->stream>>>(h->d_p1_lo, h->d_p1_hi, h->d_p1_ptr, h->d_p1_off, h->d_p1_ld, h->d_p1_rank,
+                                                  h->d_p1_row, h->d_p1_isv, h->d_farU, h->d_farV, h->d_rexp, tlen);
+    k_far_rexp2<<<h->nl, 256, 0, h->stream>>>(h->d_leaf_ptr, h->d_part_ptr, h->d_segs, h->d_farU, h->d_farV,
+                                           h->d_rexp + 2 * tlen);
+    k_far_rexp2<<<h->nl, 256, 0, h->stream>>>(h->d_leaf_ptr, h->d_zpart, h->d_zsegs, h->d_near, h->d_near,
+                                              h->d_rexp + 2 * tlen + n);
     return cudaGetLastError();
 }
 
-cudaError_t far_product64(hm_ctx *h, const double2 *U, const double2 *V, double2 *t, double2 *s, const double2 *ucl,
-                          double2 *y, int nrhs, bool near)
+template <bool NARROW>
+static cudaError_t far64_run(hm_ctx *h, const double2 *U, const double2 *V, double2 *t, double2 *s, const double2 *x,
+                             double2 *u, double2 *y, int nrhs, bool near)
+{
+    const FarPlan &F = h->fplan;
+    const int n = h->plan.n, threads = 64 * Oz<NARROW>::tiles(nrhs);
+    const size_t smem = Oz<NARROW>::smem(nrhs);
+    const int64_t len = (int64_t)n * nrhs;
+    static DeviceOnce attr;
+    cudaError_t e;
+    if (attr.need()) {
+        const int smax = (int)Oz<NARROW>::smem(16);
+        if ((e = cudaFuncSetAttribute(k_far_t64<NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax)) ||
+            (e = cudaFuncSetAttribute(k_far_y64<NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax)))
+            return e;
+        attr.done();
+    }
+    HM_LAUNCH(h, K_PERMUTE, k_far_gather64<<<nblk(len, 256), 256, 0, h->stream>>>(n, nrhs, h->d_cl2new, x, u, h->d_cexp));
+    const int ntask = (int)F.p1_lo.size();
+    if (ntask > 0)
+        HM_LAUNCH(h, K_FAR1,
+                  k_far_t64<NARROW><<<dim3(ntask, 64 / OZ_ROWS), threads, smem, h->stream>>>(
+                      h->d_p1_lo, h->d_p1_hi, h->d_p1_ptr, h->d_p1_off, h->d_p1_ld, h->d_p1_rank, h->d_p1_row,
+                      h->d_p1_isv, U, V, u, nrhs, t, s, h->d_rexp, F.tlen, h->d_cexp));
+    double2 *part = (double2 *)h->d_farpart;
+    HM_LAUNCH(h, K_FAR2,
+              k_far_y64<NARROW><<<dim3(h->nl * FAR_PARTS, (h->max_leaf + OZ_ROWS - 1) / OZ_ROWS), threads, smem, h->stream>>>(
+                  h->nl, h->d_leaf_ptr, h->d_part_ptr, h->d_seg_kcum, h->d_segs, h->d_zpart, h->d_zkcum, h->d_zsegs, U, V,
+                  near ? h->d_near : nullptr, t, s, u, h->d_cl2new, n, nrhs, part, h->d_rexp + 2 * F.tlen, h->d_cexp));
+    HM_LAUNCH(h, K_FAR2, k_far_sum<double2><<<nblk(len, 256), 256, 0, h->stream>>>(len, part, y, h->d_cexp));
+    return cudaGetLastError();
+}
+
+// complex FP64: y = Z_F x, or Z x with the near-field segments, x and y in solve order; at most 16 columns; u: n x nrhs
+// entries of scratch
+cudaError_t far_product64(hm_ctx *h, const double2 *U, const double2 *V, double2 *t, double2 *s, const double2 *x,
+                          double2 *u, double2 *y, int nrhs, bool near)
 {
     h->prof.cols[K_FAR1] += nrhs;
     h->prof.cols[K_FAR2] += nrhs;
-    if (nrhs <= 4) return far64_run<4, 4>(h, U, V, t, s, ucl, y, nrhs, near);
-    if (h->max_leaf <= 32) return far64_run<16, 8>(h, U, V, t, s, ucl, y, nrhs, near);
-    return far64_run<16, 16>(h, U, V, t, s, ucl, y, nrhs, near);
+    return nrhs <= 4 ? far64_run<true>(h, U, V, t, s, x, u, y, nrhs, near) : far64_run<false>(h, U, V, t, s, x, u, y, nrhs, near);
 }
 
 // complex FP32, 17 to 64 columns

@@ -203,6 +203,7 @@ struct hm_ctx {
     hm::FarSegD *d_segs = nullptr, *d_zsegs = nullptr;
     int *d_zpart = nullptr, *d_zkcum = nullptr;
     int max_leaf = 0;
+    int *d_rexp = nullptr, *d_cexp = nullptr;   // exponents for the split FP64 products (far.cu); d_cexp in d_rexp's allocation
     int *d_leaf_ptr = nullptr, *d_perm = nullptr;
     int *d_new2cl = nullptr, *d_cl2new = nullptr, *d_new2orig = nullptr, *d_pos = nullptr;
     // device: plan
@@ -324,8 +325,9 @@ cudaError_t make_fp32_copies(hm_ctx *h);
 cudaError_t to_solve_order(hm_ctx *h, const double2 *src, int64_t lds, double2 *dst, int nrhs);
 cudaError_t to_orig_order(hm_ctx *h, const double2 *src, double2 *dst, int64_t ldd, int nrhs);
 cudaError_t z_apply_orig(hm_ctx *h, const double2 *x, double2 *y, int nrhs);
-cudaError_t far_product64(hm_ctx *h, const double2 *U, const double2 *V, double2 *t, double2 *s, const double2 *ucl,
-                          double2 *y, int nrhs, bool near);   // near: Z_F + Z_N
+cudaError_t far64_prepare(hm_ctx *h);
+cudaError_t far_product64(hm_ctx *h, const double2 *U, const double2 *V, double2 *t, double2 *s, const double2 *x,
+                          double2 *u, double2 *y, int nrhs, bool near);   // near: Z_F + Z_N
 cudaError_t far_product32(hm_ctx *h, const float2 *U, const float2 *V, float2 *t, float2 *s, const float2 *ucl, float2 *y,
                           int nrhs);
 cudaError_t ensure_solve_workspace(hm_ctx *h, int nrhs);

@@ -1526,11 +1526,14 @@ static cudaError_t sweep(hm_ctx *h, const OpData<T> &d, bool forward, const T *x
 template <class T>
 static cudaError_t far_apply(hm_ctx *h, const OpData<T> &d, const T *x, T *y, int nrhs, T *ucl, bool near = false)
 {
-    const int n = h->plan.n;
-    HM_LAUNCH(h, K_PERMUTE, k_gather_il<T><<<nblk((int64_t)n * nrhs, 256), 256, 0, h->stream>>>(n, nrhs, h->d_cl2new, x,
-                                                                                            ucl));
-    if constexpr (sizeof(T) == 16) return far_product64(h, d.U, d.V, d.t, d.s, ucl, y, nrhs, near);
-    else return far_product32(h, d.U, d.V, d.t, d.s, ucl, y, nrhs);
+    if constexpr (sizeof(T) == 16) {
+        return far_product64(h, d.U, d.V, d.t, d.s, x, ucl, y, nrhs, near);
+    } else {
+        const int n = h->plan.n;
+        HM_LAUNCH(h, K_PERMUTE, k_gather_il<T><<<nblk((int64_t)n * nrhs, 256), 256, 0, h->stream>>>(n, nrhs, h->d_cl2new,
+                                                                                                x, ucl));
+        return far_product32(h, d.U, d.V, d.t, d.s, ucl, y, nrhs);
+    }
 }
 
 template <class T>

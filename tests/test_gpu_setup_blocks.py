@@ -157,3 +157,33 @@ def test_far_field_widths(sizes):
         assert np.array_equal(y, ref[:w])
     want = X @ F.T
     assert np.max(np.abs(ref - want)) <= 1e-5 * np.max(np.abs(want))
+
+
+def apply_z(h, X):
+    x = torch.from_numpy(X).cuda()
+    y = torch.empty_like(x)
+    torch.cuda.synchronize()
+    hm.hm_apply(h, H.OP_Z, x, y)
+    torch.cuda.synchronize()
+    return y.cpu().numpy()
+
+
+@pytest.mark.parametrize("w", [1, 4, 5, 16])
+def test_split_product_scales_exactly_and_keeps_columns_apart(w):
+    """The digits of a column follow its largest exponent: a power of two in front comes out exactly, also far from 1, and a
+    NaN or an infinity spoils its own column only."""
+    P, _, Z = problem(MIXED, 11)
+    h = hm.hmat_create(P, ordering=1)
+    rng = np.random.default_rng(4)
+    X = rng.standard_normal((w, P.n)) + 1j * rng.standard_normal((w, P.n))
+    y = apply_z(h, X)
+    for k in (-600, -60, 60, 600):
+        assert np.array_equal(apply_z(h, np.ldexp(X.real, k) + 1j * np.ldexp(X.imag, k)),
+                              np.ldexp(y.real, k) + 1j * np.ldexp(y.imag, k))
+    assert np.all(apply_z(h, 0 * X) == 0)
+    for bad in (np.nan, np.inf):
+        B = X.copy()
+        B[w - 1, 7] = bad
+        z = apply_z(h, B)
+        assert np.array_equal(z[:w - 1], y[:w - 1]) and not np.any(np.isfinite(z[w - 1].real))
+    assert np.array_equal(apply_z(h, X), y)
