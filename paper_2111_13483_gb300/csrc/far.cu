@@ -471,7 +471,7 @@ __global__ void k_far_rexp1(const int *task_lo, const int *task_hi, const int *t
     const int task = blockIdx.x, lane = threadIdx.x & 31;
     const int R = far_items(task_ptr[task], task_ptr[task + 1], item_off, item_ld, item_rank, item_isv, U, V, s_item, s_l, s_src);
     for (int rr = threadIdx.x >> 5; rr < R; rr += blockDim.x >> 5) {
-        int e = 0;
+        int e = 64;
         for (int q = lane; q < task_hi[task] - task_lo[task]; q += 32) e = max(e, oz_exp(s_src[rr][q]));
         e = __reduce_max_sync(0xffffffffu, e);
         const int it = s_item[rr];
@@ -484,9 +484,9 @@ __global__ void k_far_rexp2(const int *leaf_ptr, const int *part_ptr, const FarS
 {
     __shared__ int s_e[64];
     const int l = blockIdx.x, a = leaf_ptr[l], ni = leaf_ptr[l + 1] - a, i = threadIdx.x & 63;
-    if (threadIdx.x < 64) s_e[threadIdx.x] = 0;
+    if (threadIdx.x < 64) s_e[threadIdx.x] = 64;   // a leaf without segments: the smallest exponent
     __syncthreads();
-    int e = 0;
+    int e = 64;
     for (int q = part_ptr[l * FAR_PARTS]; q < part_ptr[(l + 1) * FAR_PARTS] && i < ni; ++q) {
         const FarSegD g = segs[q];
         const double2 *F = ((g.src & 1) ? F1 : F0) + g.foff + (int64_t)i * g.fi;

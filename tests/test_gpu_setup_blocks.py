@@ -159,11 +159,11 @@ def test_far_field_widths(sizes):
     assert np.max(np.abs(ref - want)) <= 1e-5 * np.max(np.abs(want))
 
 
-def apply_z(h, X):
+def apply_z(h, X, op=H.OP_Z):
     x = torch.from_numpy(X).cuda()
     y = torch.empty_like(x)
     torch.cuda.synchronize()
-    hm.hm_apply(h, H.OP_Z, x, y)
+    hm.hm_apply(h, op, x, y)
     torch.cuda.synchronize()
     return y.cpu().numpy()
 
@@ -187,3 +187,19 @@ def test_split_product_scales_exactly_and_keeps_columns_apart(w):
         z = apply_z(h, B)
         assert np.array_equal(z[:w - 1], y[:w - 1]) and not np.any(np.isfinite(z[w - 1].real))
     assert np.array_equal(apply_z(h, X), y)
+
+
+@pytest.mark.parametrize("w", [1, 16])
+def test_split_product_of_leaves_without_far_blocks(w):
+    """Four leaves, the second of them in no far block but one of rank 0: its rows of the far product are 0, for every
+    size of the vector, zero included."""
+    P, N, Z = problem([33, 1, 64, 2], 11)
+    h = hm.hmat_create(P, ordering=1)
+    rng = np.random.default_rng(4)
+    p = np.asarray(hm.hm_get_index_map(h))
+    row = int(np.argwhere(p == 33)[0, 0])
+    X = rng.standard_normal((w, P.n)) + 1j * rng.standard_normal((w, P.n))
+    for scale in (0.0, 1e-280, 1.0, 1e280):
+        y = apply_z(h, scale * X, H.OP_ZF)
+        assert np.all(np.isfinite(y)) and np.all(y[:, row] == 0)
+        assert scale != 0.0 or np.all(y == 0)
