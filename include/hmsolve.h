@@ -220,6 +220,9 @@ int hm_get_fill_ranks(hm_handle h, int32_t *rank);
  *   op 5: y = Z x          (near + far, ORIGINAL order; the refinement residual operator);
  *   ops 8-12: ops 0-4 with the complex-FP32 factors and arithmetic of the mixed-precision
  *       inner solve (x and y stay complex FP64); precision 1 handles only (else HM_ESTATE).
+ * The FP64 far and near products (ops 0, 3, 5 and the refinement residual) are sums of exact integer digit products
+ * below the largest exponent of each matrix row and vector column, rounded once: a column with an infinity
+ * or a NaN comes out as NaN, the others are not affected.
  * x and y must not overlap.
  */
 int hm_apply(hm_handle h, int32_t op, const void *dx, void *dy, int32_t nrhs);
@@ -233,7 +236,9 @@ int hm_get_index_map(hm_handle h, int32_t *new2orig);
  *   5 backward sweep, 6 far phase 1, 7 far phase 2, 8 block diagonal, 9 permutations,
  *   10 near product, 11 dot products, 12 vector updates, 13 small GMRES kernels,
  *   14 fill-in compression.
- * hm_profile(mode): 1 = also time each launch with CUDA events on the handle's stream,
+ * (Class 10 is part of class 7 now and counts nothing.)
+ * hm_profile(mode): 1 = also time each launch with CUDA events on the handle's stream (a setup then runs all its launches
+ * there, one after the other; otherwise the next pivot block is inverted beside the updates of the one before),
  * 0 = stop timing, 2 = zero all counters.  hm_get_profile returns, for one class, the
  * launches counted, the launches timed and their summed device time in ms.
  */

@@ -137,14 +137,4 @@ template <int SB = 8, class Ld, class St> __device__ __forceinline__ void stage_
     }
 }
 
-// Tile shape for a column count: (1, 1, 1) up to 4 columns, (2, 2, 1) up to 16, (2, 4, 2) up
-// to 64; with 256 threads every output tile of a 64-row block is covered.
-// Dispatches f.template run<TR, TC, NT>(maxw) with maxw the widest count of the shape.
-template <class T, class F> __host__ auto tile_dispatch(int nrhs, F &&f)
-{
-    if (nrhs <= 4) return f.template run<1, 1, 1>(4);
-    if (nrhs <= 16) return f.template run<2, 2, 1>(16);
-    return f.template run<2, 4, 2>(64);
-}
-
 }  // namespace hm
