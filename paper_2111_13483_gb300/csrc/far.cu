@@ -170,11 +170,11 @@ __device__ __forceinline__ void oz_pair(double x0, double x1, int e, uint32_t (&
     const uint32_t sg = __byte_perm((uint32_t)__double2hiint(x0), (uint32_t)__double2hiint(x1), 0x7632) & 0x80008000u;
     const uint32_t one = sg | 0x3c003c00u, off = sg ^ 0xe480e480u;   // +-1, -+1152
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int b = 3 - (i & 3);   // byte of the word
-        const uint32_t p = __byte_perm(i < 4 ? w0.y : w0.x, i < 4 ? w1.y : w1.x, b | b << 4 | (4 + b) << 8 | (4 + b) << 12);
-        const uint32_t q = p & 0x00ff00ffu | 0x64006400u;
-        asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d[i]) : "r"(q), "r"(one), "r"(off));
+    for (int i = 0; i < 8; i += 2) {   // bytes 3, 2 (1, 0) of both words, then each pair between bytes 0x64
+        const uint32_t p = __byte_perm(i < 4 ? w0.y : w0.x, i < 4 ? w1.y : w1.x, i & 2 ? 0x4051 : 0x6273);
+        const uint32_t q0 = __byte_perm(p, 0x64646464u, 0x4140), q1 = __byte_perm(p, 0x64646464u, 0x4342);
+        asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d[i]) : "r"(q0), "r"(one), "r"(off));
+        asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d[i + 1]) : "r"(q1), "r"(one), "r"(off));
     }
 }
 __device__ __forceinline__ void oz_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
@@ -194,9 +194,9 @@ __device__ __forceinline__ int oz_exp(double2 v)
 // the imaginary parts of the vectors share one tile, columns 0 .. 3 and 4 .. 7: 72 MMAs.  The integers of all forms are the
 // same, so a column's bits do not depend on the width.
 // Bound by latency and issue slots: 12 warps per SM issue in 40% of the cycles, the tensor pipe is a third busy, a pair of
-// entries takes 50 instructions to split.  Z on 64 columns of the 30,720-unknown sphere, phases 1 + 2: DFMA 22.8 + 47.2 ms
-// (its rate), with the digits in each warp's registers (225 of them, six warps per SM) 8.2 + 21.1, now 4.7 + 13.2; on one
-// column 0.46 + 1.43 by DFMA and 0.46 + 1.54 now, four 1.53 + 3.44 and 0.48 + 1.56.  Error of Z x against 64-bit-mantissa
+// entries takes 47 instructions to split (51 with a mask per digit: 4.7 + 13.3 ms).  Z on 64 columns of the 30,720-unknown sphere, phases 1 + 2: DFMA 22.8 + 47.2 ms
+// (its rate), with the digits in each warp's registers (225 of them, six warps per SM) 8.2 + 21.1, now 4.6 + 13.1; on one
+// column 0.46 + 1.43 by DFMA and 0.44 + 1.45 now, four 1.53 + 3.44 and 0.46 + 1.47.  Error of Z x against 64-bit-mantissa
 // products (2-norm, relative): 1.1e-16, by FP64 FMAs 1e-15.
 template <bool NARROW> struct Oz {
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
