@@ -125,16 +125,12 @@ __device__ __forceinline__ int next_chunk_ll(int p, int pend, int step, const in
 // products.  Complex FP32: the coefficient blocks of the next chunk are copied with cp.async
 // while the current chunk waits and multiplies, and the vector blocks come from the tagged
 // copy.  Tagged publication (complex FP32): next to y, every entry is also written as two
-// 8-byte words (value half, launch epoch) -- each naturally aligned 8-byte store is observed
-// whole -- so a consumer validates the data it reads instead of waiting on a flag behind a
-// fence.
-__device__ __forceinline__ uint4 ld_tag(const uint4 *p)
+// 64-bit words (value half, launch epoch), each stored and loaded whole (wait.cuh), so a
+// consumer validates the data it reads instead of waiting on a flag behind a fence.
+__device__ __forceinline__ uint4 ld_tag(const uint4 *p) { return ld_words2(p); }
+__device__ __forceinline__ void st_tag(uint4 *p, float2 v, unsigned epoch)
 {
-    uint4 v;
-    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p));
-    return v;
+    st_words2(p, make_uint4(__float_as_uint(v.x), epoch, __float_as_uint(v.y), epoch));
 }
 
 // Staging copy from the tagged array: SB words per thread are loaded together; while any of
@@ -437,8 +433,7 @@ __device__ __forceinline__ void sweep_row(int o_blk, int no, const int *size, co
         }
         for (int e = threadIdx.x; e < no * nrhs; e += blockDim.x) {
             const float2 v = buf[e];
-            tag[o + e % no + (int64_t)(e / no) * n] =
-                make_uint4(__float_as_uint(v.x), (unsigned)epoch, __float_as_uint(v.y), (unsigned)epoch);
+            st_tag(tag + o + e % no + (int64_t)(e / no) * n, v, (unsigned)epoch);
         }
         for (int e = threadIdx.x; e < no * nrhs; e += blockDim.x) y[o + e % no + (int64_t)(e / no) * n] = buf[e];
         return;
@@ -645,9 +640,7 @@ __global__ void __launch_bounds__(256, 2) k_sweep_tc(int nb, const int *size, co
 #pragma unroll
     for (int u = 0; u < NE; ++u) {
         const int e = threadIdx.x + u * blockDim.x;
-        if (e < no * nc)
-            tag[o + e % no + (int64_t)(e / no) * n] =
-                make_uint4(__float_as_uint(out[u].x), (unsigned)epoch, __float_as_uint(out[u].y), (unsigned)epoch);
+        if (e < no * nc) st_tag(tag + o + e % no + (int64_t)(e / no) * n, out[u], (unsigned)epoch);
     }
 #pragma unroll
     for (int u = 0; u < NE; ++u) {

@@ -19,9 +19,10 @@
 // newest dependencies (the previous super-row) fall on different warps.
 //
 // Hand-over: y and z of a sweep live in row-major buffers that start as all-ones words; a
-// consumer reads a word until it is no longer all ones (each 8-byte word is stored whole, and a
-// result that is that NaN pattern is stored as another NaN), so neither flags nor fences are
-// needed, and a row that is never published ends every wait on it at the handle's bound.
+// consumer reads a word until it is no longer all ones (a result that is that NaN pattern is
+// stored as another NaN), so neither flags nor fences are needed, and a row that is never
+// published ends every wait on it at the handle's bound.  A word has 64 bits and is an element of
+// that size in the load and in the store (wait.cuh), so a half of it is never taken for a result.
 //
 // What binds it now: at one column the chain (69 super-rows of the 30,720-unknown sphere, 8.6 us each); at 64
 // columns the instructions (two CTAs of eight warps per SM issue every other cycle, a fifth of them FMAs: blocks
@@ -77,16 +78,9 @@ template <class T, int GW> struct S2Vec {
 };
 template <bool WIDE> __device__ __forceinline__ uint4 s2_ld(const void *p)
 {
-    uint4 v;
-    if constexpr (WIDE)
-        asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                     : "l"(p));
-    else {
-        asm volatile("ld.volatile.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
-        v.z = v.w = 0;
-    }
-    return v;
+    if constexpr (WIDE) return ld_words2(p);
+    const uint2 v = ld_word(p);
+    return make_uint4(v.x, v.y, 0, 0);
 }
 __device__ __forceinline__ bool s2_stale(uint4 v) { return (v.x & v.y) == ~0u || (v.z & v.w) == ~0u; }
 
@@ -121,15 +115,15 @@ __device__ __forceinline__ void s2_publish(float2 *p, float2 v)
 {
     unsigned a = __float_as_uint(v.x), b = __float_as_uint(v.y);
     if ((a & b) == ~0u) a = 0x7fffffffu;
-    asm volatile("st.volatile.global.v2.u32 [%0], {%1, %2};" ::"l"(p), "r"(a), "r"(b) : "memory");
+    st_word(p, make_uint2(a, b));
 }
 __device__ __forceinline__ void s2_publish(double2 *p, double2 v)
 {
-    unsigned long long a = (unsigned long long)__double_as_longlong(v.x),
-                       b = (unsigned long long)__double_as_longlong(v.y);
-    if (a == ~0ull) a = 0x7fffffffffffffffull;
-    if (b == ~0ull) b = 0x7fffffffffffffffull;
-    asm volatile("st.volatile.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
+    uint4 w = make_uint4((unsigned)__double2loint(v.x), (unsigned)__double2hiint(v.x), (unsigned)__double2loint(v.y),
+                         (unsigned)__double2hiint(v.y));
+    if ((w.x & w.y) == ~0u) w.y = 0x7fffffffu;
+    if ((w.z & w.w) == ~0u) w.w = 0x7fffffffu;
+    st_words2(p, w);
 }
 
 // One warp's reader of vector blocks: issue() starts the loads of rows [row, row + nc) of a
