@@ -220,9 +220,10 @@ int hm_get_fill_ranks(hm_handle h, int32_t *rank);
  *   op 5: y = Z x          (near + far, ORIGINAL order; the refinement residual operator);
  *   ops 8-12: ops 0-4 with the complex-FP32 factors and arithmetic of the mixed-precision
  *       inner solve (x and y stay complex FP64); precision 1 handles only (else HM_ESTATE).
- * The FP64 far and near products (ops 0, 3, 5 and the refinement residual) are sums of exact integer digit products
- * below the largest exponent of each matrix row and vector column, rounded once: a column with an infinity
- * or a NaN comes out as NaN, the others are not affected.
+ * The FP64 far and near products (ops 0, 3, 5 and the refinement residual) are summed as exact integer digit products
+ * below the largest entries of pieces of a matrix row and of a vector column, or, where that could be less accurate
+ * than FP64 FMAs, with those: no scale of U against V, of one block against another or of one part of a vector against
+ * another costs accuracy.  A column with an infinity or a NaN comes out as NaN, the others are not affected.
  * x and y must not overlap.
  */
 int hm_apply(hm_handle h, int32_t op, const void *dx, void *dy, int32_t nrhs);

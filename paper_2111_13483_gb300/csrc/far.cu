@@ -144,9 +144,18 @@ __global__ void __launch_bounds__(256) k_far_t(const int *task_lo, const int *ta
 // a vector column, an entry x is the integer v = x 2^(1084 - e), |v| < 2^62, truncated below 1, in eight signed
 // digits of 8 bits.  Products of digits i + j <= 7 are summed by mma.sync m16n8k16 (FP16 digits, FP32 sums): every sum of
 // 64 entries stays within 2^24 and is exact, and goes into 64-bit integers.  So a result is the exact sum of
-// truncated integers, in any order and at any width, with an error of about 2^-62 of (row maximum x column maximum)
-// per term: 2^-9 of an FP64 rounding, which leaves room for entries far below the maxima.  A row or column with
-// an infinity or a NaN gives NaN.
+// truncated integers, in any order and at any width.  Its error per term, relative to 2^(sum of the two exponents), is
+// 2^-58.8 at most (the digit products left out, at most 2^64.8 of 2^124, and the two truncations) and about 2^-62 as a rule,
+// whatever the term's own size.
+// That is FP64's accuracy or better where row and column do not both hold terms far below their largest entries.
+// Two things see to that.  The exponents are local: a CTA takes them from the rows and the piece of the
+// contraction that it sums, and what multiplies different vectors (t, s, u in the far field, u in the near field) is summed
+// apart (FarPlan::zsegs), so that neither the scale of U against V nor that of one table against another matters.
+// And a result below OZ_MIN of row maximum x column maximum is computed again with FP64 FMAs, a warp per output
+// (OzAgain): for it the bound, 2 K 2^-58.8 for the K complex terms, may lie above that of FMAs, 2 K 2^-53 sum |a x|, for
+// whose sum the result itself stands in.  At OZ_MIN = 2^-5.75 the two meet.  Of the outputs of a sphere and a plate, with
+// random vectors, plane waves and solutions, that is 0.1% to 0.5%.
+constexpr double OZ_MIN = 5.5e18;   // 2^62.25 of 2^68 units
 constexpr int OZ_KC = 16, OZ_FOLD = 4;   // chunk = one step of the MMA; steps between foldings
 constexpr int OZ_ROWS = 32;               // rows of a CTA
 
@@ -155,7 +164,7 @@ __device__ __forceinline__ uint2 oz_bytes(double x, int e)
 {
     const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
     const uint32_t mh = hi & 0xfffff | 0x100000, a = __funnelshift_l(lo, mh, 9), b = lo << 9;
-    const uint32_t r = (uint32_t)(e - (int)(hi >> 20 & 0x7ff));   // e >= 64 (oz_exp): a zero is shifted out
+    const uint32_t r = (uint32_t)(e - (int)(hi >> 20 & 0x7ff));   // e >= 64: a zero is shifted out
     uint32_t l, h, l2;   // (a : b) >> r
     asm("shr.u32 %0, %1, %2;" : "=r"(h) : "r"(a), "r"(r));        // shifts of 32 and more give 0
     l = __funnelshift_rc(b, a, r);
@@ -183,21 +192,18 @@ __device__ __forceinline__ void oz_mma(float (&c)[4], const uint32_t (&a)[4], ui
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ int oz_exp(double2 v)
-{
-    return max(64, max(__double2hiint(v.x) >> 20 & 0x7ff, __double2hiint(v.y) >> 20 & 0x7ff));
-}
-
 // A CTA takes 32 rows x NT column tiles of 8 right-hand sides, one warp per 16 x 8 outputs.  Per chunk of 16 contraction
 // entries: the raw entries land in one of two buffers (cp.async), the warps turn them into digit fragments in
 // shared memory, once for all warps that use them, and then each runs its 144 MMAs.  Up to four columns (NARROW) the real and
 // the imaginary parts of the vectors share one tile, columns 0 .. 3 and 4 .. 7: 72 MMAs.  The integers of all forms are the
 // same, so a column's bits do not depend on the width.
 // Bound by latency and issue slots: 12 warps per SM issue in 40% of the cycles, the tensor pipe is a third busy, a pair of
-// entries takes 47 instructions to split (51 with a mask per digit: 4.7 + 13.3 ms).  Z on 64 columns of the 30,720-unknown sphere, phases 1 + 2: DFMA 22.8 + 47.2 ms
-// (its rate), with the digits in each warp's registers (225 of them, six warps per SM) 8.2 + 21.1, now 4.6 + 13.1; on one
-// column 0.46 + 1.43 by DFMA and 0.44 + 1.45 now, four 1.53 + 3.44 and 0.46 + 1.47.  Error of Z x against 64-bit-mantissa
-// products (2-norm, relative): 1.1e-16, by FP64 FMAs 1e-15.
+// entries takes 47 instructions to split.  Z on 64 columns of the 30,720-unknown sphere, phases 1 + 2: DFMA 22.8 + 47.2 ms
+// (its rate), with the digits in each warp's registers (225 of them, six warps per SM) 8.2 + 21.1, with one exponent
+// for all of a row and a column, and so only for balanced factors, 4.6 + 13.1, now 5.0 + 15.6: four tables instead of two
+// 1.3 ms, the columns' exponents 0.4, the outputs computed again 1.5.  One column: 0.46 + 1.43 by DFMA, 0.47 + 1.67 now; four:
+// 1.53 + 3.44 and 0.51 + 1.79.  Error of Z x against products with 64-bit mantissas, of |Z| |x| per entry: 1.5e-16 to 3.6e-16;
+// 2-norm, relative: 1.1e-16 to 1.3e-16, by FP64 FMAs 6e-16 to 1.1e-15.
 template <bool NARROW> struct Oz {
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     int nct, ldr;                  // column tiles; row stride of the raw vector entries
@@ -221,6 +227,10 @@ template <bool NARROW> struct Oz {
         sum = (int64_t *)(bd + nct * 8 * (NARROW ? 16 : 32));
         raw = (double2 *)(sum + nw * 16 * 32);
         sum += wp * 16 * 32 + lane;
+        reset();
+    }
+    __device__ __forceinline__ void reset()
+    {
 #pragma unroll
         for (int x = 0; x < 16; ++x) sum[32 * x] = 0;
         clear();
@@ -247,7 +257,7 @@ template <bool NARROW> struct Oz {
         if constexpr (NARROW) {   // two warps, a word of the vector fragments (entries + 8 word) each; by column real or imaginary part
             uint32_t d[8];
             const double *y0 = (const double *)(Ys + (k + 8 * wp) * ldr + (g & 3)) + (g >> 2);
-            oz_pair(y0[0], y0[2 * ldr], ce(g & 3), d);
+            oz_pair(y0[0], y0[2 * ldr], max(ce(g & 3), 64), d);
 #pragma unroll
             for (int i = 0; i < 8; ++i) ((uint32_t *)bd)[(i * 32 + lane) * 2 + wp] = d[i];
         } else {   // 8 halves of coefficient fragments, then 2 of each column tile's, dealt out to the warps
@@ -258,11 +268,11 @@ template <bool NARROW> struct Oz {
                     const int r = 16 * (x >> 2) + g;
                     if (r - g >= rows) continue;
                     const double *w0 = (const double *)(Ws + (k + 8 * (x & 1)) * ldw + r) + (x >> 1 & 1);
-                    oz_pair(w0[0], w0[2 * ldw], re(r), d[0]);
-                    oz_pair(w0[16], w0[2 * ldw + 16], re(r + 8), d[1]);
+                    oz_pair(w0[0], w0[2 * ldw], max(re(r), 64), d[0]);
+                    oz_pair(w0[16], w0[2 * ldw + 16], max(re(r + 8), 64), d[1]);
                     dst = (uint2 *)(ad + (x >> 1) * 8 * 32 + lane) + (x & 1);
                 } else {   // words q: entries + 8 q of one part
-                    const int t = x - 8 >> 1, part = x & 1, e = ce(8 * t + g);
+                    const int t = x - 8 >> 1, part = x & 1, e = max(ce(8 * t + g), 64);
                     const double *y0 = (const double *)(Ys + k * ldr + 8 * t + g) + part;
                     oz_pair(y0[0], y0[2 * ldr], e, d[0]);
                     oz_pair(y0[16 * ldr], y0[18 * ldr], e, d[1]);
@@ -292,7 +302,7 @@ template <bool NARROW> struct Oz {
             for (int q = 0; q < 4; ++q) {
                 const int r = row0() + g + 8 * (q & 1);
                 const double *w0 = (const double *)(ws(ch) + (k + 8 * (q >> 1)) * ldw + r) + part;
-                oz_pair(w0[0], w0[2 * ldw], re(r), d[q]);
+                oz_pair(w0[0], w0[2 * ldw], max(re(r), 64), d[q]);
             }
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -364,13 +374,14 @@ template <bool NARROW> struct Oz {
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         __syncthreads();
     }
-    // put(row, column, value) for the outputs of the warp (rows, columns of the CTA); whole warps call it
+    // put(row, column, value, again) for the outputs of the warp (rows, columns of the CTA); whole warps call it.  re, ce:
+    // largest exponents of the row and the column, 0 with nothing but zeros; again: the value is to be computed by FP64 FMAs
     template <class RE, class CE, class Put>
     __device__ __forceinline__ void store(int rows, int nrhs, RE &&re, CE &&ce, Put &&put)
     {
         if (row0() >= rows) return;
         fold();
-#pragma unroll
+#pragma unroll 1
         for (int x = 0; x < 4; ++x) {
             const int row = row0() + (lane >> 2) + 8 * (x >> 1), col = col0() + 2 * (lane & 3) + (x & 1);
             int64_t v[2][2];
@@ -384,15 +395,77 @@ template <bool NARROW> struct Oz {
                     v[1][p] += r2;
                 }
             }
-            if (row >= rows || col >= nrhs) continue;
-            const int ea = re(row), eb = ce(col), e = ea + eb - 2112, eh = e / 2;
-            double2 y = make_double2(nan(""), nan(""));
-            if (ea != 0x7ff && eb != 0x7ff) {   // in two steps: 2^e alone may be below the smallest power of two
+            const bool ok = row < rows && col < nrhs && (!NARROW || (lane & 3) < 2);
+            double2 y = make_double2(0.0, 0.0);
+            bool again = false;
+            if (ok) {
+                const int ra = re(row), rb = ce(col), e = max(ra, 64) + max(rb, 64) - 2112, eh = e / 2;
+                y.x = fma((double)v[0][0], 4294967296.0, (double)v[0][1]);
+                y.y = fma((double)v[1][0], 4294967296.0, (double)v[1][1]);
+                again = ra && rb && (fmax(fabs(y.x), fabs(y.y)) < OZ_MIN || ra == 0x7ff || rb == 0x7ff);
+                // in two steps: 2^e alone may be below the smallest power of two
                 const double s0 = __hiloint2double(eh + 1023 << 20, 0), s1 = __hiloint2double(e - eh + 1023 << 20, 0);
-                y.x = fma((double)v[0][0], 4294967296.0, (double)v[0][1]) * s0 * s1;
-                y.y = fma((double)v[1][0], 4294967296.0, (double)v[1][1]) * s0 * s1;
+                y.x = y.x * s0 * s1;
+                y.y = y.y * s0 * s1;
             }
-            put(row, col, y);
+            if (ok) put(row, col, y, again);
+        }
+    }
+};
+// the largest exponent of entries: 0 for zeros alone
+__device__ __forceinline__ int oz_exp(double2 v)
+{
+    const int hx = __double2hiint(v.x) & 0x7fffffff, hy = __double2hiint(v.y) & 0x7fffffff;
+    const int e = max(hx, hy) >> 20;
+    return e ? e : (hx | hy | __double2loint(v.x) | __double2loint(v.y)) != 0;   // 1: nothing but subnormals
+}
+// A CTA's outputs to be computed again, row * 16 + column, dealt out to the warps at its end (a warp that
+// did so at once held up the others: phase 2 of 64 columns of the 30,720-unknown sphere 17.3 ms for 16.5)
+struct OzAgain {
+    int n;
+    uint16_t list[OZ_ROWS * 16];
+    uint8_t tabs[OZ_ROWS * 16];   // phase 2: the tables concerned, a bit each
+};
+__device__ __forceinline__ double2 warp_sum(double2 v)
+{
+    for (int o = 16; o > 0; o >>= 1) {
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+    }
+    return v;
+}
+
+// Column exponents of pieces of the vectors.  The kernels that write u, t and s also write their entries' exponents, 16 per
+// row, so that a piece is 32 bytes a row to look at instead of 256: eight columns per thread (four when NARROW).
+constexpr int VEXP = 16;
+template <bool NARROW> struct OzCols {
+    static constexpr int HV = NARROW ? 1 : 2;   // threads abreast over a row
+    uint4 m = make_uint4(0, 0, 0, 0);           // pairs of columns
+    __device__ __forceinline__ void row(const uint16_t *e)
+    {
+        if (NARROW) {
+            const uint2 v = *(const uint2 *)e;
+            m.x = __vmaxu2(m.x, v.x);
+            m.y = __vmaxu2(m.y, v.y);
+        } else {
+            const uint4 v = *(const uint4 *)(e + 8 * (threadIdx.x & 1));
+            m.x = __vmaxu2(m.x, v.x);
+            m.y = __vmaxu2(m.y, v.y);
+            m.z = __vmaxu2(m.z, v.z);
+            m.w = __vmaxu2(m.w, v.w);
+        }
+    }
+    __device__ __forceinline__ void max_into(int *s_ce)   // whole warps
+    {
+        uint32_t w[4] = {m.x, m.y, m.z, m.w};
+#pragma unroll
+        for (int i = 0; i < (NARROW ? 2 : 4); ++i) {
+#pragma unroll
+            for (int o = HV; o < 32; o <<= 1) w[i] = __vmaxu2(w[i], __shfl_xor_sync(0xffffffffu, w[i], o));
+            if ((threadIdx.x & 31) < HV) {
+                atomicMax(&s_ce[8 * (threadIdx.x & 1) + 2 * i], (int)(w[i] & 0xffff));
+                atomicMax(&s_ce[8 * (threadIdx.x & 1) + 2 * i + 1], (int)(w[i] >> 16));
+            }
         }
     }
 };
@@ -405,17 +478,18 @@ __device__ __forceinline__ void oz_cp(double2 *dst, const double2 *src, bool ok)
 }
 
 // phase 1, tasks as in k_far_t, blockIdx.y: which 32 of its factor columns; rexp: exponents of the factor columns, of V
-// (tlen), then of U; cexp: of the columns of u (read), then of t and s (written)
+// (tlen), then of U; vexp: of the entries of t, s (written) and u (read)
 template <bool NARROW>
 __global__ void __launch_bounds__(NARROW ? 64 : 128, NARROW ? 6 : 3) k_far_t64(const int *task_lo, const int *task_hi, const int *task_ptr,
                                                     const int64_t *item_off, const int *item_ld, const int *item_rank,
                                                     const int *item_row, const int *item_isv, const double2 *U,
                                                     const double2 *V, const double2 *u, int nrhs, double2 *t, double2 *s,
-                                                    const int *rexp, int64_t tlen, int *cexp)
+                                                    const uint16_t *rexp, uint16_t *vexp, int64_t tlen)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ int s_item[64], s_l[64], s_cmax[16], s_re[OZ_ROWS], s_ce[16];
+    __shared__ int s_item[64], s_l[64], s_re[OZ_ROWS], s_ce[16];
     __shared__ const double2 *s_src[64];
+    __shared__ OzAgain s_ag;
     const int task = blockIdx.x, f0 = OZ_ROWS * blockIdx.y;
     const int lo = task_lo[task], hi = task_hi[task], i0 = task_ptr[task], i1 = task_ptr[task + 1];
     const int R = far_items(i0, i1, item_off, item_ld, item_rank, item_isv, U, V, s_item, s_l, s_src) - f0;
@@ -425,12 +499,17 @@ __global__ void __launch_bounds__(NARROW ? 64 : 128, NARROW ? 6 : 3) k_far_t64(c
         const int it = s_item[f0 + row];
         return (item_isv[it] ? 0 : tlen) + item_row[it] + s_l[f0 + row];
     };
-    if (threadIdx.x < 16) {
-        s_cmax[threadIdx.x] = 0;
-        s_ce[threadIdx.x] = threadIdx.x < nrhs ? cexp[threadIdx.x] : 64;
-    }
-    if (threadIdx.x < OZ_ROWS) s_re[threadIdx.x] = threadIdx.x < rows ? rexp[dest(threadIdx.x)] : 64;
+    if (threadIdx.x == 0) s_ag.n = 0;
+    if (threadIdx.x < 16) s_ce[threadIdx.x] = 0;
+    if (threadIdx.x < OZ_ROWS) s_re[threadIdx.x] = threadIdx.x < rows ? rexp[dest(threadIdx.x)] : 0;
     Oz<NARROW> oz(smraw, nrhs);
+    __syncthreads();
+    {   // the columns' exponents over the task's rows
+        OzCols<NARROW> cm;
+#pragma unroll 4
+        for (int q = lo + threadIdx.x / cm.HV; q < hi; q += blockDim.x / cm.HV) cm.row(vexp + (2 * tlen + q) * VEXP);
+        cm.max_into(s_ce);
+    }
     const int nch = (hi - lo + OZ_KC - 1) / OZ_KC;
     auto stage = [&](int c) {   // factor column rr of row c0 + qq, half a warp each; then the vector rows
         if (c < nch) {
@@ -452,65 +531,76 @@ __global__ void __launch_bounds__(NARROW ? 64 : 128, NARROW ? 6 : 3) k_far_t64(c
     auto re = [&](int row) { return s_re[row]; };
     auto ce = [&](int col) { return s_ce[col]; };
     oz.run(nch, rows, stage, re, ce);
-    oz.store(rows, nrhs, re, ce, [&](int row, int col, double2 v) {
+    auto put = [&](int row, int col, double2 v) {
         const int64_t d = dest(row);
         (d < tlen ? t + d * nrhs : s + (d - tlen) * nrhs)[col] = v;
-        atomicMax(&s_cmax[col], oz_exp(v));
+        vexp[d * VEXP + col] = (uint16_t)oz_exp(v);
+    };
+    oz.store(rows, nrhs, re, ce, [&](int row, int col, double2 v, bool again) {
+        if (again) s_ag.list[atomicAdd(&s_ag.n, 1)] = (uint16_t)(row * 16 + col);
+        else put(row, col, v);
     });
     __syncthreads();
-    if (threadIdx.x < nrhs) atomicMax(&cexp[16 + threadIdx.x], s_cmax[threadIdx.x]);
+    for (int x = oz.wp; x < s_ag.n; x += oz.nw) {   // a lane per row of the range, in turn
+        const int row = s_ag.list[x] >> 4, col = s_ag.list[x] & 15;
+        const double2 *f = s_src[f0 + row];
+        double2 v = make_double2(0.0, 0.0);
+#pragma unroll 8
+        for (int q = oz.lane; q < hi - lo; q += 32) v = cfma(f[q], u[(int64_t)(lo + q) * nrhs + col], v);
+        v = warp_sum(v);
+        if (oz.lane == 0) put(row, col, v);
+    }
 }
 
 // exponents of the factor columns (see k_far_t64): task as there, one warp per factor column
 __global__ void k_far_rexp1(const int *task_lo, const int *task_hi, const int *task_ptr, const int64_t *item_off,
                             const int *item_ld, const int *item_rank, const int *item_row, const int *item_isv,
-                            const double2 *U, const double2 *V, int *rexp, int64_t tlen)
+                            const double2 *U, const double2 *V, uint16_t *rexp, int64_t tlen)
 {
     __shared__ int s_item[64], s_l[64];
     __shared__ const double2 *s_src[64];
     const int task = blockIdx.x, lane = threadIdx.x & 31;
     const int R = far_items(task_ptr[task], task_ptr[task + 1], item_off, item_ld, item_rank, item_isv, U, V, s_item, s_l, s_src);
     for (int rr = threadIdx.x >> 5; rr < R; rr += blockDim.x >> 5) {
-        int e = 64;
+        int e = 0;
         for (int q = lane; q < task_hi[task] - task_lo[task]; q += 32) e = max(e, oz_exp(s_src[rr][q]));
         e = __reduce_max_sync(0xffffffffu, e);
         const int it = s_item[rr];
-        if (lane == 0) rexp[(item_isv[it] ? 0 : tlen) + item_row[it] + s_l[rr]] = e;
+        if (lane == 0) rexp[(item_isv[it] ? 0 : tlen) + item_row[it] + s_l[rr]] = (uint16_t)e;
     }
 }
-// exponents of the coefficient rows of a leaf (one CTA): over its far segments (F0 = U, F1 = V) or its near ones
-__global__ void k_far_rexp2(const int *leaf_ptr, const int *part_ptr, const FarSegD *segs, const double2 *F0,
-                            const double2 *F1, int *rexp)
+// exponents of the coefficient rows of one part (blockIdx.x, see FarPlan::zpart) of a leaf in one table (blockIdx.y):
+// rexp[(table * FAR_PARTS + part) * n + row]
+__global__ void k_far_rexp2(int nl, int n, const int *leaf_ptr, const int *zpart, const FarSegD *segs, const double2 *U,
+                            const double2 *V, const double2 *nearp, uint16_t *rexp)
 {
     __shared__ int s_e[64];
-    const int l = blockIdx.x, a = leaf_ptr[l], ni = leaf_ptr[l + 1] - a, i = threadIdx.x & 63;
-    if (threadIdx.x < 64) s_e[threadIdx.x] = 64;   // a leaf without segments: the smallest exponent
+    const int l = blockIdx.x / FAR_PARTS, pp = blockIdx.x % FAR_PARTS, tab = blockIdx.y;
+    const int a = leaf_ptr[l], ni = leaf_ptr[l + 1] - a, i = threadIdx.x & 63;
+    const int *pt = zpart + tab * (nl * FAR_PARTS + 1) + blockIdx.x;
+    if (threadIdx.x < 64) s_e[threadIdx.x] = 0;
     __syncthreads();
-    int e = 64;
-    for (int q = part_ptr[l * FAR_PARTS]; q < part_ptr[(l + 1) * FAR_PARTS] && i < ni; ++q) {
+    int e = 0;
+    for (int q = pt[0]; q < pt[1] && i < ni; ++q) {
         const FarSegD g = segs[q];
-        const double2 *F = ((g.src & 1) ? F1 : F0) + g.foff + (int64_t)i * g.fi;
+        const double2 *F = (tab == FAR_TABS - 1 ? nearp : (g.src & 1) ? V : U) + g.foff + (int64_t)i * g.fi;
         for (int kk = threadIdx.x >> 6; kk < g.len; kk += blockDim.x >> 6) e = max(e, oz_exp(F[(int64_t)kk * g.fk]));
     }
     atomicMax(&s_e[i], e);
     __syncthreads();
-    if (threadIdx.x < ni) rexp[a + threadIdx.x] = s_e[threadIdx.x];
+    if (threadIdx.x < ni) rexp[(int64_t)(tab * FAR_PARTS + pp) * n + a + threadIdx.x] = (uint16_t)s_e[threadIdx.x];
 }
-// u[i * nrhs + r] = x[idx[i] + r * n] and the exponents of its columns, cexp[r] (cexp is zero before)
-__global__ void k_far_gather64(int n, int nrhs, const int *idx, const double2 *x, double2 *u, int *cexp)
+// u[i * nrhs + r] = x[idx[i] + r * n], its exponent; bit r of *bad (zero before): an infinity or a NaN in column r
+__global__ void k_far_gather64(int n, int nrhs, const int *idx, const double2 *x, double2 *u, uint16_t *uexp, int *bad)
 {
-    __shared__ int s_e[16];
-    if (threadIdx.x < 16) s_e[threadIdx.x] = 0;
-    __syncthreads();
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e < (int64_t)n * nrhs) {
-        const int i = (int)(e / nrhs), r = (int)(e - (int64_t)i * nrhs);
-        const double2 v = x[idx[i] + (int64_t)r * n];
-        u[e] = v;
-        atomicMax(&s_e[r], oz_exp(v));
-    }
-    __syncthreads();
-    if (threadIdx.x < nrhs) atomicMax(&cexp[threadIdx.x], s_e[threadIdx.x]);
+    if (e >= (int64_t)n * nrhs) return;
+    const int i = (int)(e / nrhs), r = (int)(e - (int64_t)i * nrhs);
+    const double2 v = x[idx[i] + (int64_t)r * n];
+    const int ex = oz_exp(v);
+    u[e] = v;
+    uexp[(int64_t)i * VEXP + r] = (uint16_t)ex;
+    if (ex == 0x7ff) atomicOr(bad, 1 << r);
 }
 
 // Phase 2: one CTA per leaf over the leaf's segments (FarSegD, list order, len <= 32).
@@ -799,46 +889,55 @@ __global__ void __launch_bounds__(256) k_far_y32(int nl, const int *leaf_ptr, co
         }
 }
 
-// complex FP64, phase 2: the segments of the far list and, with nearp, those of the leaf's near-field blocks (zpart /
-// zkcum / zsegs), which gives Z u in one pass; blockIdx.y: which 32 of the leaf's rows; rexp: exponents of the far rows (n),
-// then of the near rows
+// complex FP64, phase 2: the segments of the tables of the far field and, with nearp, those of the leaf's near-field
+// blocks, which gives Z u in one pass, the tables added in their order; blockIdx.y: which 32 of the leaf's rows; rexp: see
+// k_far_rexp2; vexp: see k_far_t64
 template <bool NARROW>
-__global__ void __launch_bounds__(NARROW ? 64 : 128, NARROW ? 6 : 3) k_far_y64(int nl, const int *leaf_ptr, const int *part_ptr, const int *kcum,
-                                                    const FarSegD *segs, const int *zpart, const int *zkcum,
-                                                    const FarSegD *zsegs, const double2 *U, const double2 *V,
+__global__ void __launch_bounds__(NARROW ? 64 : 128, NARROW ? 6 : 3) k_far_y64(int nl, const int *leaf_ptr, const int *zpart,
+                                                    const int *kc, const FarSegD *sg, const double2 *U, const double2 *V,
                                                     const double2 *nearp, const double2 *t, const double2 *s,
                                                     const double2 *u, const int *cl2new, int n, int nrhs, double2 *part,
-                                                    const int *rexp, const int *cexp)
+                                                    const uint16_t *rexp, const uint16_t *vexp, int64_t tlen)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ int s_re[OZ_ROWS], s_ce[16];
+    __shared__ OzAgain s_ag;
     const int l = blockIdx.x / FAR_PARTS, pp = blockIdx.x % FAR_PARTS;
     if (l >= nl) return;
     const int r0 = OZ_ROWS * blockIdx.y, a = leaf_ptr[l] + r0, rows = min(leaf_ptr[l + 1] - a, OZ_ROWS);
     if (rows <= 0) return;
-    if (threadIdx.x < OZ_ROWS) {
-        int e = 64;
-        if (threadIdx.x < rows) e = nearp ? max(rexp[a + threadIdx.x], rexp[n + a + threadIdx.x]) : rexp[a + threadIdx.x];
-        s_re[threadIdx.x] = e;
-    }
-    if (threadIdx.x < 16) s_ce[threadIdx.x] = threadIdx.x < nrhs ? max(cexp[threadIdx.x], cexp[16 + threadIdx.x]) : 64;
+    double2 *out = part + (size_t)pp * n * nrhs + cl2new[leaf_ptr[l]] + r0;
     Oz<NARROW> oz(smraw, nrhs);
     auto re = [&](int row) { return s_re[row]; };
     auto ce = [&](int col) { return s_ce[col]; };
-    for (int tab = 0; tab < (nearp ? 2 : 1); ++tab) {
-        const int *kc = tab ? zkcum : kcum;
-        const FarSegD *sg = tab ? zsegs : segs;
-        const double2 *F0 = tab ? nearp : U, *F1 = tab ? nearp : V;
-        const int p0 = (tab ? zpart : part_ptr)[blockIdx.x], w1 = (tab ? zpart : part_ptr)[blockIdx.x + 1];
-        const int k0 = p0 < w1 ? kc[p0] : 0, K = p0 < w1 ? kc[w1] - k0 : 0, nch = (K + OZ_KC - 1) / OZ_KC;
+    if (threadIdx.x == 0) s_ag.n = 0;
+    for (int x = threadIdx.x; x < OZ_ROWS * 16; x += blockDim.x) s_ag.tabs[x] = 0;
+    bool first = true;
+    for (int tab = 0; tab < (nearp ? FAR_TABS : FAR_TABS - 1); ++tab) {
+        const int *pt = zpart + tab * (nl * FAR_PARTS + 1) + blockIdx.x;
+        const int p0 = pt[0], w1 = pt[1];
+        if (p0 >= w1) continue;
+        const int k0 = kc[p0], K = kc[w1] - k0, nch = (K + OZ_KC - 1) / OZ_KC;
+        const double2 *F0 = tab == FAR_TABS - 1 ? nearp : U, *F1 = tab == FAR_TABS - 1 ? nearp : V;
+        const double2 *Y = tab == 0 ? t : tab == 1 ? s : u;
+        if (threadIdx.x < OZ_ROWS)
+            s_re[threadIdx.x] = threadIdx.x < rows ? rexp[(int64_t)(tab * FAR_PARTS + pp) * n + a + threadIdx.x] : 0;
+        if (threadIdx.x < 16) s_ce[threadIdx.x] = 0;
+        __syncthreads();
+        {   // the columns' exponents over the part, eight rows of a segment side by side
+            const uint16_t *ve = vexp + (tab == 0 ? 0 : tab == 1 ? tlen : 2 * tlen) * VEXP;
+            OzCols<NARROW> cm;
+            for (int q = p0 + threadIdx.x / (8 * cm.HV); q < w1; q += blockDim.x / (8 * cm.HV)) {
+                const int64_t y0 = sg[q].yrow;
+                const int len = sg[q].len;
+                for (int kk = threadIdx.x / cm.HV & 7; kk < len; kk += 8) cm.row(ve + (y0 + kk) * VEXP);
+            }
+            cm.max_into(s_ce);
+        }
         // lane o and o + 16 of every warp follow contraction entry o of the chunks through the segments, with the next
         // segment's descriptor on its way
-        int q = p0, qlo = 0, qhi = 0, hn = 0;
-        FarSegD gn = {};
-        if (K > 0) {
-            gn = sg[p0];
-            hn = kc[p0 + 1] - k0;
-        }
+        int q = p0, qlo = 0, qhi = 0, hn = kc[p0 + 1] - k0;
+        FarSegD gn = sg[p0];
         const double2 *F = nullptr, *Yb = nullptr;
         int fi = 0, fk = 0;
         auto stage = [&](int c) {
@@ -847,8 +946,7 @@ __global__ void __launch_bounds__(NARROW ? 64 : 128, NARROW ? 6 : 3) k_far_y64(i
                 const int o = oz.lane & 15, kk = c * OZ_KC + o;
                 while (kk < K && kk >= qhi) {
                     F = ((gn.src & 1) ? F1 : F0) + gn.foff + (int64_t)r0 * gn.fi;
-                    const int ys = gn.src >> 1;
-                    Yb = (ys == 0 ? t : (ys == 1 ? s : u)) + gn.yrow * nrhs;
+                    Yb = Y + gn.yrow * nrhs;
                     fi = gn.fi;
                     fk = gn.fk;
                     qlo = qhi;
@@ -879,9 +977,46 @@ __global__ void __launch_bounds__(NARROW ? 64 : 128, NARROW ? 6 : 3) k_far_y64(i
             cp_async_commit();
         };
         oz.run(nch, rows, stage, re, ce);
+        oz.store(rows, nrhs, re, ce, [&](int row, int col, double2 v, bool again) {   // one lane's, in every table
+            if (again) {
+                uint8_t *b = s_ag.tabs + row * 16 + col;
+                if (!*b) s_ag.list[atomicAdd(&s_ag.n, 1)] = (uint16_t)(row * 16 + col);
+                *b |= (uint8_t)(1 << tab);
+                v = make_double2(0.0, 0.0);
+            }
+            double2 *o = out + row + (int64_t)col * n;
+            *o = first ? v : make_double2(o->x + v.x, o->y + v.y);
+        });
+        oz.reset();
+        first = false;
+        __syncthreads();   // the exponents are read
     }
-    double2 *out = part + (size_t)pp * n * nrhs + cl2new[leaf_ptr[l]] + r0;
-    oz.store(rows, nrhs, re, ce, [&](int row, int col, double2 v) { out[row + (int64_t)col * n] = v; });
+    for (int x = oz.wp; x < s_ag.n; x += oz.nw) {
+        const int row = s_ag.list[x] >> 4, col = s_ag.list[x] & 15;
+        double2 *o = out + row + (int64_t)col * n, w = make_double2(0.0, 0.0);
+        for (int tabs = s_ag.tabs[row * 16 + col]; tabs; tabs &= tabs - 1) {
+            const int tab = __ffs(tabs) - 1;
+            const int *pt = zpart + tab * (nl * FAR_PARTS + 1) + blockIdx.x;
+            const double2 *F0 = tab == FAR_TABS - 1 ? nearp : U, *F1 = tab == FAR_TABS - 1 ? nearp : V;
+            const double2 *Y = tab == 0 ? t : tab == 1 ? s : u;
+            const int J = tab < 2 ? 1 : 4;   // a lane per (short) segment of rank vectors, four per segment of blocks
+            double2 v = make_double2(0.0, 0.0);
+            for (int q = pt[0] + oz.lane / J; q < pt[1]; q += 32 / J) {
+                const FarSegD g = sg[q];
+                const double2 *f = ((g.src & 1) ? F1 : F0) + g.foff + (int64_t)(r0 + row) * g.fi;
+                const double2 *y = Y + g.yrow * nrhs + col;
+#pragma unroll 4
+                for (int kk = oz.lane % J; kk < g.len; kk += J) v = cfma(f[(int64_t)kk * g.fk], y[kk * nrhs], v);
+            }
+            v = warp_sum(v);
+            w.x += v.x;
+            w.y += v.y;
+        }
+        if (oz.lane == 0) *o = make_double2(o->x + w.x, o->y + w.y);
+    }
+    if (first)
+        for (int e = threadIdx.x; e < rows * nrhs; e += blockDim.x)
+            out[e % rows + (int64_t)(e / rows) * n] = make_double2(0.0, 0.0);
 }
 
 // ---- complex FP32 on the tensor cores ------------------------------------------------------
@@ -1088,12 +1223,10 @@ __global__ void __launch_bounds__(256, 2) k_far_y_tc(int nl, const int *leaf_ptr
     acc.close();
 }
 
-// y = sum of the FAR_PARTS partial products, added in part order
-// (the column exponents of the FP64 product are cleared here, for its next call)
-template <class T> __global__ void k_far_sum(int64_t len, const T *part, T *y, int *cexp = nullptr)
+// y = sum of the FAR_PARTS partial products, added in part order; bad: see k_far_gather64
+template <class T> __global__ void k_far_sum(int n, int64_t len, const T *part, T *y, const int *bad = nullptr)
 {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (cexp && e < 32) cexp[e] = 0;
     if (e >= len) return;
     T v = part[e];
     for (int p = 1; p < FAR_PARTS; ++p) {
@@ -1101,9 +1234,12 @@ template <class T> __global__ void k_far_sum(int64_t len, const T *part, T *y, i
         v.x += w.x;
         v.y += w.y;
     }
+    if constexpr (sizeof(T) == 16) {
+        const int b = bad ? *bad : 0;
+        if (b && b >> (int)(e / n) & 1) v = make_double2(nan(""), nan(""));
+    }
     y[e] = v;
 }
-
 
 namespace {
 template <class T> struct FarLaunch {
@@ -1140,7 +1276,7 @@ template <class T> struct FarLaunch {
                       h->nl, h->d_leaf_ptr, h->d_part_ptr, h->d_seg_kcum, h->d_segs, U, V, t, s, ucl, h->d_cl2new,
                       n, nrhs, part, budget)));
         const int64_t len = (int64_t)n * nrhs;
-        HM_LAUNCH(h, K_FAR2, k_far_sum<T><<<nblk(len, 256), 256, 0, h->stream>>>(len, part, y));
+        HM_LAUNCH(h, K_FAR2, k_far_sum<T><<<nblk(len, 256), 256, 0, h->stream>>>(n, len, part, y));
         return cudaGetLastError();
     }
 };
@@ -1172,28 +1308,29 @@ static cudaError_t far_tc_launch(hm_ctx *h, const float2 *U, const float2 *V, fl
                   h->nl, h->d_leaf_ptr, h->d_part_ptr, h->d_seg_kcum, h->d_segs, U, V, t, s, ucl, h->d_cl2new, n, nrhs,
                   part, h->d_err)));
     const int64_t len = (int64_t)n * nrhs;
-    HM_LAUNCH(h, K_FAR2, k_far_sum<float2><<<nblk(len, 256), 256, 0, h->stream>>>(len, part, y));
+    HM_LAUNCH(h, K_FAR2, k_far_sum<float2><<<nblk(len, 256), 256, 0, h->stream>>>(n, len, part, y));
     return cudaGetLastError();
 }
 
-// exponents of the coefficient rows for the FP64 products, once per handle (h->d_rexp: V columns, U columns, far rows,
-// near rows)
+// exponents of the coefficient rows for the FP64 products, once per handle (h->d_rexp: V columns, U columns, then the rows
+// of the leaves by table and part)
 cudaError_t far64_prepare(hm_ctx *h)
 {
     const FarPlan &F = h->fplan;
-    const int64_t tlen = F.tlen, n = h->n;
+    const int64_t tlen = F.tlen, n = h->n, len = 2 * tlen + FAR_TABS * FAR_PARTS * n;
     cudaError_t e;
-    if ((e = h->arena.alloc((void **)&h->d_rexp, sizeof(int) * (size_t)(2 * tlen + 2 * n + 32)))) return e;
-    h->d_cexp = h->d_rexp + 2 * tlen + 2 * n;
-    if ((e = cudaMemsetAsync(h->d_rexp, 0, sizeof(int) * (size_t)(2 * tlen + 2 * n + 32), h->stream))) return e;
+    if ((e = h->arena.alloc((void **)&h->d_rexp, sizeof(uint16_t) * (size_t)len)) ||
+        (e = h->arena.alloc((void **)&h->d_vexp, sizeof(uint16_t) * VEXP * (size_t)(2 * tlen + n))) ||
+        (e = h->arena.alloc((void **)&h->d_colbad, sizeof(int))))
+        return e;
+    if ((e = cudaMemsetAsync(h->d_rexp, 0, sizeof(uint16_t) * (size_t)len, h->stream))) return e;
     const int ntask = (int)F.p1_lo.size();
     if (ntask > 0)
         k_far_rexp1<<<ntask, 256, 0, h->stream>>>(h->d_p1_lo, h->d_p1_hi, h->d_p1_ptr, h->d_p1_off, h->d_p1_ld, h->d_p1_rank,
                                                   h->d_p1_row, h->d_p1_isv, h->d_farU, h->d_farV, h->d_rexp, tlen);
-    k_far_rexp2<<<h->nl, 256, 0, h->stream>>>(h->d_leaf_ptr, h->d_part_ptr, h->d_segs, h->d_farU, h->d_farV,
-                                           h->d_rexp + 2 * tlen);
-    k_far_rexp2<<<h->nl, 256, 0, h->stream>>>(h->d_leaf_ptr, h->d_zpart, h->d_zsegs, h->d_near, h->d_near,
-                                              h->d_rexp + 2 * tlen + n);
+    k_far_rexp2<<<dim3(h->nl * FAR_PARTS, FAR_TABS), 256, 0, h->stream>>>(h->nl, h->n, h->d_leaf_ptr, h->d_zpart, h->d_zsegs,
+                                                                       h->d_farU, h->d_farV, h->d_near,
+                                                                       h->d_rexp + 2 * tlen);
     return cudaGetLastError();
 }
 
@@ -1214,19 +1351,21 @@ static cudaError_t far64_run(hm_ctx *h, const double2 *U, const double2 *V, doub
             return e;
         attr.done();
     }
-    HM_LAUNCH(h, K_PERMUTE, k_far_gather64<<<nblk(len, 256), 256, 0, h->stream>>>(n, nrhs, h->d_cl2new, x, u, h->d_cexp));
+    if ((e = cudaMemsetAsync(h->d_colbad, 0, sizeof(int), h->stream))) return e;
+    HM_LAUNCH(h, K_PERMUTE, k_far_gather64<<<nblk(len, 256), 256, 0, h->stream>>>(n, nrhs, h->d_cl2new, x, u,
+                                                                              h->d_vexp + 2 * F.tlen * VEXP, h->d_colbad));
     const int ntask = (int)F.p1_lo.size();
     if (ntask > 0)
         HM_LAUNCH(h, K_FAR1,
                   k_far_t64<NARROW><<<dim3(ntask, 64 / OZ_ROWS), threads, smem, h->stream>>>(
                       h->d_p1_lo, h->d_p1_hi, h->d_p1_ptr, h->d_p1_off, h->d_p1_ld, h->d_p1_rank, h->d_p1_row,
-                      h->d_p1_isv, U, V, u, nrhs, t, s, h->d_rexp, F.tlen, h->d_cexp));
+                      h->d_p1_isv, U, V, u, nrhs, t, s, h->d_rexp, h->d_vexp, F.tlen));
     double2 *part = (double2 *)h->d_farpart;
     HM_LAUNCH(h, K_FAR2,
               k_far_y64<NARROW><<<dim3(h->nl * FAR_PARTS, (h->max_leaf + OZ_ROWS - 1) / OZ_ROWS), threads, smem, h->stream>>>(
-                  h->nl, h->d_leaf_ptr, h->d_part_ptr, h->d_seg_kcum, h->d_segs, h->d_zpart, h->d_zkcum, h->d_zsegs, U, V,
-                  near ? h->d_near : nullptr, t, s, u, h->d_cl2new, n, nrhs, part, h->d_rexp + 2 * F.tlen, h->d_cexp));
-    HM_LAUNCH(h, K_FAR2, k_far_sum<double2><<<nblk(len, 256), 256, 0, h->stream>>>(len, part, y, h->d_cexp));
+                  h->nl, h->d_leaf_ptr, h->d_zpart, h->d_zkcum, h->d_zsegs, U, V, near ? h->d_near : nullptr, t, s, u,
+                  h->d_cl2new, n, nrhs, part, h->d_rexp + 2 * F.tlen, h->d_vexp, F.tlen));
+    HM_LAUNCH(h, K_FAR2, k_far_sum<double2><<<nblk(len, 256), 256, 0, h->stream>>>(n, len, part, y, h->d_colbad));
     return cudaGetLastError();
 }
 
@@ -1270,7 +1409,7 @@ static cudaError_t far32_run(hm_ctx *h, const float2 *U, const float2 *V, float2
                   h->nl, h->d_leaf_ptr, h->d_part_ptr, h->d_seg_kcum, h->d_segs, U, V, t, s, ucl, h->d_cl2new, n, nrhs,
                   part, np, v16));
     const int64_t len = (int64_t)n * nrhs;
-    HM_LAUNCH(h, K_FAR2, k_far_sum<float2><<<nblk(len, 256), 256, 0, h->stream>>>(len, part, y));
+    HM_LAUNCH(h, K_FAR2, k_far_sum<float2><<<nblk(len, 256), 256, 0, h->stream>>>(n, len, part, y));
     return cudaGetLastError();
 }
 

@@ -109,6 +109,7 @@ struct FarSegD {
 };
 
 constexpr int FAR_PARTS = 8;
+constexpr int FAR_TABS = 4;   // tables of the FP64 product: U t, V s, dense far blocks, near blocks
 
 // far-field incidence lists (cluster order): per leaf l, entries (b << 2 | kind), kind
 // 0 = low-rank row side, 1 = low-rank column side, 2 = dense row side, 3 = dense column side
@@ -131,8 +132,10 @@ struct FarPlan {
     // each leaf's segments in FAR_PARTS consecutive parts of about equal contraction length:
     // part (l, p) covers segments part_ptr[l*FAR_PARTS + p] .. part_ptr[l*FAR_PARTS + p + 1]
     std::vector<int> part_ptr;
-    // the near-field blocks of each leaf as segments of the same form (F from the near blocks, Y = u), in
-    // FAR_PARTS parts: the Z u of the refinement residual
+    // the FP64 product's segments in four tables, by what they multiply: U t, V s, dense far blocks u, near-field blocks
+    // u (F from the near blocks; the Z u of the refinement residual).  Each table holds each leaf's segments in
+    // FAR_PARTS parts: part (table, l, p) covers segments zpart[i] .. zpart[i + 1], i = table * (nl * FAR_PARTS + 1) +
+    // l * FAR_PARTS + p; zkcum as seg_kcum
     std::vector<int> zpart, zkcum;
     std::vector<FarSegD> zsegs;
 };
@@ -199,11 +202,13 @@ struct hm_ctx {
     int *d_p1_lo = nullptr, *d_p1_hi = nullptr, *d_p1_ptr = nullptr, *d_p1_ld = nullptr, *d_p1_rank = nullptr,
         *d_p1_row = nullptr, *d_p1_isv = nullptr;
     int64_t *d_p1_off = nullptr;
-    int *d_seg_ptr = nullptr, *d_seg_kcum = nullptr, *d_part_ptr = nullptr;
+    int *d_seg_kcum = nullptr, *d_part_ptr = nullptr;
     hm::FarSegD *d_segs = nullptr, *d_zsegs = nullptr;
     int *d_zpart = nullptr, *d_zkcum = nullptr;
     int max_leaf = 0;
-    int *d_rexp = nullptr, *d_cexp = nullptr;   // exponents for the split FP64 products (far.cu); d_cexp in d_rexp's allocation
+    uint16_t *d_rexp = nullptr;   // exponents of the coefficient rows of the split FP64 products (far.cu)
+    uint16_t *d_vexp = nullptr;   // and of the vector entries: t, s, u, 16 columns each
+    int *d_colbad = nullptr;      // its vector columns with an infinity or a NaN, one bit each
     int *d_leaf_ptr = nullptr, *d_perm = nullptr;
     int *d_new2cl = nullptr, *d_cl2new = nullptr, *d_new2orig = nullptr, *d_pos = nullptr;
     // device: plan

@@ -614,32 +614,44 @@ void plan_far(hm_ctx *h)
     F.seg_kcum.assign(F.segs.size() + 1, 0);
     for (size_t q = 0; q < F.segs.size(); ++q) F.seg_kcum[q + 1] = F.seg_kcum[q] + F.segs[q].len;
     cut_parts(F.seg_ptr, F.seg_kcum, F.part_ptr);
-    // the near-field blocks as segments: leaf l is the row leaf t (F = B) or the column leaf s (F = B^T)
+    // the same segments for the FP64 product, sorted by what they multiply, and the near-field blocks: leaf l is the row
+    // leaf t (F = B) or the column leaf s (F = B^T)
     std::vector<std::vector<int>> nl_lists(nl);
     for (size_t b = 0; b < h->near_t.size(); ++b) {
         nl_lists[h->near_t[b]].push_back((int)(b << 1));
         if (h->near_t[b] != h->near_s[b]) nl_lists[h->near_s[b]].push_back((int)((b << 1) | 1));
     }
-    std::vector<int> zptr(nl + 1, 0);
+    std::vector<int> zptr[FAR_TABS];
     F.zsegs.clear();
-    for (int l = 0; l < nl; ++l) {
-        for (int en : nl_lists[l]) {
-            const int b = en >> 1, side = en & 1, o = side ? h->near_t[b] : h->near_s[b];
-            const int mt = h->leaf_ptr[h->near_t[b] + 1] - h->leaf_ptr[h->near_t[b]], K = h->leaf_ptr[o + 1] - h->leaf_ptr[o];
-            const FarSegD g = {h->near_off[b], h->leaf_ptr[o], side ? mt : 1, side ? 1 : mt, 0, 2 << 1};
-            for (int k0 = 0; k0 < K; k0 += 32) {
-                FarSegD q = g;
-                q.foff += (int64_t)k0 * g.fk;
-                q.yrow += k0;
-                q.len = std::min(32, K - k0);
-                F.zsegs.push_back(q);
+    for (int tab = 0; tab < FAR_TABS; ++tab) {
+        zptr[tab].assign(nl + 1, (int)F.zsegs.size());
+        for (int l = 0; l < nl; ++l) {
+            for (int q = F.seg_ptr[l]; q < F.seg_ptr[l + 1]; ++q)
+                if (F.segs[q].src >> 1 == tab) F.zsegs.push_back(F.segs[q]);
+            for (size_t x = 0; tab == FAR_TABS - 1 && x < nl_lists[l].size(); ++x) {
+                const int b = nl_lists[l][x] >> 1, side = nl_lists[l][x] & 1, o = side ? h->near_t[b] : h->near_s[b];
+                const int mt = h->leaf_ptr[h->near_t[b] + 1] - h->leaf_ptr[h->near_t[b]];
+                const int K = h->leaf_ptr[o + 1] - h->leaf_ptr[o];
+                const FarSegD g = {h->near_off[b], h->leaf_ptr[o], side ? mt : 1, side ? 1 : mt, 0, 2 << 1};
+                for (int k0 = 0; k0 < K; k0 += 32) {
+                    FarSegD q = g;
+                    q.foff += (int64_t)k0 * g.fk;
+                    q.yrow += k0;
+                    q.len = std::min(32, K - k0);
+                    F.zsegs.push_back(q);
+                }
             }
+            zptr[tab][l + 1] = (int)F.zsegs.size();
         }
-        zptr[l + 1] = (int)F.zsegs.size();
     }
     F.zkcum.assign(F.zsegs.size() + 1, 0);
     for (size_t q = 0; q < F.zsegs.size(); ++q) F.zkcum[q + 1] = F.zkcum[q] + F.zsegs[q].len;
-    cut_parts(zptr, F.zkcum, F.zpart);
+    F.zpart.clear();
+    for (int tab = 0; tab < FAR_TABS; ++tab) {
+        std::vector<int> part;
+        cut_parts(zptr[tab], F.zkcum, part);
+        F.zpart.insert(F.zpart.end(), part.begin(), part.end());
+    }
     h->max_leaf = 0;
     for (int l = 0; l < nl; ++l) h->max_leaf = std::max(h->max_leaf, h->leaf_ptr[l + 1] - h->leaf_ptr[l]);
     // rank-vector tasks: group the factor columns by the range they contract over
