@@ -315,6 +315,10 @@ int precond_setup(hm_handle h)
     cudaEventRecord(e0, h->stream);
     int bad = -1;
     e = setup_run(h, &bad);
+    h->arena.release(h->d_A, 0);   // before the coefficients' store and the sweeps ask for memory of their own
+    h->arena.release(h->d_A32, 0);
+    h->d_A = nullptr;
+    h->d_A32 = nullptr;
     if (!e && bad < 0) e = compress_run(h);
     if (!e && bad < 0) e = pack_run(h);
     if (!e && bad < 0) e = sweep2_setup(h);
@@ -324,10 +328,6 @@ int precond_setup(hm_handle h)
     cudaEventElapsedTime(&ms, e0, e1);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    h->arena.release(h->d_A, 0);
-    h->arena.release(h->d_A32, 0);
-    h->d_A = nullptr;
-    h->d_A32 = nullptr;
     if (e) return cuda_fail(h, e, "precond_setup");
     if (bad >= 0) {
         h->err = "pivot block D_" + std::to_string(bad) + " (solve order; leaf " + std::to_string(P.order[bad]) +

@@ -1,0 +1,54 @@
+"""hbm_budget and the two-level data of the sweeps."""
+import numpy as np
+import pytest
+import torch
+
+import efie_problem as ep
+import paper_2111_13483_gb300 as hm
+
+pytestmark = pytest.mark.gpu
+H = hm.hmsolve
+MESH = dict(kind="sphere", d=2, a=0.3, leaf=64, eta=1.0, aca_eps=1e-3)   # one super-row
+
+
+def used(h):
+    return hm.hmat_stats(h)["device_bytes"]
+
+
+def sweep(h, prec, X):
+    x = torch.from_numpy(X).cuda()
+    y = torch.empty_like(x)
+    hm.hm_apply(h, (H.OP32 if prec else 0) + H.OP_LINV, x, y)
+    return y.cpu().numpy()
+
+
+def sizes(P, prec, fill_tol=0.0):
+    """Bytes after a setup and the operator's workspace of one column; a vector; L^{-1} of it by both sweeps."""
+    g = hm.hmat_create(P, ordering=1, precision=prec, fill_tol=fill_tol)
+    hm.precond_setup(g)
+    full = used(g)
+    rng = np.random.default_rng(4)
+    X = rng.standard_normal((1, P.n)) + 1j * rng.standard_normal((1, P.n))
+    two = sweep(g, prec, X)
+    work = used(g) - full
+    H.hm_set_sweep_schedule(g, 1, 1, 0)
+    return full, work, X, two, sweep(g, prec, X)
+
+
+@pytest.mark.parametrize("prec,fill_tol", [(0, 0.0), (1, 0.0), (1, 1e-2)])
+def test_a_budget_of_the_steady_state_keeps_the_two_level_sweeps(prec, fill_tol):
+    """What the handle holds after a setup is smaller than what the elimination takes on the way (its workspace); a budget
+    that holds either has room for the sweeps' data, also in a second setup (which, with compressed coefficients, has
+    their store beside the elimination)."""
+    P = ep.build(dict(MESH, d=3, a=0.6))
+    full, work, X, two, one = sizes(P, prec, fill_tol)
+    assert not np.array_equal(two, one)
+    g = hm.hmat_create(P, ordering=1, precision=prec, fill_tol=fill_tol)
+    before = used(g)   # the elimination: its workspace beside the dense coefficients and the diagonal blocks, twice
+    f = hm.hmat_stats(g)
+    c, d = f["coef_entries_dense"], f["diag_entries"]
+    elimination = before + (16 * (2 * c + 2 * d) if prec == 0 else 8 * (2 * c + 2 * d) + 16 * d)
+    h = hm.hmat_create(P, ordering=1, precision=prec, fill_tol=fill_tol, hbm_budget=max(elimination, full) + work + 8192)
+    for _ in range(1 if fill_tol else 2):
+        hm.precond_setup(h)
+        assert np.array_equal(sweep(h, prec, X), two)
