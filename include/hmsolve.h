@@ -282,7 +282,10 @@ int hm_far_apply_noalloc(hm_handle h, const void *dx, void *dy, int32_t nrhs);
  * form a super-row whose unit triangle is inverted once per setup, so that its rows run side by
  * side (a fixed summation order of its own, bitwise the same for every batch width).  Where
  * hbm_budget leaves no room for their data, the library instead times kind 1 with 1, 2 and 4
- * groups and each tile on its first calls of each width and keeps the fastest.
+ * groups and each tile on its first calls of each width and keeps the fastest.  A solve or a
+ * batch that fits only without those data takes their memory and runs that way; they are
+ * formed again when it has returned its own, if there is room then.  A call that does not fit
+ * at all leaves them as they are.
  * Kinds 2 and 3 apply to groups of at most 16 columns (kind 1 otherwise).  With compressed
  * fill-in blocks (fill_tol > 0) kinds 2-4 take kind 1.  `tile` (kind 1) selects the
  * register tile of each thread -- rows x columns x tiles per thread -- for groups of 5-16
@@ -367,7 +370,8 @@ int hm_set_pivot_schedule(hm_handle h, int32_t ctas);
  * step share one multi-column launch); a slot whose solve has ended is reported, its
  * result is read with hm_batch_result, which frees the slot for the next submission.
  * Requests can therefore join while others are in flight.  A column's result is bitwise
- * the same as solve() on that column alone.  The paper has no serving loop: this layer
+ * the same as solve() on that column alone with the same sweeps (hm_set_sweep_schedule: a
+ * tight hbm_budget can give the two different ones).  The paper has no serving loop: this layer
  * only schedules its solve.
  *
  * One batch per handle at a time; the handle's stream carries all of its work and a batch

@@ -10,25 +10,28 @@
 
 namespace hm {
 
+bool Arena::room(size_t bytes) const { return !budget || used + bytes <= budget + (spare ? spare(owner) : 0); }
+
 cudaError_t Arena::alloc(void **p, size_t bytes)
 {
     *p = nullptr;
-    if (bytes == 0) bytes = 16;
-    bytes = (bytes + 255) & ~size_t(255);
-    const bool over = budget && used + bytes > budget;
-    cudaError_t e = over ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
-    if (e == cudaErrorMemoryAllocation) {
+    bytes = rounded(bytes);
+    for (bool again = false;; again = true) {
+        const bool over = budget && used + bytes > budget;
+        const cudaError_t e = over ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+        if (e == cudaSuccess) {
+            used += bytes;
+            ptrs.push_back(*p);
+            sizes.push_back(bytes);
+            return e;
+        }
         cudaGetLastError();
         *p = nullptr;
-        return reclaim && reclaim(owner) ? alloc(p, bytes) : e;
+        const size_t sp = e == cudaErrorMemoryAllocation && !again && spare ? spare(owner) : 0;
+        size_t have = 0, total = 0;
+        if (!sp || !room(bytes) || (!over && (cudaMemGetInfo(&have, &total) || have + sp < bytes))) return e;
+        reclaim(owner);
     }
-    if (e == cudaSuccess) {
-        used += bytes;
-        ptrs.push_back(*p);
-        sizes.push_back(bytes);
-    } else
-        cudaGetLastError();
-    return e;
 }
 
 void Arena::release(void *p, size_t)
@@ -182,12 +185,16 @@ int hmat_create(const hm_desc *d, const hm_opts *opts, hm_handle *out)
     cudaSetDevice(h->dev);
     h->arena.budget = h->opts.hbm_budget;
     h->arena.owner = h;
-    h->arena.reclaim = [](void *p) {   // the two-level sweeps' memory: the other sweeps do without
+    // the two-level sweeps' memory: the other sweeps do without, once they have their tagged words
+    h->arena.spare = [](void *p) {
+        const hm_ctx *c = (const hm_ctx *)p;
+        return c->s2.on && c->s2.bytes > ytag_bytes(c) ? c->s2.bytes - ytag_bytes(c) : size_t(0);
+    };
+    h->arena.reclaim = [](void *p) {
         hm_ctx *c = (hm_ctx *)p;
-        if (!c->s2.on) return false;
         cudaStreamSynchronize(c->stream);
         sweep2_release(c);
-        return true;
+        c->s2.given = true;
     };
     if (h->opts.stream)
         h->stream = (cudaStream_t)h->opts.stream;
@@ -306,9 +313,16 @@ int precond_setup(hm_handle h)
                       (e = h->arena.alloc((void **)&h->d_Ad, sizeof(double2) * P.diag_entries)))))
             return cuda_fail(h, e, "precond_setup allocation");
     }
-    if ((e = mixed ? h->arena.alloc((void **)&h->d_A32, sizeof(float2) * P.coef_entries)
-                   : h->arena.alloc((void **)&h->d_A, sizeof(double2) * P.coef_entries)))
-        return cuda_fail(h, e, "precond_setup workspace");
+    auto workspace = [&]() {
+        return mixed ? h->arena.alloc((void **)&h->d_A32, sizeof(float2) * P.coef_entries)
+                     : h->arena.alloc((void **)&h->d_A, sizeof(double2) * P.coef_entries);
+    };
+    e = workspace();
+    if (e == cudaErrorMemoryAllocation && h->s2.on) {   // the last setup's two-level data, formed anew below
+        sweep2_release(h);
+        e = workspace();
+    }
+    if (e) return cuda_fail(h, e, "precond_setup workspace");
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -374,8 +388,12 @@ int solve(hm_handle h, const hm_c128 *V, int32_t nrhs, int64_t ldv, double tol, 
     double2 *dV = nullptr, *dI = nullptr;
     cudaError_t e;
     const size_t col = sizeof(double2) * (size_t)h->n;
+    const bool args = restart >= 1 && maxit >= 0 && tol >= 0;   // else solve_device says so
+    if (args && !h->arena.room(2 * Arena::rounded(col * nrhs) + gmres_bytes(h, nrhs, restart)))
+        return cuda_fail(h, cudaErrorMemoryAllocation, "solve workspace");
     if ((e = h->arena.alloc((void **)&dV, col * nrhs)) || (e = h->arena.alloc((void **)&dI, col * nrhs))) {
         h->arena.release(dV, 0);
+        sweep2_restore(h);
         return cuda_fail(h, e, "solve staging");
     }
     int s = HM_OK;
@@ -389,6 +407,7 @@ int solve(hm_handle h, const hm_c128 *V, int32_t nrhs, int64_t ldv, double tol, 
     }
     h->arena.release(dV, 0);
     h->arena.release(dI, 0);
+    sweep2_restore(h);
     return s;
 }
 

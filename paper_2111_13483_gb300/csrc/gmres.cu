@@ -357,7 +357,29 @@ struct Engine {
         return b;
     }
 
-    cudaError_t open(hm_ctx *hh, int slots, int restart)
+    int pack() const { return std::min(S, fp32 ? 64 : 16); }   // columns of the widest operator call
+
+    // the device buffers of the engine
+    std::vector<std::pair<void **, size_t>> buffers()
+    {
+        std::vector<std::pair<void **, size_t>> b;
+        auto A = [&](auto **p, size_t count) { b.push_back({(void **)p, sizeof(**p) * count}); };
+        const size_t vs = (size_t)n * S, s1 = S;
+        A(&B, vs), A(&XO, vs), A(&R, vs), A(&C, vs), A(&XT, vs), A(&Vb, vs * (m + 1));
+        A(&PX, vs), A(&PY, vs), A(&PT, vs), A(&part, part_len(n, S, m));
+        A(&h2, s1 * (m + 1)), A(&s.hj, s1 * (m + 1)), A(&s.H, s1 * (m + 1) * m), A(&s.g, s1 * (m + 1));
+        A(&s.sn, s1 * m), A(&s.y, s1 * m), A(&s.cs, s1 * m), A(&s.nrm, s1), A(&s.res, s1), A(&s.wn, s1), A(&tmp, s1);
+        A(&s.J, s1), A(&d_idx, s1 * NIDX), A(&d_iota, s1);
+        return b;
+    }
+    static size_t buffer_bytes(const std::vector<std::pair<void **, size_t>> &bufs)
+    {
+        size_t t = 0;
+        for (const auto &b : bufs) t += Arena::rounded(b.second);
+        return t;
+    }
+
+    void shape(hm_ctx *hh, int slots, int restart)
     {
         h = hh;
         S = slots;
@@ -366,6 +388,11 @@ struct Engine {
         nchunk = (n + dot_chunk(n) - 1) / dot_chunk(n);
         fp32 = h->opts.precision == 1;
         left = h->opts.preconditioner == 2;
+    }
+
+    cudaError_t open(hm_ctx *hh, int slots, int restart)
+    {
+        shape(hh, slots, restart);
         sl.assign(S, Slot());
         cudaError_t e;
         auto A = [&](void **p, size_t b) {
@@ -373,28 +400,16 @@ struct Engine {
             if (r == cudaSuccess) allocs.push_back(*p);
             return r;
         };
-        const size_t vs = sizeof(double2) * (size_t)n * S;
-        if ((e = A((void **)&B, vs)) || (e = A((void **)&XO, vs)) || (e = A((void **)&R, vs)) ||
-            (e = A((void **)&C, vs)) || (e = A((void **)&XT, vs)) || (e = A((void **)&Vb, vs * (m + 1))) ||
-            (e = A((void **)&PX, vs)) || (e = A((void **)&PY, vs)) || (e = A((void **)&PT, vs)) ||
-            (e = A((void **)&part, sizeof(double2) * part_len(n, S, m))) ||
-            (e = A((void **)&h2, sizeof(double2) * (size_t)S * (m + 1))) ||
-            (e = A((void **)&s.hj, sizeof(double2) * (size_t)S * (m + 1))) ||
-            (e = A((void **)&s.H, sizeof(double2) * (size_t)S * (m + 1) * m)) ||
-            (e = A((void **)&s.g, sizeof(double2) * (size_t)S * (m + 1))) ||
-            (e = A((void **)&s.sn, sizeof(double2) * (size_t)S * m)) ||
-            (e = A((void **)&s.y, sizeof(double2) * (size_t)S * m)) ||
-            (e = A((void **)&s.cs, sizeof(double) * (size_t)S * m)) || (e = A((void **)&s.nrm, sizeof(double) * S)) ||
-            (e = A((void **)&s.res, sizeof(double) * S)) || (e = A((void **)&s.wn, sizeof(double) * S)) ||
-            (e = A((void **)&tmp, sizeof(double) * S)) || (e = A((void **)&s.J, sizeof(int) * S)) ||
-            (e = A((void **)&d_idx, sizeof(int) * (size_t)S * NIDX)) || (e = A((void **)&d_iota, sizeof(int) * S)))
-            return e;
+        const std::vector<std::pair<void **, size_t>> bufs = buffers();
+        if (!h->arena.room(buffer_bytes(bufs) + solve_workspace_growth(h, pack()))) return cudaErrorMemoryAllocation;
+        for (const auto &b : bufs)
+            if ((e = A(b.first, b.second))) return e;
         if ((e = cudaMallocHost((void **)&h_idx, sizeof(int) * (size_t)S * NIDX))) return e;
         std::vector<int> io(S);
         for (int c = 0; c < S; ++c) io[c] = c;
         if ((e = cudaMemcpyAsync(d_iota, io.data(), sizeof(int) * S, cudaMemcpyHostToDevice, h->stream))) return e;
         // the operator workspace for the widest pack
-        if ((e = ensure_solve_workspace(h, std::min(S, fp32 ? 64 : 16)))) return e;
+        if ((e = ensure_solve_workspace(h, pack()))) return e;
         return cudaStreamSynchronize(h->stream);
     }
 
@@ -740,16 +755,25 @@ struct Engine {
     }
 };
 
+// slots of a solve's engine: the FP32 operator takes 64 columns per sweep launch, the FP64 one 16
+static int solve_slots(const hm_ctx *h, int nrhs) { return std::min(nrhs, h->opts.precision == 1 ? 64 : 16); }
+
+size_t gmres_bytes(hm_ctx *h, int nrhs, int restart)
+{
+    Engine E;
+    E.shape(h, solve_slots(h, nrhs), restart);
+    return Engine::buffer_bytes(E.buffers()) + solve_workspace_growth(h, E.pack());
+}
+
 int gmres_solve(hm_ctx *h, const double2 *dV, int nrhs, int64_t ldv, double tol, int restart, int maxit, double2 *dI,
                 int64_t ldi, int *iters, double *relres)
 {
-    // slots of the engine: the FP32 operator takes 64 columns per sweep launch, the FP64 one 16
-    const int width = h->opts.precision == 1 ? 64 : 16;
     Engine E;
     cudaError_t e;
     cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream);
-    if ((e = E.open(h, std::min(nrhs, width), restart))) {
+    if ((e = E.open(h, solve_slots(h, nrhs), restart))) {
         E.close();
+        sweep2_restore(h);
         h->err = std::string("solve workspace: ") + cudaGetErrorString(e);
         return e == cudaErrorMemoryAllocation ? HM_ENOMEM : HM_ECUDA;
     }
@@ -785,6 +809,7 @@ int gmres_solve(hm_ctx *h, const double2 *dV, int nrhs, int64_t ldv, double tol,
     }
     if ((e = cudaStreamSynchronize(h->stream)) && status != HM_ECUDA) status = E.fail(e);
     E.close();
+    sweep2_restore(h);
     return status;
 }
 
@@ -821,6 +846,7 @@ int hm_batch_open(hm_handle h, int32_t slots, int32_t restart, hm_batch *out)
     if (e) {
         b->E.close();
         delete b;
+        hm::sweep2_restore(h);
         h->err = std::string("batch workspace: ") + cudaGetErrorString(e);
         return e == cudaErrorMemoryAllocation ? HM_ENOMEM : HM_ECUDA;
     }
@@ -879,6 +905,7 @@ int hm_batch_close(hm_batch b)
     cudaSetDevice(b->h->dev);
     b->E.close();
     b->h->batch_open = false;
+    hm::sweep2_restore(b->h);
     delete b;
     return HM_OK;
 }

@@ -17,10 +17,15 @@ struct Arena {
     size_t used = 0, budget = 0;
     std::vector<void *> ptrs;
     std::vector<size_t> sizes;
-    // frees memory the handle can do without when an allocation fails; true if it freed any
-    bool (*reclaim)(void *) = nullptr;
+    // memory the handle can do without: its bytes (0 = none), and what gives it back
+    size_t (*spare)(void *) = nullptr;
+    void (*reclaim)(void *) = nullptr;
     void *owner = nullptr;
-    cudaError_t alloc(void **p, size_t bytes);
+    static size_t rounded(size_t bytes) { return ((bytes ? bytes : 16) + 255) & ~size_t(255); }
+    // whether the budget has room for `bytes` more, the spare memory given back if need be: asked for all allocations of
+    // a call together before the first, so that a call that is refused costs the handle nothing
+    bool room(size_t bytes) const;
+    cudaError_t alloc(void **p, size_t bytes);   // gives the spare memory back where that makes the request fit
     void release(void *p, size_t bytes);
     void release_all();
 };
@@ -156,6 +161,8 @@ struct S2State {   // index 0 forward, 1 backward
     int4 *deps[2] = {nullptr, nullptr};
     void *N[2] = {nullptr, nullptr};
     void *buf = nullptr;   // ticket and hand-over buffers
+    size_t bytes = 0;      // device memory of all of it, also when it is not there
+    bool given = false;    // given back to the arena; formed again when there is room
 };
 
 // Online choice of the schedule of a sweep launch -- the number of independent column
@@ -336,9 +343,13 @@ cudaError_t far_product64(hm_ctx *h, const double2 *U, const double2 *V, double2
 cudaError_t far_product32(hm_ctx *h, const float2 *U, const float2 *V, float2 *t, float2 *s, const float2 *ucl, float2 *y,
                           int nrhs);
 cudaError_t ensure_solve_workspace(hm_ctx *h, int nrhs);
+size_t solve_workspace_growth(hm_ctx *h, int nrhs);   // bytes ensure_solve_workspace would add
 void sweep_tune_release(hm_ctx *h);
 cudaError_t sweep2_setup(hm_ctx *h);
 void sweep2_release(hm_ctx *h);
+void sweep2_restore(hm_ctx *h);
+size_t ytag_bytes(const hm_ctx *h);
+size_t gmres_bytes(hm_ctx *h, int nrhs, int restart);
 template <class T> cudaError_t sweep2_run(hm_ctx *h, bool fwd, const T *W, const T *x, T *y, int nrhs);
 int gmres_solve(hm_ctx *h, const double2 *dV, int nrhs, int64_t ldv, double tol, int restart, int maxit,
                 double2 *dI, int64_t ldi, int *iters, double *relres);

@@ -1546,10 +1546,36 @@ static void set_attrs()
     cudaFuncSetAttribute(k_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(T) * 128 * 64));
 }
 
+size_t ytag_bytes(const hm_ctx *h)   // of the tagged words still to be allocated: 64 columns, complex-FP32 sweeps
+{
+    return h->opts.precision == 1 && !h->d_ytag ? Arena::rounded(sizeof(uint4) * (size_t)h->plan.n * 64) : 0;
+}
+
+size_t solve_workspace_growth(hm_ctx *h, int nrhs)
+{
+    const size_t n = h->plan.n, tl = std::max<int64_t>(1, h->fplan.tlen);
+    const auto more = [](bool grows, size_t bytes, size_t times, bool have, size_t old) {
+        return grows ? times * (Arena::rounded(bytes) - (have ? Arena::rounded(old) : 0)) : 0;
+    };
+    size_t b = h->d_flags ? 0 : Arena::rounded(sizeof(int) * h->plan.nb * SWEEP_GMAX * 2);
+    b += more(h->t_cols < nrhs, sizeof(double2) * tl * nrhs, 2, h->d_t, sizeof(double2) * tl * h->t_cols);
+    const size_t fpb = (size_t)FAR_PARTS * n * nrhs * sizeof(double2);
+    b += more(h->farpart_bytes < fpb, fpb, 1, h->d_farpart, h->farpart_bytes);
+    b += more(h->work_cols < 3 * nrhs, sizeof(double2) * n * 3 * nrhs, 1, h->d_work, sizeof(double2) * n * h->work_cols);
+    if (h->opts.precision == 1) {
+        b += more(h->t32_cols < nrhs, sizeof(float2) * tl * nrhs, 2, h->d_t32, sizeof(float2) * tl * h->t32_cols);
+        b += more(h->t32_cols < nrhs, sizeof(float2) * n * 5 * nrhs, 1, h->d_work32, sizeof(float2) * n * 5 * h->t32_cols);
+        if (!h->s2.on || h->sweep_fixed) b += ytag_bytes(h);
+    }
+    return b;
+}
+
 cudaError_t ensure_solve_workspace(hm_ctx *h, int nrhs)
 {
     cudaError_t e;
     const int n = h->plan.n;
+    const size_t growth = solve_workspace_growth(h, nrhs);
+    if (growth && !h->arena.room(growth)) return cudaErrorMemoryAllocation;
     if (!h->d_flags) {
         if ((e = h->arena.alloc((void **)&h->d_flags, sizeof(int) * h->plan.nb * SWEEP_GMAX * 2))) return e;
         if ((e = cudaMemsetAsync(h->d_flags, 0, sizeof(int) * h->plan.nb * SWEEP_GMAX * 2, h->stream))) return e;

@@ -691,6 +691,11 @@ template <class T> cudaError_t s2_build(hm_ctx *h, const T *W)
             off[1][j] = len1;
             len1 += (int64_t)P.size[j] * (P.boff[std::min(P.nb, j / S2_K * S2_K + S2_K)] - P.boff[j + 1]);
         }
+        h->s2.bytes = 2 * (Arena::rounded(sizeof(S2Row) * P.nb) + Arena::rounded(sizeof(int64_t) * P.nb) +
+                           Arena::rounded(sizeof(int4) * std::max(ne, 1)) +
+                           Arena::rounded(sizeof(T) * (size_t)std::max<int64_t>(len, 1))) +
+                      Arena::rounded(s2_buf_bytes<T>(P.n));
+        if (!h->arena.room(h->s2.bytes)) return cudaErrorMemoryAllocation;
         for (int d = 0; d < 2; ++d) {
             const std::vector<S2Row> rows = s2_rows(P, d == 0, off[d]);
             if ((e = h->arena.alloc((void **)&h->s2.rows[d], sizeof(S2Row) * P.nb)) ||
@@ -778,7 +783,7 @@ void sweep2_release(hm_ctx *h)
 // for them (hbm_budget) the sweeps stay with the kinds of ops.cu.
 cudaError_t sweep2_setup(hm_ctx *h)
 {
-    h->s2.on = false;
+    h->s2.on = h->s2.given = false;
     const cudaError_t e = h->opts.precision == 1 ? s2_build<float2>(h, h->d_Wc32) : s2_build<double2>(h, h->d_Wc);
     if (e == cudaErrorMemoryAllocation) {
         sweep2_release(h);
@@ -786,6 +791,20 @@ cudaError_t sweep2_setup(hm_ctx *h)
     }
     h->s2.on = e == cudaSuccess;
     return e;
+}
+
+// Where a solve or a batch made the handle give the data back and has returned its own memory: formed again.
+void sweep2_restore(hm_ctx *h)
+{
+    if (!h->s2.given || !h->setup_done) return;
+    const size_t tags = h->d_ytag && !h->sweep_fixed ? Arena::rounded(sizeof(uint4) * (size_t)h->plan.n * 64) : 0;
+    if (h->arena.budget && h->arena.used - tags + h->s2.bytes > h->arena.budget) return;
+    if (tags) {   // the other sweeps' words, which are no longer needed
+        h->arena.release(h->d_ytag, 0);
+        h->d_ytag = nullptr;
+    }
+    if (sweep2_setup(h)) cudaGetLastError();
+    h->s2.given = !h->s2.on;
 }
 
 // Column groups: one column alone; 4 in FP64 and in complex FP32 up to 16 columns (on the 30,720-unknown

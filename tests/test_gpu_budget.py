@@ -1,4 +1,5 @@
-"""hbm_budget and the two-level data of the sweeps."""
+"""hbm_budget and the two-level data of the sweeps: when there is room for them, and what a call that does not fit, and
+one that fits only in their place, leave behind."""
 import numpy as np
 import pytest
 import torch
@@ -8,7 +9,7 @@ import paper_2111_13483_gb300 as hm
 
 pytestmark = pytest.mark.gpu
 H = hm.hmsolve
-MESH = dict(kind="sphere", d=2, a=0.3, leaf=64, eta=1.0, aca_eps=1e-3)   # one super-row
+MESH = dict(kind="sphere", d=2, a=0.3, leaf=64, eta=1.0, aca_eps=1e-3)   # one super-row, larger than the elimination's workspace
 
 
 def used(h):
@@ -52,3 +53,47 @@ def test_a_budget_of_the_steady_state_keeps_the_two_level_sweeps(prec, fill_tol)
     for _ in range(1 if fill_tol else 2):
         hm.precond_setup(h)
         assert np.array_equal(sweep(h, prec, X), two)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_refused_call_leaves_the_sweeps(prec):
+    P = ep.build(MESH)
+    full, work, X, two, one = sizes(P, prec)
+    assert not np.array_equal(two, one)
+    h = hm.hmat_create(P, ordering=1, precision=prec, hbm_budget=full + work + 4096)
+    hm.precond_setup(h)
+    assert np.array_equal(sweep(h, prec, X), two)
+    before = used(h)
+    with pytest.raises(Exception):
+        hm.Batch(h, 1024, 50)
+    V = np.zeros((P.n, 64), dtype=np.complex128)
+    with pytest.raises(Exception):
+        hm.solve(h, V, tol=1e-6, restart=2000)
+    assert used(h) == before
+    assert np.array_equal(sweep(h, prec, X), two)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_sweeps_come_back_after_a_batch(prec):
+    P = ep.build(MESH)
+    full, work, X, two, one = sizes(P, prec)
+    engine = hm.Batch.bytes(h := hm.hmat_create(P, ordering=1, precision=prec), 1, 5)
+    hm.hmat_destroy(h)
+    h = hm.hmat_create(P, ordering=1, precision=prec, hbm_budget=full + work + engine // 2)
+    hm.precond_setup(h)
+    assert np.array_equal(sweep(h, prec, X), two)
+    before = used(h)
+    b = hm.Batch(h, 1, 5)                      # fits only in the place of the two-level data
+    assert np.array_equal(sweep(h, prec, X), one)
+    V = P.plane_wave([0.0, 0.0, -1.0], [1.0, 0.0, 0.0])
+    b.submit(V, tol=1e-4)
+    fin = []
+    while not fin:
+        fin = b.step()
+    assert b.result(fin[0])[3] == 0
+    b.close()
+    assert used(h) == before
+    assert np.array_equal(sweep(h, prec, X), two)
+    x, it, rr, code = hm.solve(h, V, tol=1e-4, restart=5)   # the same for a solve
+    assert code == 0 and used(h) == before
+    assert np.array_equal(sweep(h, prec, X), two)
