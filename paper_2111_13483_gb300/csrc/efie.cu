@@ -120,8 +120,8 @@ __device__ __forceinline__ double2 csc(double s, double2 a) { return make_double
 
 // ---------------------------------------------------------------------------------------
 // Integrals of the ACA.  On a regular mesh its pivot search meets moduli that are equal but for rounding, and which of
-// them wins decides the factors; so it keeps one fixed sequence of roundings, while the dense blocks below use the
-// cheaper one.
+// them wins decides the factors.  Any of them are as good; to have the same ones from build to build the ACA keeps one
+// fixed sequence of roundings, while the dense blocks below use the cheaper one.
 // S0 = int_T 1/|r - r'| ds' and Sv = int_T (r' - rho)/|r - r'| ds' over the flat triangle P
 // (unit normal n), rho the projection of r on its plane.  Per edge a -> b with unit tangent l
 // and in-plane outward normal u = l x n, h = n.(r - P0): l+- = (b|a - rho).l,
@@ -366,8 +366,9 @@ __device__ __forceinline__ void potential(const Geometry &G, int q, V3 r, double
 }
 
 // sin x and off + cos x (off 0 or -1, the latter without cancellation) for x >= 0: reduction by multiples of pi/2 in
-// two parts (Cody and Waite), then the Taylor series on |r| <= pi/4, the terms from r^12 on (1e-10 of the sum) in
-// FP32: a warp's FP64 operation holds its scheduler for 64 cycles, so the 20 that are left are the price.
+// two parts (Cody and Waite), then the Taylor series on |r| <= pi/4, the terms from r^12 on (at most 1.2e-10) in
+// FP32, whose rounding there is 1.4e-17, an eighth of an FP64 rounding of the cosine: a warp's FP64 operation
+// holds its scheduler for 64 cycles, so the 20 that are left are the price.
 __device__ __forceinline__ void sin_cos(double x, double off, double &sn, double &cs)
 {
     if (!(x < 1e5)) {
