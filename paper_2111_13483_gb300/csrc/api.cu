@@ -185,10 +185,12 @@ int hmat_create(const hm_desc *d, const hm_opts *opts, hm_handle *out)
     cudaSetDevice(h->dev);
     h->arena.budget = h->opts.hbm_budget;
     h->arena.owner = h;
-    // the two-level sweeps' memory: the other sweeps do without, once they have their tagged words
+    // the two-level sweeps' memory: the other sweeps do without, once they have their tagged words (which a call asks
+    // for itself where a schedule is set)
     h->arena.spare = [](void *p) {
         const hm_ctx *c = (const hm_ctx *)p;
-        return c->s2.on && c->s2.bytes > ytag_bytes(c) ? c->s2.bytes - ytag_bytes(c) : size_t(0);
+        const size_t words = c->sweep_fixed ? 0 : ytag_bytes(c);
+        return c->s2.on && c->s2.bytes > words ? c->s2.bytes - words : size_t(0);
     };
     h->arena.reclaim = [](void *p) {
         hm_ctx *c = (hm_ctx *)p;
@@ -668,7 +670,10 @@ int hm_apply(hm_handle h, int32_t op, const void *dx, void *dy, int32_t nrhs)
     else if (op >= 8) e = hm::op_apply32(h, op - 8, (const double2 *)dx, (double2 *)dy, nrhs);
     else e = op_apply(h, op, (const double2 *)dx, (double2 *)dy, nrhs);
     if (!e) e = cudaStreamSynchronize(h->stream);
-    if (e) return cuda_fail(h, e, "hm_apply");
+    if (e) {
+        sweep2_restore(h);
+        return cuda_fail(h, e, "hm_apply");
+    }
     int herr = 0;
     cudaMemcpy(&herr, h->d_err, sizeof(int), cudaMemcpyDeviceToHost);
     if (herr) {

@@ -6,6 +6,7 @@ import torch
 
 import efie_problem as ep
 import paper_2111_13483_gb300 as hm
+from test_gpu_setup_blocks import problem
 
 pytestmark = pytest.mark.gpu
 H = hm.hmsolve
@@ -97,3 +98,23 @@ def test_sweeps_come_back_after_a_batch(prec):
     x, it, rr, code = hm.solve(h, V, tol=1e-4, restart=5)   # the same for a solve
     assert code == 0 and used(h) == before
     assert np.array_equal(sweep(h, prec, X), two)
+
+
+@pytest.mark.parametrize("sizes_", [[64], [64, 33], [5, 40, 64, 17]])
+def test_a_schedule_set_later_takes_the_place_of_the_two_level_data(sizes_):
+    """A few blocks, whose two-level data are little more than their hand-over buffers: the words of the sweeps that are
+    asked for fit in their place."""
+    P = problem(sizes_, 3)[0]
+    g = hm.hmat_create(P, ordering=1, precision=1)
+    hm.precond_setup(g)
+    rng = np.random.default_rng(4)
+    X = rng.standard_normal((1, P.n)) + 1j * rng.standard_normal((1, P.n))
+    two = sweep(g, 1, X)
+    full = used(g)
+    H.hm_set_sweep_schedule(g, 1, 1, 0)
+    one = sweep(g, 1, X)
+    h = hm.hmat_create(P, ordering=1, precision=1, hbm_budget=full)
+    hm.precond_setup(h)
+    assert np.array_equal(sweep(h, 1, X), two)
+    H.hm_set_sweep_schedule(h, 1, 1, 0)
+    assert np.array_equal(sweep(h, 1, X), one)
