@@ -280,7 +280,8 @@ int hm_far_apply_noalloc(hm_handle h, const void *dx, void *dy, int32_t nrhs);
  * and 6 give bitwise the same result, and kind 4 gives bitwise the same result for every
  * number of groups.  (0, 0) is the default: two-level sweeps, in which 16 consecutive block rows
  * form a super-row whose unit triangle is inverted once per setup, so that its rows run side by
- * side (a fixed summation order of its own, bitwise the same for every batch width).  Where
+ * side (a fixed summation order of its own, bitwise the same for every batch width; an infinity
+ * or a NaN reaches all later rows of its super-row, in its own column).  Where
  * hbm_budget leaves no room for their data, the library instead times kind 1 with 1, 2 and 4
  * groups and each tile on its first calls of each width and keeps the fastest.  A solve or a
  * batch that fits only without those data takes their memory and runs that way; they are
